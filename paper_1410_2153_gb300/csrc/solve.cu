@@ -1321,7 +1321,7 @@ template <class T>
 int enqueue_body(asmg_s& h, Slot& S, cudaStream_t s, cudaGraphConditionalHandle hnd, int use_hnd) {
   int launches = enqueue_precond<T>(h, S, S.r.p, s);
   const T* z = slotprec<T>(S).uf.p;
-  const int G = RED_BLOCKS, GV = VEC_BLOCKS;
+  const int G = red_grid(h.npad, RED_BLOCKS), GV = red_grid(h.npad, VEC_BLOCKS);
   const int64_t n = h.n, sz = sizeof(T);
   LAUNCH(ASMG_PROF_CG_VECTOR, n * (sz + 16),
          launch(h.prm.use_pdl, k_dots<T>, GV, TPB, s, h.npad, z, S.r.p, S.q.p, S.partial.p, S.ticket.p, S.scal.p));
@@ -1340,7 +1340,7 @@ template <class T>
 int enqueue_iteration(asmg_s& h, Slot& S, cudaStream_t s, cudaGraphConditionalHandle hnd, int use_hnd) {
   int launches = enqueue_precond<T>(h, S, S.r.p, s);
   const T* z = slotprec<T>(S).uf.p;
-  const int G = RED_BLOCKS;
+  const int G = red_grid(h.npad, RED_BLOCKS);
   const int64_t n = h.n, sz = sizeof(T);
   LAUNCH(ASMG_PROF_CG_VECTOR, n * (sz + 16), launch(h.prm.use_pdl, k_xpz<T>, G, TPB, s, h.npad, z, S.x.p));
   LAUNCH(ASMG_PROF_CG_SPMV, h.A64.nnz_real * 12 + n * 24,
@@ -1360,7 +1360,7 @@ int enqueue_body_any(asmg_s& h, Slot& S, cudaStream_t s, cudaGraphConditionalHan
 
 void enqueue_init(asmg_s& h, Slot& S, double rtol, cudaStream_t s, cudaGraphConditionalHandle hnd, int use_hnd) {
   LAUNCH(ASMG_PROF_CG_VECTOR, h.A64.nnz_real * 12 + h.n * 32,
-         launch(h.prm.use_pdl, k_pcg_init, RED_BLOCKS, TPB, s, h.npad, view(h.A64), S.b.p, S.x.p, S.r.p, S.partial.p, S.ticket.p,
+         launch(h.prm.use_pdl, k_pcg_init, red_grid(h.npad, RED_BLOCKS), TPB, s, h.npad, view(h.A64), S.b.p, S.x.p, S.r.p, S.partial.p, S.ticket.p,
                                                S.scal.p, rtol, h.prm.max_iter, S.hist.p, hnd, use_hnd));
   ASMG_CUDA(cudaGetLastError());
 }

@@ -945,12 +945,13 @@ void enqueue_body_k(asmg_s& h, MultiSlot& S, cudaStream_t s, cudaGraphConditiona
   enqueue_precond_k<T>(h, S, S.r.p, s);
   const T* z = mprec_of<T>(S).uf.p;
   const bool pdl = h.prm.use_pdl;
-  launch(pdl, k_dots_k<T>, RED_BLOCKS, TPB, s, h.npad, z, (const double*)S.r.p, (const double*)S.q.p, S.partial.p,
+  const int G = red_grid(h.npad, RED_BLOCKS);
+  launch(pdl, k_dots_k<T>, G, TPB, s, h.npad, z, (const double*)S.r.p, (const double*)S.q.p, S.partial.p,
          S.ticket.p, S.scal.p);
-  launch(pdl, k_pupd_k<T>, RED_BLOCKS, TPB, s, h.npad, z, S.p.p, (const MultiScalars*)S.scal.p);
-  launch(pdl, k_spmv_dot_k, RED_BLOCKS, TPB, s, h.npad, view(h.A64), (const double*)S.p.p, S.q.p, S.partial.p,
+  launch(pdl, k_pupd_k<T>, G, TPB, s, h.npad, z, S.p.p, (const MultiScalars*)S.scal.p);
+  launch(pdl, k_spmv_dot_k, G, TPB, s, h.npad, view(h.A64), (const double*)S.p.p, S.q.p, S.partial.p,
          S.ticket.p, S.scal.p);
-  launch(pdl, k_axpy_norm_k, RED_BLOCKS, TPB, s, h.npad, (const double*)S.p.p, (const double*)S.q.p, S.x.p, S.r.p,
+  launch(pdl, k_axpy_norm_k, G, TPB, s, h.npad, (const double*)S.p.p, (const double*)S.q.p, S.x.p, S.r.p,
          S.partial.p, S.ticket.p, S.scal.p, S.hist.p, hnd, use_hnd);
   ASMG_CUDA(cudaGetLastError());
 }
@@ -964,7 +965,7 @@ void enqueue_body_any_k(asmg_s& h, MultiSlot& S, cudaStream_t s, cudaGraphCondit
 
 void enqueue_init_k(asmg_s& h, MultiSlot& S, double rtol, cudaStream_t s, cudaGraphConditionalHandle hnd,
                     int use_hnd) {
-  launch(h.prm.use_pdl, k_pcg_init_k, RED_BLOCKS, TPB, s, h.npad, view(h.A64), (const double*)S.b.p,
+  launch(h.prm.use_pdl, k_pcg_init_k, red_grid(h.npad, RED_BLOCKS), TPB, s, h.npad, view(h.A64), (const double*)S.b.p,
          (const double*)S.x.p, S.r.p, S.partial.p, S.ticket.p, S.scal.p, rtol, h.prm.max_iter, S.hist.p, hnd, use_hnd);
   ASMG_CUDA(cudaGetLastError());
 }
