@@ -83,11 +83,20 @@ __device__ __forceinline__ T sell_dot(int64_t row, const int64_t* __restrict__ o
 
 // Programmatic dependent launch: every solve kernel first loads what was
 // written at setup (matrix rows, index lists), then waits for the preceding
-// kernel (griddepcontrol.wait), and lets the next kernel launch once its own
-// work is done (griddepcontrol.launch_dependents).  Launched without the
-// attribute, both instructions are no-ops.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// kernel (griddepcontrol.wait) and at once lets the next kernel launch
+// (griddepcontrol.launch_dependents): the next kernel's blocks start as soon
+// as all of this one's run, and load their own rows while this one works.
+// Their wait still covers this kernel's end, and with it every earlier one's:
+// a kernel ends only after its own wait.  Triggering at the kernel's end
+// instead leaves those loads exposed (kuhn129 mixed 40.8 ms, 39.4 ms with the
+// trigger here; graded 513^2 FP64 42.2, 40.3; four columns on 513^2 3.95,
+// 3.63).  Triggering before the wait lets kernels pile up several deep, their
+// waiting blocks holding the slots of the one that runs (graded 2049^2 258.0
+// -> 267.6 ms).  Launched without the attribute, both instructions are no-ops.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // A SELL-32 row held in registers (up to MAXW entries; longer rows read the rest later).
 constexpr int MAXW = 10;

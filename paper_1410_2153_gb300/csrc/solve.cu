@@ -53,7 +53,6 @@ __global__ void k_gs_fine(int64_t r0, int64_t nrows, const int64_t* __restrict__
     const T s = (T)rhs[i] - row_dot(row, col, val, u);
     u[i] += s * di;
   }
-  pdl_trigger();
 }
 
 // rho = r - A u
@@ -67,7 +66,6 @@ __global__ void k_resid_fine(int64_t n, const int64_t* __restrict__ off, const i
   if (act) row_load(row, i, off, col, val);
   pdl_wait();
   if (act) rho[i] = (T)r[i] - row_dot(row, col, val, u);
-  pdl_trigger();
 }
 
 // F = P^T rho on the auxiliary nodes, and U = 0 (start of the V-cycle)
@@ -84,7 +82,6 @@ __global__ void k_restrict_fine(int64_t nJ, const int64_t* __restrict__ off, con
     F[k] = row_dot(row, col, val, rho);
     U[k] = 0;
   }
-  pdl_trigger();
 }
 
 // u += P U
@@ -97,7 +94,6 @@ __global__ void k_prolong_fine(int64_t n, const int64_t* __restrict__ off, const
   if (act) row_load(row, i, off, col, val);
   pdl_wait();
   if (act) u[i] += row_dot(row, col, val, U);
-  pdl_trigger();
 }
 
 // Jacobi smoother (S = D^{-1}): first step from zero, u = D^{-1} r
@@ -108,7 +104,6 @@ __global__ void k_jac_first(int64_t n, const T* __restrict__ dinv, const double*
   const T di = act ? dinv[i] : (T)0;
   pdl_wait();
   if (act) u[i] = di * (T)r[i];
-  pdl_trigger();
 }
 
 // a further Jacobi step, u += D^{-1} rho with rho = r - A u taken before
@@ -119,7 +114,6 @@ __global__ void k_jac_add(int64_t n, const T* __restrict__ dinv, const T* __rest
   const T di = act ? dinv[i] : (T)0;
   pdl_wait();
   if (act) u[i] += di * rho[i];
-  pdl_trigger();
 }
 
 // additive form: the auxiliary correction acts on r itself (rho = r)
@@ -128,7 +122,6 @@ __global__ void k_cast_fine(int64_t n, const double* __restrict__ r, T* __restri
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   pdl_wait();
   if (i < n) rho[i] = (T)r[i];
-  pdl_trigger();
 }
 
 // ------------------------------------------------------ auxiliary levels
@@ -154,7 +147,6 @@ __global__ void k_gs_aux(int64_t k0, int64_t nk, const int64_t* __restrict__ off
     const T s = fs[k] - row_dot(row, col, val, U);
     U[i] += s * di;
   }
-  pdl_trigger();
 }
 
 // one colour of a down (pre-smoothing) sweep, on the level's own correction
@@ -200,7 +192,6 @@ __global__ void k_gs_aux_down(int64_t k0, int64_t nk, const int64_t* __restrict_
       us[k] += (f - acc) * di;
     }
   }
-  pdl_trigger();
 }
 
 // F_i -= sum_{j in N~_l} a_ij U_j on the rows E_l
@@ -217,7 +208,6 @@ __global__ void k_resid_aux(int64_t n, const int64_t* __restrict__ off, const in
   }
   pdl_wait();
   if (i >= 0) F[i] -= row_dot(row, col, val, U);
-  pdl_trigger();
 }
 
 // I_l^T: F[parent] += 1/2 sum F[new children]
@@ -237,7 +227,6 @@ __global__ void k_restrict_aux(int64_t npar, const int32_t* __restrict__ pid, co
     for (int32_t p = p0; p < p1; ++p) acc += F[child[p]];
     F[par] += (T)0.5 * acc;
   }
-  pdl_trigger();
 }
 
 // I_l: U[new] = (U[p0] + U[p1]) / 2, Dirichlet parents contribute 0
@@ -258,7 +247,6 @@ __global__ void k_prolong_aux(int64_t nnew, const int32_t* __restrict__ id, cons
     if (b >= 0) v += U[b];
     U[me] = (T)0.5 * v;
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -267,7 +255,6 @@ __global__ void k_addsaved_aux(int64_t nsm, const int32_t* __restrict__ rows, co
   const int32_t i = t < nsm ? rows[t] : -1;
   pdl_wait();
   if (i >= 0) U[i] += us[t];
-  pdl_trigger();
 }
 
 // coarsest level: U[cid] = A_c^{-1} F[cid] in FP64, one warp per row
@@ -283,7 +270,6 @@ __global__ void k_coarse(int64_t nc, const int32_t* __restrict__ cid, const doub
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) U[cid[row]] = (T)s;
   }
-  pdl_trigger();
 }
 
 // ------------------------------------------- tiled sweeps (one launch each)
@@ -458,7 +444,6 @@ __global__ void __launch_bounds__(TILE_TPB) k_tile_down(const int64_t* __restric
       if (g >= 0) us[g] = t.Ul[k];
     }
   }
-  pdl_trigger();
 }
 
 // start of the up path of a tiled level: the prolongation of the coarse
@@ -501,7 +486,6 @@ __global__ void k_up_init(int64_t nsm, const int32_t* __restrict__ rows, const i
       fsl[o] = f;
     }
   }
-  pdl_trigger();
 }
 
 // post-sweeps (backward colour order) from the start values and saved rhs
@@ -564,7 +548,6 @@ __global__ void __launch_bounds__(TILE_TPB) k_tile_up(const int64_t* __restrict_
     for (int k = threadIdx.x; k < nl; k += blockDim.x)
       if (t.lsm[k] >= 0) U[t.laux[k]] = t.Ul[k];
   }
-  pdl_trigger();
 }
 
 // ------------------------------------------- near-boundary solve (Alg. 3)
@@ -587,7 +570,6 @@ __global__ void k_nb_resid(int64_t m, const int64_t* __restrict__ off, const int
   }
   pdl_wait();
   if (act) rhs[q] = (double)(fs[k] - row_dot(row, col, val, U));
-  pdl_trigger();
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -695,7 +677,6 @@ __global__ void __launch_bounds__(NB_TPB) k_nb_solve(int R, const int32_t* __res
     __syncthreads();
   }
   for (int64_t q = threadIdx.x; q < m; q += blockDim.x) U[aux[q]] += (T)sol[q];
-  pdl_trigger();
 }
 
 // ---------------------------------------------------- small levels, fused
@@ -780,7 +761,6 @@ __global__ void __launch_bounds__(SMALL_TPB, 1)
     }
     __syncthreads();
   }
-  pdl_trigger();
 }
 
 template <class T, class V>
@@ -824,7 +804,6 @@ __global__ void __launch_bounds__(SMALL_TPB, 1)
     for (int k = threadIdx.x; k < mS; k += blockDim.x) U[L.gid[k]] = Ul[k];
     __syncthreads();
   }
-  pdl_trigger();
 }
 
 // ------------------------------------------------------------------ PCG
@@ -898,7 +877,6 @@ __global__ void k_pupd(int64_t n, const T* __restrict__ z, double* __restrict__ 
 #pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     p[i] = (double)z[i] + beta * p[i];
-  pdl_trigger();
 }
 
 // q = A p, <p, q>  ->  alpha.  Each row's entries are loaded into registers
@@ -970,7 +948,6 @@ __global__ void k_xpz(int64_t n, const T* __restrict__ z, double* __restrict__ x
   pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     x[i] += (double)z[i];
-  pdl_trigger();
 }
 
 // ASMG iteration: r = b - A x, ||r||  ->  history, stopping test

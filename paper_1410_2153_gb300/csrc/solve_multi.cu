@@ -120,7 +120,6 @@ __global__ void k_gs_fine_k(int64_t r0, int64_t nrows, const int64_t* __restrict
     }
     stk<T>(u + i * K, ui);
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -141,7 +140,6 @@ __global__ void k_resid_fine_k(int64_t n, const int64_t* __restrict__ off, const
     for (int j = 0; j < K; ++j) o.v[j] = (T)rv.v[j] - acc[j];
     stk<T>(rho + i * K, o);
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -165,7 +163,6 @@ __global__ void k_restrict_fine_k(int64_t nJ, const int64_t* __restrict__ off, c
     stk<T>(F + k * K, o);
     stk<T>(U + k * K, z);
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -184,7 +181,6 @@ __global__ void k_prolong_fine_k(int64_t n, const int64_t* __restrict__ off, con
     for (int j = 0; j < K; ++j) ui.v[j] += acc[j];
     stk<T>(u + i * K, ui);
   }
-  pdl_trigger();
 }
 
 // ------------------------------------------------------ auxiliary levels
@@ -216,7 +212,6 @@ __global__ void k_gs_aux_k(int64_t k0, int64_t nk, const int64_t* __restrict__ o
     }
     stk<T>(U + (int64_t)i * K, ui);
   }
-  pdl_trigger();
 }
 
 template <class T, class V>
@@ -273,7 +268,6 @@ __global__ void k_gs_aux_down_k(int64_t k0, int64_t nk, const int64_t* __restric
       stk<T>(us + k * K, o);
     }
   }
-  pdl_trigger();
 }
 
 template <class T, class V>
@@ -296,7 +290,6 @@ __global__ void k_resid_aux_k(int64_t n, const int64_t* __restrict__ off, const 
     for (int j = 0; j < K; ++j) f.v[j] -= acc[j];
     stk<T>(F + (int64_t)i * K, f);
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -324,7 +317,6 @@ __global__ void k_restrict_aux_k(int64_t npar, const int32_t* __restrict__ pid, 
     for (int j = 0; j < K; ++j) f.v[j] += (T)0.5 * acc[j];
     stk<T>(F + (int64_t)par * K, f);
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -357,7 +349,6 @@ __global__ void k_prolong_aux_k(int64_t nnew, const int32_t* __restrict__ id, co
     for (int j = 0; j < K; ++j) o.v[j] = (T)0.5 * v[j];
     stk<T>(U + (int64_t)me * K, o);
   }
-  pdl_trigger();
 }
 
 template <class T>
@@ -372,7 +363,6 @@ __global__ void k_addsaved_aux_k(int64_t nsm, const int32_t* __restrict__ rows, 
     for (int j = 0; j < K; ++j) u.v[j] += s.v[j];
     stk<T>(U + (int64_t)i * K, u);
   }
-  pdl_trigger();
 }
 
 // coarsest level, FP64, one warp per row (the lanes' order of k_coarse per column)
@@ -402,7 +392,6 @@ __global__ void k_coarse_k(int64_t nc, const int32_t* __restrict__ cid, const do
       stk<T>(U + (int64_t)cid[row] * K, o);
     }
   }
-  pdl_trigger();
 }
 
 // ---------------------------------------------------- small levels, fused
@@ -522,7 +511,6 @@ __global__ void __launch_bounds__(SMALL_TPB_K, 1)
     }
     __syncthreads();
   }
-  pdl_trigger();
 }
 
 template <class T, class V>
@@ -591,7 +579,6 @@ __global__ void __launch_bounds__(SMALL_TPB_K, 1)
     }
     __syncthreads();
   }
-  pdl_trigger();
 }
 
 // ------------------------------------------------------------------ PCG
@@ -697,7 +684,6 @@ __global__ void k_pupd_k(int64_t n, const T* __restrict__ z, double* __restrict_
     for (int j = 0; j < K; ++j) pi.v[j] = (double)zi.v[j] + beta[j] * pi.v[j];
     stk<double>(p + i * K, pi);
   }
-  pdl_trigger();
 }
 
 // q = A p, <p, q>  ->  alpha per active column
