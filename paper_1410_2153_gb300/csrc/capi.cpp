@@ -1,5 +1,6 @@
 // C ABI entry points (include/asmg.h) and the setup pipeline.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <chrono>
 #include <cmath>
@@ -56,17 +57,16 @@ void copy_out(double* dst, const double* src, int64_t n, cudaStream_t s) {
 
 int64_t pad32(int64_t n) { return (n + 31) / 32 * 32; }
 
-// Temporally blocked sweeps (asmg_params::tile_rows = 0): tile sizes tried in
-// order (own rows per tile) on levels of two colour classes and on levels of
-// more (whose longer dependency chains make deeper halos, which larger tiles
-// amortise: measured on graded 2049^2, 512-row tiles run the 5-class levels
-// 10-35% faster than 256-row ones, the 2-class levels no faster), the shared
-// memory a tile may use (two thread blocks per SM), and the largest halo
+// Temporally blocked sweeps (asmg_params::tile_rows = 0): own rows per tile on
+// levels of two colour classes, and on levels of more (whose longer dependency
+// chains make deeper halos, which larger tiles amortise) as a share of the rows
+// a block holds (1,024).  A larger share overflows and its tiles are halved
+// (graded 2049^2 with BF16 levels, post-sweeps at a share of 0.5: 4,104 tiles
+// where 3,758 of 0.375 do, 232.3 against 231.6 ms); a smaller one carries more
+// halo (0.38 down and 0.3 up: 235.1 ms).  TILE_MAX_HALO: the largest halo
 // accepted, as a multiple of the own rows.
-constexpr int TILE_SIZES_2COL[] = {256};
-constexpr int TILE_SIZES_MULTI[] = {512, 256};
-constexpr size_t TILE_SMEM = 110 * 1024;
-constexpr size_t TILE_SMEM_MAX = TILE_SMEM_LIMIT;  // one thread block per SM
+constexpr int TILE_ROWS_2COL = 256;
+constexpr double TILE_OWN_DOWN = 0.5, TILE_OWN_UP = 0.375;
 constexpr double TILE_MAX_HALO = 1.5;
 
 // f(begin, end) over contiguous ranges of [0, n) on host threads
@@ -230,7 +230,8 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
 }
 
 // Tiles of one sweep direction of a level (TileSweeps).  The own rows of a
-// tile are tile_rows consecutive smoothing rows in aux-ID order.  Its rows
+// tile are at most tile_rows consecutive smoothing rows in aux-ID order (a
+// tile whose rows do not fit the kernel's registers is cut in half).  Its rows
 // are the closure of the pairs (row, sweep) that the own rows' final values
 // depend on: a row's value after sweep s reads its own value after sweep
 // s - 1 and each coupled row j of N~_l either after sweep s (j's class is
@@ -242,16 +243,16 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
 // closure reads it.  Entries of the post-sweeps' rows whose column lies
 // outside N~_l become the tile's outside values.  SMd: SM-order rows with
 // their N~_l columns as SM rows; SM: the same rows with all columns as aux
-// IDs; pos: aux ID -> SM row.  Returns false (and builds nothing) when a tile
-// needs more than smem_max bytes of shared memory or more than 65,535 local
-// values, or when the halo exceeds max_halo times the own rows.
+// IDs; pos: aux ID -> SM row.  Returns false (and builds nothing) when a row
+// is longer than TILE_MAXW, when the closure of a single row does not fit, or
+// when the halo exceeds max_halo times the own rows.
 template <class T>
 bool build_tiles(bool up, int nu, int tile_rows, const std::vector<int64_t>& sel, const std::vector<int64_t>& cstart,
                  const std::vector<T>& dinv, const HostCSR& SMd, const HostCSR& SM, const std::vector<int32_t>& pos,
-                 size_t smem_max, double max_halo, unsigned max_threads, bool bf16, TileSweeps<T>& TS,
-                 cudaStream_t s) {
+                 double max_halo, unsigned max_threads, bool bf16, TileSweeps<T>& TS, cudaStream_t s) {
   const int64_t nsm = (int64_t)sel.size();
   const int ncol = (int)cstart.size() - 1;
+  const int max_slots = TILE_SLOTS_MAX;
   std::vector<int32_t> colr(nsm);
   for (int c = 0; c < ncol; ++c)
     for (int64_t k = cstart[c]; k < cstart[c + 1]; ++k) colr[k] = c;
@@ -259,250 +260,273 @@ bool build_tiles(bool up, int nu, int tile_rows, const std::vector<int64_t>& sel
   for (int64_t k = 0; k < nsm; ++k)
     if (sel[k] >= 0) own.push_back((int32_t)k);
   std::sort(own.begin(), own.end(), [&](int32_t a, int32_t b) { return sel[a] < sel[b]; });
-  const int64_t ntiles = ((int64_t)own.size() + tile_rows - 1) / tile_rows;
+  const int64_t nbase = ((int64_t)own.size() + tile_rows - 1) / tile_rows;
+  // a tile before its place in the level's arrays is known
   struct Out {
-    std::vector<int32_t> lrow, phase, ext;
-    std::vector<unsigned char> blob;
-    int64_t interior = 0, halo = 0, nnz = 0, nnz_real = 0;
-    bool ok = true;
+    int slots = 0;
+    std::vector<int32_t> lrow;         // [slots * TILE_THREADS] SM row, -2 - SM row (halo) or -1
+    std::vector<TileSlice> hdr;        // [slots * TILE_WARPS]
+    std::vector<int32_t> rptr;         // entries of each local row
+    std::vector<int32_t> rcol;         // local row, or -1 - e for the e-th outside value
+    std::vector<double> rval;
+    std::vector<int32_t> ext;
+    uint32_t cmask = 0;
+    int64_t words = 0, vals = 0;       // rows of 32 in its words and values
+    TileLayout lay{};
+    int64_t interior = 0, halo = 0, nnz = 0;
+    int width = 0;
   };
-  std::vector<Out> out(ntiles);
-  const unsigned nt = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)max_threads, ntiles));
+  std::vector<std::vector<Out>> out(nbase);
+  std::atomic<bool> fits(true);
+  const unsigned nt = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)max_threads, nbase));
   std::vector<std::thread> th;
-  for (unsigned w = 0; w < nt; ++w)
-    th.emplace_back([&, w] {
-      // stamps: mark[sw * nsm + k] == tile: pair (k, sw) needed; inx[k] == tile: k kept
+  for (unsigned wk = 0; wk < nt; ++wk)
+    th.emplace_back([&, wk] {
+      // stamps: mark[sw * nsm + k] == tag: pair (k, sw) needed; inx[k] == tag: k kept
       std::vector<int32_t> mark((size_t)nu * nsm, -1), inx(nsm, -1), loc(nsm, 0), ownm(nsm, -1);
       std::vector<std::pair<int32_t, int32_t>> stack;
       std::vector<int32_t> X;
       std::unordered_map<int32_t, int32_t> extpos;
-      std::vector<int64_t> rptr;
-      std::vector<int32_t> rcol;
-      std::vector<double> rval;
       std::vector<std::pair<int64_t, int32_t>> rlen;
-      for (int64_t t = ntiles * w / nt; t < ntiles * (w + 1) / nt; ++t) {
-        const int32_t tag = (int32_t)t;
-        stack.clear();
-        X.clear();
-        auto keep = [&](int32_t k) {
-          if (inx[k] != tag) {
-            inx[k] = tag;
-            X.push_back(k);
-          }
-        };
-        auto need = [&](int32_t k, int sw) {
-          int32_t& m = mark[(size_t)sw * nsm + k];
-          if (m != tag) {
-            m = tag;
-            stack.push_back({k, sw});
-          }
-        };
-        const int64_t o0 = t * tile_rows, o1 = std::min<int64_t>((int64_t)own.size(), o0 + tile_rows);
-        for (int64_t q = o0; q < o1; ++q) {
-          ownm[own[q]] = tag;
-          need(own[q], nu - 1);
-        }
-        while (!stack.empty()) {
-          const auto [k, sw] = stack.back();
-          stack.pop_back();
-          keep(k);
-          if (sw >= 1) need(k, sw - 1);
-          for (int64_t p = SMd.ptr[k]; p < SMd.ptr[k + 1]; ++p) {
-            const int32_t j = SMd.col[p];
-            if (j == k) continue;
-            const int cj = colr[j], ck = colr[k];
-            const bool before = up ? cj > ck : cj < ck;
-            if (before || cj == ck) need(j, sw);
-            if (!before) {
-              if (sw >= 1) need(j, sw - 1);
-              else if (up) keep(j);
+      std::vector<std::pair<int64_t, int64_t>> todo;
+      int32_t tag = -1;
+      for (int64_t t = nbase * wk / nt; t < nbase * (wk + 1) / nt && fits.load(std::memory_order_relaxed); ++t) {
+        todo.assign(1, {t * tile_rows, std::min<int64_t>((int64_t)own.size(), (t + 1) * tile_rows)});
+        while (!todo.empty()) {
+          const auto [o0, o1] = todo.back();
+          todo.pop_back();
+          ++tag;
+          stack.clear();
+          X.clear();
+          auto keep = [&](int32_t k) {
+            if (inx[k] != tag) {
+              inx[k] = tag;
+              X.push_back(k);
             }
-          }
-        }
-        // local rows: grouped by colour class (SM order); within a class,
-        // where order does not matter, longest rows first so that the slices
-        // carry little padding
-        auto row_len = [&](int32_t k) {
-          int64_t n = 0;
-          if (!up) {
-            for (int64_t p = SMd.ptr[k]; p < SMd.ptr[k + 1]; ++p) n += inx[SMd.col[p]] == tag;
-          } else {
-            for (int64_t p = SM.ptr[k]; p < SM.ptr[k + 1]; ++p) {
-              const int32_t j = pos[SM.col[p]];
-              n += j < 0 || inx[j] == tag;
+          };
+          auto need = [&](int32_t k, int sw) {
+            int32_t& m = mark[(size_t)sw * nsm + k];
+            if (m != tag) {
+              m = tag;
+              stack.push_back({k, sw});
             }
+          };
+          for (int64_t q = o0; q < o1; ++q) {
+            ownm[own[q]] = tag;
+            need(own[q], nu - 1);
           }
-          return n;
-        };
-        std::sort(X.begin(), X.end());
-        rlen.resize(X.size());
-        for (size_t q = 0; q < X.size(); ++q) rlen[q] = {-row_len(X[q]), X[q]};
-        Out& O = out[t];
-        O.phase.assign(ncol + 1, 0);
-        size_t x = 0;
-        for (int c = 0; c < ncol; ++c) {
-          O.phase[c] = (int32_t)O.lrow.size();
-          const size_t x0 = x;
-          while (x < X.size() && X[x] < cstart[c + 1]) ++x;
-          std::sort(rlen.begin() + x0, rlen.begin() + x);
-          for (size_t q = x0; q < x; ++q) {
-            const int32_t k = rlen[q].second;
-            loc[k] = (int32_t)O.lrow.size();
-            const bool mine = ownm[k] == tag;
-            O.lrow.push_back(mine ? k : -2 - k);
-            if (mine) ++O.interior;
-            else ++O.halo;
-          }
-          while (O.lrow.size() % 32) O.lrow.push_back(-1);
-        }
-        O.phase[ncol] = (int32_t)O.lrow.size();
-        const int nl = (int)O.lrow.size();
-        // rows with local columns (outside values numbered after the rows)
-        extpos.clear();
-        rptr.assign(1, 0);
-        rcol.clear();
-        rval.clear();
-        for (int32_t g : O.lrow) {
-          if (g != -1) {
-            const int32_t k = g >= 0 ? g : -2 - g;
-            if (!up) {
-              for (int64_t p = SMd.ptr[k]; p < SMd.ptr[k + 1]; ++p) {
-                const int32_t j = SMd.col[p];
-                if (inx[j] != tag) continue;
-                rcol.push_back(loc[j]);
-                rval.push_back(SMd.val[p]);
+          while (!stack.empty()) {
+            const auto [k, sw] = stack.back();
+            stack.pop_back();
+            keep(k);
+            if (sw >= 1) need(k, sw - 1);
+            for (int64_t p = SMd.ptr[k]; p < SMd.ptr[k + 1]; ++p) {
+              const int32_t j = SMd.col[p];
+              if (j == k) continue;
+              const int cj = colr[j], ck = colr[k];
+              const bool before = up ? cj > ck : cj < ck;
+              if (before || cj == ck) need(j, sw);
+              if (!before) {
+                if (sw >= 1) need(j, sw - 1);
+                else if (up) keep(j);
               }
+            }
+          }
+          // rows by colour class; within a class, where order does not
+          // matter, longest first so that the slices carry little padding
+          auto row_len = [&](int32_t k) {
+            int64_t n = 0;
+            if (!up) {
+              for (int64_t p = SMd.ptr[k]; p < SMd.ptr[k + 1]; ++p) n += inx[SMd.col[p]] == tag;
             } else {
               for (int64_t p = SM.ptr[k]; p < SM.ptr[k + 1]; ++p) {
-                const int32_t a = SM.col[p];
-                const int32_t j = pos[a];
-                if (j >= 0) {
-                  if (inx[j] != tag) continue;
-                  rcol.push_back(loc[j]);
-                } else {
-                  auto it = extpos.find(a);
-                  int32_t e;
-                  if (it == extpos.end()) {
-                    e = (int32_t)O.ext.size();
-                    extpos.emplace(a, e);
-                    O.ext.push_back(a);
-                  } else {
-                    e = it->second;
-                  }
-                  rcol.push_back(nl + e);
-                }
-                rval.push_back(SM.val[p]);
+                const int32_t j = pos[SM.col[p]];
+                n += j < 0 || inx[j] == tag;
               }
             }
+            return n;
+          };
+          std::sort(X.begin(), X.end());
+          rlen.resize(X.size());
+          for (size_t q = 0; q < X.size(); ++q) rlen[q] = {-row_len(X[q]), X[q]};
+          Out O;
+          std::vector<std::array<int64_t, 3>> slices;  // first and last + 1 in rlen, colour
+          for (size_t x = 0, c = 0; c < (size_t)ncol; ++c) {
+            const size_t x0 = x;
+            while (x < X.size() && X[x] < cstart[c + 1]) ++x;
+            std::sort(rlen.begin() + x0, rlen.begin() + x);
+            for (size_t q = x0; q < x; q += 32)
+              slices.push_back({(int64_t)q, (int64_t)std::min(x, q + 32), (int64_t)c});
           }
-          rptr.push_back((int64_t)rcol.size());
-        }
-        if (nl + (int64_t)O.ext.size() > 65535) {
-          O.ok = false;
-          continue;
-        }
-        // the tile's block: SELL-32 slice offsets, uint16 columns, values, then
-        // per local row the diagonal inverse, the SM row (own: k, halo:
-        // -2 - k, padding: -1) and the aux ID, then the outside values' aux
-        // IDs; each part padded to 16 bytes
-        const int nsl = nl / 32;
-        std::vector<int32_t> soff(nsl + 1, 0);
-        for (int sl = 0; sl < nsl; ++sl) {
-          int64_t wmax = 0;
-          for (int r = sl * 32; r < sl * 32 + 32; ++r) wmax = std::max(wmax, rptr[r + 1] - rptr[r]);
-          soff[sl + 1] = soff[sl] + (int32_t)(wmax * 32);
-        }
-        const int64_t ne_ = soff[nsl], nx = (int64_t)O.ext.size();
-        O.nnz = ne_;
-        O.nnz_real = rptr[nl];
-        const TileLayout lay =
-            tile_layout((int64_t)nl, ne_, nx, (int64_t)sizeof(T), bf16 ? (int64_t)sizeof(bf16v) : (int64_t)sizeof(T));
-        O.blob.assign(lay.end, 0);
-        std::memcpy(O.blob.data(), soff.data(), 4 * (size_t)(nsl + 1));
-        uint16_t* cc = reinterpret_cast<uint16_t*>(O.blob.data() + lay.col);
-        T* vv = reinterpret_cast<T*>(O.blob.data() + lay.val);
-        bf16v* vb = reinterpret_cast<bf16v*>(O.blob.data() + lay.val);
-        for (int r = 0; r < nl; ++r) {
-          const int sl = r / 32, lane = r % 32;
-          int64_t e = 0;
-          for (int64_t p = rptr[r]; p < rptr[r + 1]; ++p, ++e) {
-            cc[soff[sl] + e * 32 + lane] = (uint16_t)rcol[p];
-            if (bf16)
-              vb[soff[sl] + e * 32 + lane].bits = bf16_bits((float)rval[p]);
-            else
-              vv[soff[sl] + e * 32 + lane] = (T)rval[p];
+          // the slices of a class spread over the warps, each warp's slots filled evenly
+          bool ok = (int)slices.size() <= max_slots * TILE_WARPS;
+          if (ok) {
+            O.slots = std::max(1, ((int)slices.size() + TILE_WARPS - 1) / TILE_WARPS);
+            O.lrow.assign((size_t)O.slots * TILE_THREADS, -1);
+            O.hdr.assign((size_t)O.slots * TILE_WARPS, TileSlice{0, 0, 0, -1});
+            int total[TILE_WARPS] = {}, inclass[TILE_WARPS] = {};
+            int64_t cls = -1;
+            for (const auto& sl : slices) {
+              if (sl[2] != cls) std::fill(inclass, inclass + TILE_WARPS, 0);
+              cls = sl[2];
+              int w = -1;
+              for (int v = 0; v < TILE_WARPS; ++v)
+                if (total[v] < O.slots &&
+                    (w < 0 || inclass[v] < inclass[w] || (inclass[v] == inclass[w] && total[v] < total[w])))
+                  w = v;
+              const int slot = total[w]++;
+              ++inclass[w];
+              TileSlice& H = O.hdr[(size_t)slot * TILE_WARPS + w];
+              H.colour = (int16_t)cls;
+              H.w = (int16_t)std::min<int64_t>(-rlen[sl[0]].first, INT16_MAX);
+              O.width = std::max<int>(O.width, H.w);
+              for (int64_t q = sl[0]; q < sl[1]; ++q) {
+                const int32_t k = rlen[q].second, r = slot * TILE_THREADS + w * 32 + (int32_t)(q - sl[0]);
+                loc[k] = r;
+                const bool mine = ownm[k] == tag;
+                O.lrow[r] = mine ? k : -2 - k;
+                ++(mine ? O.interior : O.halo);
+              }
+              O.cmask |= 1u << std::min<int64_t>(cls, 31);
+            }
+            extpos.clear();
+            O.rptr.assign(1, 0);
+            for (int32_t g : O.lrow) {
+              if (g != -1) {
+                const int32_t k = g >= 0 ? g : -2 - g;
+                const HostCSR& M = up ? SM : SMd;
+                for (int64_t p = M.ptr[k]; p < M.ptr[k + 1]; ++p) {
+                  const int32_t a = M.col[p], j = up ? pos[a] : a;
+                  if (j >= 0) {
+                    if (inx[j] != tag) continue;
+                    O.rcol.push_back(loc[j]);
+                  } else {
+                    const auto it = extpos.emplace(a, (int32_t)O.ext.size());
+                    if (it.second) O.ext.push_back(a);
+                    O.rcol.push_back(-1 - it.first->second);
+                  }
+                  O.rval.push_back(M.val[p]);
+                }
+              }
+              O.rptr.push_back((int32_t)O.rcol.size());
+            }
+            // a row of 32 words per entry (BF16) or per two entries, a row of
+            // 32 values per entry (FP32, FP64)
+            for (TileSlice& H : O.hdr) {
+              H.words = (uint16_t)O.words;
+              H.vals = (uint16_t)O.vals;
+              O.words += bf16 ? H.w : (H.w + 1) / 2;
+              O.vals += bf16 ? 0 : H.w;
+              O.nnz += 32 * (int64_t)H.w;
+            }
           }
-        }
-        T* dd = reinterpret_cast<T*>(O.blob.data() + lay.dinv);
-        int32_t* ls = reinterpret_cast<int32_t*>(O.blob.data() + lay.lsm);
-        int32_t* la = reinterpret_cast<int32_t*>(O.blob.data() + lay.laux);
-        for (int r = 0; r < nl; ++r) {
-          const int32_t g = O.lrow[r];
-          ls[r] = g;
-          if (g == -1) {
-            dd[r] = (T)0;
-            la[r] = -1;
-          } else {
-            const int32_t k = g >= 0 ? g : -2 - g;
-            dd[r] = dinv[k];
-            la[r] = (int32_t)sel[k];
+          if (ok && O.width > TILE_MAXW) {
+            fits = false;
+            break;
           }
+          if (ok) {
+            const int64_t values = max_slots * TILE_THREADS + (int64_t)O.ext.size();
+            O.lay = tile_layout(O.slots, (int)O.words, (int)O.vals, (int)O.ext.size(), sizeof(T));
+            ok = values <= TILE_VALUES_MAX && values * (int64_t)sizeof(T) + O.lay.end + 1024 <= TILE_SMEM_MAX;
+          }
+          if (!ok) {
+            if (o1 - o0 <= 1) {
+              fits = false;
+              break;
+            }
+            const int64_t mid = (o0 + o1) / 2;
+            todo.push_back({mid, o1});
+            todo.push_back({o0, mid});
+            continue;
+          }
+          out[t].push_back(std::move(O));
         }
-        if (nx) std::memcpy(O.blob.data() + lay.ext, O.ext.data(), 4 * (size_t)nx);
       }
     });
   for (auto& x : th) x.join();
-  int64_t maxloc = 0, maxext = 0, maxblob = 0, interior = 0, halo = 0;
-  for (auto& O : out) {
-    if (!O.ok) return false;
-    maxloc = std::max<int64_t>(maxloc, (int64_t)O.lrow.size());
-    maxext = std::max<int64_t>(maxext, (int64_t)O.ext.size());
-    maxblob = std::max<int64_t>(maxblob, (int64_t)O.blob.size());
-    interior += O.interior;
-    halo += O.halo;
-  }
-  const size_t smem = (size_t)maxblob + (size_t)(maxloc + (maxext + 3) / 4 * 4) * sizeof(T) + (size_t)maxloc * sizeof(T);
-  if (smem > smem_max || (double)halo > max_halo * (double)interior) return false;
-  std::vector<int64_t> loc_off(1, 0), blob_off(1, 0), ext_off(1, 0);
-  std::vector<int32_t> phase;
-  std::vector<unsigned char> blob;
-  for (auto& O : out) {
-    loc_off.push_back(loc_off.back() + (int64_t)O.lrow.size());
-    blob_off.push_back(blob_off.back() + (int64_t)O.blob.size());
-    ext_off.push_back(ext_off.back() + (int64_t)O.ext.size());
-    phase.insert(phase.end(), O.phase.begin(), O.phase.end());
-    blob.insert(blob.end(), O.blob.begin(), O.blob.end());
+  if (!fits.load()) return false;
+  std::vector<const Out*> tiles;
+  for (auto& v : out)
+    for (auto& O : v) tiles.push_back(&O);
+  const int64_t ntiles = (int64_t)tiles.size();
+  std::vector<TileHead> head(ntiles);
+  int64_t bytes = 0;
+  for (int64_t t = 0; t < ntiles; ++t) {
+    const Out& O = *tiles[t];
+    TS.slots = std::max(TS.slots, O.slots);
+    TS.width = std::max(TS.width, O.width);
+    TS.maxext = std::max(TS.maxext, (int)O.ext.size());
+    TS.maxblob = std::max(TS.maxblob, O.lay.end);
+    TS.interior += O.interior;
+    TS.halo += O.halo;
     TS.nnz += O.nnz;
-    TS.nnz_real += O.nnz_real;
+    TS.nnz_real += (int64_t)O.rcol.size();
+    head[t] = TileHead{bytes, (int32_t)O.lay.end, (int32_t)O.words, (int32_t)O.vals, (int32_t)O.ext.size(), O.slots,
+                       O.cmask};
+    bytes += O.lay.end;
   }
+  const int64_t per = (int64_t)TS.slots * TILE_THREADS;  // local rows of a tile
+  if ((double)TS.halo > max_halo * (double)TS.interior || ntiles * per > INT32_MAX ||
+      (int64_t)TS.smem() > TILE_SMEM_MAX) {
+    TS = TileSweeps<T>();
+    return false;
+  }
+  TS.ntiles = ntiles;
+  TS.nloc = ntiles * per;
+  std::vector<unsigned char> blob((size_t)bytes, 0);
+  std::vector<int32_t> lsm((size_t)(up ? TS.nloc : 0), -1);
+  auto pack = [&](int64_t t0, int64_t t1) {
+    for (int64_t t = t0; t < t1; ++t) {
+      const Out& O = *tiles[t];
+      unsigned char* B = blob.data() + head[t].off;
+      TileSlice* hdr = reinterpret_cast<TileSlice*>(B);
+      uint32_t* words = reinterpret_cast<uint32_t*>(B + O.lay.words);
+      T* val = reinterpret_cast<T*>(B + O.lay.val);
+      T* dd = reinterpret_cast<T*>(B + O.lay.dinv);
+      int32_t* sm = reinterpret_cast<int32_t*>(B + O.lay.lsm);
+      int32_t* ax = reinterpret_cast<int32_t*>(B + O.lay.laux);
+      std::copy(O.hdr.begin(), O.hdr.end(), hdr);
+      std::copy(O.ext.begin(), O.ext.end(), reinterpret_cast<int32_t*>(B + O.lay.ext));
+      if (up) std::copy(O.lrow.begin(), O.lrow.end(), lsm.begin() + t * per);
+      for (int r = 0; r < O.slots * TILE_THREADS; ++r) {
+        const TileSlice& H = hdr[r / 32];
+        const int lane = r % 32;
+        const int32_t g = O.lrow[r];
+        sm[r] = g;
+        if (g == -1) continue;
+        const int32_t k = g >= 0 ? g : -2 - g;
+        ax[r] = (int32_t)sel[k];
+        dd[r] = dinv[k];
+        for (int32_t p = O.rptr[r], e = 0; p < O.rptr[r + 1]; ++p, ++e) {
+          const int32_t c = O.rcol[p];
+          const uint32_t off = (uint32_t)((c >= 0 ? c : per + (-1 - c)) * (int64_t)sizeof(T));
+          if (bf16) {
+            words[(H.words + e) * 32 + lane] = ((uint32_t)bf16_bits((float)O.rval[p]) << 16) | off;
+          } else {
+            words[(H.words + e / 2) * 32 + lane] |= off << (16 * (e & 1));
+            val[(H.vals + e) * 32 + lane] = (T)O.rval[p];
+          }
+        }
+      }
+    }
+  };
+  th.clear();
+  for (unsigned wk = 0; wk < nt; ++wk) th.emplace_back([&, wk] { pack(ntiles * wk / nt, ntiles * (wk + 1) / nt); });
+  for (auto& x : th) x.join();
   if (up) {
     // where each SM row sits in tile order (own and halo copies)
     std::vector<int64_t> pptr(nsm + 1, 0);
-    for (auto& O : out)
-      for (int32_t g : O.lrow)
-        if (g != -1) ++pptr[(g >= 0 ? g : -2 - g) + 1];
+    for (int32_t g : lsm)
+      if (g != -1) ++pptr[(g >= 0 ? g : -2 - g) + 1];
     for (int64_t k = 0; k < nsm; ++k) pptr[k + 1] += pptr[k];
-    std::vector<int32_t> pos(pptr[nsm]);
+    std::vector<int32_t> place(pptr[nsm]);
     std::vector<int64_t> fill(pptr.begin(), pptr.end() - 1);
-    for (int64_t t = 0; t < ntiles; ++t)
-      for (size_t k = 0; k < out[t].lrow.size(); ++k) {
-        const int32_t g = out[t].lrow[k];
-        if (g != -1) pos[fill[g >= 0 ? g : -2 - g]++] = (int32_t)(loc_off[t] + (int64_t)k);
-      }
+    for (int64_t q = 0; q < TS.nloc; ++q)
+      if (lsm[q] != -1) place[fill[lsm[q] >= 0 ? lsm[q] : -2 - lsm[q]]++] = (int32_t)q;
     TS.pos_ptr.upload(pptr, s);
-    TS.pos.upload(pos, s);
+    TS.pos.upload(place, s);
   }
-  TS.ntiles = ntiles;
-  TS.nloc = loc_off.back();
-  TS.maxloc = (int)maxloc;
-  TS.maxext = (int)((maxext + 3) / 4 * 4);  // F follows U in shared memory, 16-byte aligned
-  TS.maxblob = maxblob;
-  TS.interior = interior;
-  TS.halo = halo;
-  TS.loc_off.upload(loc_off, s);
-  TS.blob_off.upload(blob_off, s);
-  TS.ext_off.upload(ext_off, s);
-  TS.phase.upload(phase, s);
+  TS.head.upload(head, s);
   TS.blob.upload(blob, s);
   ASMG_CUDA(cudaStreamSynchronize(s));
   return true;
@@ -636,25 +660,21 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
     }
   D.sm_rows.upload(rows, s);
   D.sm_dinv.upload(dinv, s);
-  // temporal blocking of the level's sweeps (TileSweeps): the first tile size
-  // of TILE_SIZES_2COL / TILE_SIZES_MULTI (or the requested size) whose tiles
-  // fit the shared-memory budget with a halo of at most TILE_MAX_HALO times the
-  // own rows; the level needs at least two tiles and every new node must be a
-  // smoothing row (k_up_init prolongs through the smoothing rows)
+  // temporal blocking of the level's sweeps (TileSweeps), with the default own
+  // rows per tile and a halo of at most TILE_MAX_HALO times the own rows, or the
+  // requested rows and any halo; the level needs at least two tiles and every
+  // new node must be a smoothing row (k_up_init prolongs through the smoothing
+  // rows)
   D.tiled = false;
   if (prm.tile_rows >= 0 && prm.nu_post >= 1) {
     bool ok = true;
     for (int32_t id : L.new_id)
       if (pos[id] < 0) ok = false;
-    std::vector<int> sizes;
-    if (prm.tile_rows > 0) sizes.push_back(prm.tile_rows);
-    else if (ncol <= 2) sizes.assign(std::begin(TILE_SIZES_2COL), std::end(TILE_SIZES_2COL));
-    else sizes.assign(std::begin(TILE_SIZES_MULTI), std::end(TILE_SIZES_MULTI));
-    // a requested size takes any halo and up to TILE_SMEM_MAX of shared memory
     const double max_halo = prm.tile_rows > 0 ? 1e30 : TILE_MAX_HALO;
-    const size_t smem_max = prm.tile_rows > 0 ? TILE_SMEM_MAX : TILE_SMEM;
-    for (int trows : sizes) {
-      if (!ok || D.nsm_real < 2 * (int64_t)trows) continue;
+    const int cap = TILE_SLOTS_MAX * TILE_THREADS;
+    const int rd = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN_DOWN);
+    const int ru = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN_UP);
+    if (ok && D.nsm_real >= 2 * (int64_t)std::max(rd, ru)) {
       // the two directions are built at the same time, each on half the host threads
       TileSweeps<T> td, tu;
       const unsigned half = std::max(1u, std::thread::hardware_concurrency() / 2);
@@ -662,34 +682,32 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
       std::exception_ptr eu, ed;
       std::thread up_th([&] {
         try {
-          oku = build_tiles<T>(true, prm.nu_post, trows, sel, D.cstart, dinv, SMd, SM, pos, smem_max, max_halo, half,
-                               bf16, tu, s);
+          oku = build_tiles<T>(true, prm.nu_post, ru, sel, D.cstart, dinv, SMd, SM, pos, max_halo, half, bf16, tu, s);
         } catch (...) {
           eu = std::current_exception();
         }
       });
       try {
-        okd = build_tiles<T>(false, prm.nu_pre, trows, sel, D.cstart, dinv, SMd, SM, pos, smem_max, max_halo, half,
-                             bf16, td, s);
+        okd = build_tiles<T>(false, prm.nu_pre, rd, sel, D.cstart, dinv, SMd, SM, pos, max_halo, half, bf16, td, s);
       } catch (...) {
         ed = std::current_exception();
       }
       up_th.join();
       if (ed) std::rethrow_exception(ed);
       if (eu) std::rethrow_exception(eu);
-      if (!okd || !oku) continue;
-      std::vector<int32_t> p0(sel.size(), -3), p1(sel.size(), -3);
-      for (size_t t = 0; t < L.new_id.size(); ++t) {
-        p0[pos[L.new_id[t]]] = L.new_p0[t];
-        p1[pos[L.new_id[t]]] = L.new_p1[t];
+      if (okd && oku) {
+        std::vector<int32_t> p0(sel.size(), -3), p1(sel.size(), -3);
+        for (size_t t = 0; t < L.new_id.size(); ++t) {
+          p0[pos[L.new_id[t]]] = L.new_p0[t];
+          p1[pos[L.new_id[t]]] = L.new_p1[t];
+        }
+        D.sm_par0.upload(p0, s);
+        D.sm_par1.upload(p1, s);
+        D.tdown = std::move(td);
+        D.tup = std::move(tu);
+        D.tiled = D.tiled_down = D.tiled_up = true;
+        D.tile_rows = rd;
       }
-      D.sm_par0.upload(p0, s);
-      D.sm_par1.upload(p1, s);
-      D.tdown = std::move(td);
-      D.tup = std::move(tu);
-      D.tiled = D.tiled_down = D.tiled_up = true;
-      D.tile_rows = trows;
-      break;
     }
   }
   // residual rows: every row with an entry in a smoothing column

@@ -304,58 +304,90 @@ struct SmallLevelDev {
 // shared memory and write back only the tile's own rows.  The results equal
 // the class-by-class launches bit for bit (see build_tiles).
 //
-// A tile's rows are stored as one block of bytes (16-byte aligned, a multiple
-// of 16 bytes long; layout in TileLayout) that the kernel copies into shared
-// memory with one bulk copy: SELL-32 slice offsets (int32, relative to the
-// tile), the column of every entry (uint16: a local row, or nl + e for the
-// tile's e-th outside value), the values (T), then per local row its
-// diagonal inverse (T), SM row (int32: own row k, halo row -2 - k, padding
-// -1) and aux ID (int32), then the outside values' aux IDs.  Outside values
-// are the columns outside N~_l of the post-sweeps' rows: the sweeps do not
-// change them, so the tile reads them from U once.
-// dynamic shared memory a tile launch may use (bytes)
-constexpr size_t TILE_SMEM_LIMIT = 200 * 1024;
+// A thread block of TILE_THREADS threads runs a tile with the tile's matrix in
+// registers: a thread holds up to `slots` rows, one per slot, and the rows of
+// a (slot, warp) pair are a slice of 32 rows of one colour class (SELL-32,
+// width = the slice's longest row), so a colour phase is one test per slot.
+// The rows' values live in shared memory: local row r = slot * TILE_THREADS +
+// thread at byte r * sizeof(T), then the tile's outside values (the columns
+// outside N~_l of the post-sweeps' rows, which the sweeps do not change).
+// Stored columns are those byte offsets, in 16 bits.  A tile's setup data is
+// one block of bytes (TileLayout), copied into shared memory by one bulk copy
+// while the block sweeps its previous tile.
+constexpr int TILE_THREADS = 256;
+constexpr int TILE_WARPS = TILE_THREADS / 32;
+constexpr int TILE_MAXW = 16;                 // longest row a tile kernel holds
+constexpr int64_t TILE_VALUES_MAX = 5632;     // values of a tile: byte offsets fit 16 bits
+constexpr int64_t TILE_SMEM_MAX = 100 * 1024; // shared memory of a block (two per SM)
 
-struct TileLayout {
-  int64_t col, val, dinv, lsm, laux, ext, end;  // byte offsets of the parts, and the total
+// most slots per thread: the entries of a row of 8 take 8 registers as packed
+// (BF16 value, column) words, 12 as FP32 values with paired columns, 20 as FP64
+constexpr int TILE_SLOTS_MAX = 4;
+
+// one (slot, warp) slice: its first row of 32 in the tile's words and values,
+// its width, its colour class (-1: empty slice)
+struct TileSlice {
+  uint16_t words, vals;
+  int16_t w, colour;
 };
 
-// nl local rows (a multiple of 32), ne stored entries, nx outside values, s bytes per value
-// (diagonal inverses), sv bytes per stored matrix value
-inline __host__ __device__ TileLayout tile_layout(int64_t nl, int64_t ne, int64_t nx, int64_t s, int64_t sv) {
-  auto pad16 = [](int64_t b) { return (b + 15) & ~(int64_t)15; };
+// the block of a tile with `slots` slots: slices [slots * TILE_WARPS], words
+// (BF16: value bits << 16 | column offset, a row of 32 per entry; else two
+// columns per word), FP32 / FP64 values (a row of 32 per entry), then per
+// local row its diagonal inverse (T), SM row (int32: own row k, halo row
+// -2 - k, padding -1) and aux ID (int32), then the outside values' aux IDs
+struct TileLayout {
+  int64_t words, val, dinv, lsm, laux, ext, end;  // byte offsets of the parts, and the total
+};
+// nwords, nvals: rows of 32; s: bytes per value (T)
+inline __host__ __device__ TileLayout tile_layout(int slots, int nwords, int nvals, int nx, int64_t s) {
+  const int64_t nl = (int64_t)slots * TILE_THREADS;
   TileLayout t;
-  t.col = pad16(4 * (nl / 32 + 1));
-  t.val = t.col + pad16(2 * ne);
-  t.dinv = t.val + pad16(sv * ne);
-  t.lsm = t.dinv + pad16(s * nl);
-  t.laux = t.lsm + pad16(4 * nl);
-  t.ext = t.laux + pad16(4 * nl);
-  t.end = t.ext + pad16(4 * nx);
+  t.words = (int64_t)slots * TILE_WARPS * (int64_t)sizeof(TileSlice);
+  t.val = t.words + 128 * (int64_t)nwords;
+  t.dinv = t.val + 32 * s * nvals;
+  t.lsm = t.dinv + s * nl;
+  t.laux = t.lsm + 4 * nl;
+  t.ext = t.laux + 4 * nl;
+  t.end = (t.ext + 4 * (int64_t)nx + 15) / 16 * 16;
   return t;
 }
 
+// where a tile's block lies and what it holds
+struct TileHead {
+  int64_t off;             // byte offset of its block (a multiple of 16)
+  int32_t bytes;           // a multiple of 16
+  int32_t nwords, nvals, nx;
+  int32_t slots;
+  uint32_t cmask;          // colour classes 0..30 present, bit 31: any other
+};
+
+template <class T>
+struct TileView {
+  const TileHead* head;
+  const unsigned char* blob;
+  int64_t ntiles;
+};
+
 template <class T>
 struct TileSweeps {
-  int64_t ntiles = 0, nloc = 0;  // tiles, local rows (each colour group padded to 32)
-  int maxloc = 0, maxext = 0;    // largest local row count and outside-value count of a tile
-  int tpb = 256;                 // threads per block
-  int64_t maxblob = 0;           // largest tile block (bytes)
+  int64_t ntiles = 0, nloc = 0;  // tiles, local rows (ntiles * slots * TILE_THREADS)
+  int slots = 0, width = 0;      // slots per thread, longest row
+  int maxext = 0;                // largest outside-value count of a tile
+  int64_t maxblob = 0;           // largest block (bytes)
   int64_t interior = 0, halo = 0;  // real rows: the tiles' own, and halo copies
   int64_t nnz = 0, nnz_real = 0;   // stored / real entries over all tiles
-  DBuf<int64_t> loc_off;         // [ntiles + 1] first local row of each tile (multiples of 32)
-  DBuf<int64_t> blob_off;        // [ntiles + 1] byte offset of each tile's block
-  DBuf<int64_t> ext_off;         // [ntiles + 1] first outside value of each tile
-  DBuf<int32_t> phase;           // [ntiles * (ncol + 1)] colour-class starts within each tile
-  DBuf<unsigned char> blob;      // the tiles' blocks
+  DBuf<TileHead> head;
+  DBuf<unsigned char> blob;
   // post-sweeps: every place (local row of some tile) where each SM row sits,
   // own or halo (CSR by SM row), so that k_up_init can write the start values
-  // and saved rhs straight into tile order for the tiles to copy in
+  // and saved rhs straight into tile order
   DBuf<int64_t> pos_ptr;         // [nsm + 1]
   DBuf<int32_t> pos;             // positions in [0, nloc)
-  // shared memory of a launch: the largest block, then U (rows and outside
-  // values) and F of the largest tile
-  size_t smem() const { return (size_t)maxblob + (size_t)(maxloc + maxext) * sizeof(T) + (size_t)maxloc * sizeof(T); }
+  TileView<T> view() const { return TileView<T>{head.p, blob.p, ntiles}; }
+  // values (rows and outside values), then the block
+  int64_t smem_values() const { return ((int64_t)(slots * TILE_THREADS + maxext) * (int64_t)sizeof(T) + 15) / 16 * 16; }
+  size_t smem() const { return (size_t)(smem_values() + maxblob); }
 };
 
 // The exact near-boundary solve of Algorithm 3 on the device: the block

@@ -273,20 +273,29 @@ __global__ void k_coarse(int64_t nc, const int32_t* __restrict__ cid, const doub
 }
 
 // ------------------------------------------- tiled sweeps (one launch each)
-// One thread block per tile (see TileSweeps): the tile's rows -- its own rows
-// of N~_l plus the halo its sweeps read -- are copied into shared memory with
-// one bulk copy (cp.async.bulk, completion on an mbarrier), and the rows'
-// rhs, diagonal inverse and current value live there too; the colour phases
-// of all nu sweeps are separated by __syncthreads.  Each row is updated with
-// the same arithmetic, over the same stored entries in the same order, as
-// k_gs_aux_down / k_gs_aux do; the entries a tile leaves out are exactly
-// those whose value cannot reach the tile's own rows' results, so those
-// results equal the class-by-class launches bit for bit.  Halo results are
-// discarded.
-constexpr int TILE_TPB = 256;
-// bound on the wait for the bulk copy (SM clock cycles, about 1 s): when it
+// One thread block per tile (see TileSweeps), a persistent grid over the
+// tiles: the tile's rows -- its own rows of N~_l plus the halo its sweeps read
+// -- are held in registers for all nu sweeps, one row per slot and thread; the
+// rows' values live in shared memory and the colour phases are separated by
+// __syncthreads.  A tile's block of setup data arrives by one bulk copy
+// (cp.async.bulk, completion on an mbarrier): the first before the wait on the
+// previous kernel, each further one while the block sweeps the tile before.
+// Each row is updated with the same arithmetic, over the same stored entries
+// in the same order, as k_gs_aux_down / k_gs_aux do; the entries a tile leaves
+// out are exactly those whose value cannot reach the tile's own rows' results,
+// so those results equal the class-by-class launches bit for bit.  Halo
+// results are discarded.
+//
+// What bounds them is instructions and waits per colour phase, not the bytes:
+// with the rows read from shared memory entry by entry a level of 3.46 M rows
+// in five classes (graded 2049^2, BF16) took 118 us a direction at 18% of the
+// DRAM rate; with the rows in registers, no test per entry and four blocks per
+// SM it takes 78 us (graded 2049^2 solve 254.7 -> 231.6 ms, graded 513^2 FP64
+// 40.3 -> 38.2 ms, 331^2 mixed 2.04 -> 1.98 ms).
+
+// bound on the wait for a bulk copy (SM clock cycles, about 1 s): when it
 // expires the block records the timeout, waits once more (bounded) for its
-// copy to land, and skips its work
+// copy to land, and ends
 constexpr long long TILE_WAIT_CYCLES = 2000000000LL;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -301,156 +310,201 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// bounded wait for phase 0 of the mbarrier
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar) {
+// bounded wait for the mbarrier's phase of the given parity
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, 0))
+  while (!mbar_try_wait(bar, parity))
     if (clock64() - t0 > TILE_WAIT_CYCLES) return false;
   return true;
 }
 
-// Stage the tile's block of `bytes` bytes (16-byte aligned, multiple of 16)
-// into shared memory: thread 0 arms the barrier and issues the copy.  The
-// mbarrier lives in static shared memory.
-__device__ __forceinline__ void tile_stage(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  if (threadIdx.x == 0) {
-    const uint32_t b = smem_addr(bar);
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(b)
-                 : "memory");
-  }
-}
-
-// Every thread waits for the copy (bounded); false in every thread when any
-// thread's wait expired, after the timeout is recorded and the copy given a
-// second bounded wait.  inject != 0 (failure injection, asmg_params::
-// inject_timeout) takes the expired path without polling; the copy is still
-// waited for before the block exits.
-__device__ __forceinline__ bool tile_staged(uint64_t* bar, int* timeout, int inject) {
+// one thread: arm the barrier and start the copy of a tile's block; the block's
+// earlier reads of the same shared memory came before a __syncthreads
+__device__ __forceinline__ void tile_fetch(void* dst, const unsigned char* blob, const TileHead& h, uint64_t* bar) {
   const uint32_t b = smem_addr(bar);
-  __syncthreads();  // the barrier was initialised by thread 0 before this point
-  const bool ok = __syncthreads_and(!inject && mbar_wait_bounded(b));
-  if (!ok) {
-    if (threadIdx.x == 0) atomicExch(timeout, 1);
-    mbar_wait_bounded(b);
-    __syncthreads();
-  }
-  return ok;
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"((uint32_t)h.bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(blob + h.off), "r"((uint32_t)h.bytes), "r"(b)
+               : "memory");
 }
 
-// the row's entries in stored order, four loaded ahead of their use (the sum
-// is formed in the same order as a plain loop)
-template <class T, class V>
-__device__ __forceinline__ T tile_row_dot(int r, const int32_t* soff, const uint16_t* col, const V* val, const T* Ul) {
-  const int sl = r >> 5, lane = r & 31;
-  const int b = soff[sl], w = (soff[sl + 1] - b) >> 5;
+__device__ __forceinline__ void tile_bar_init(uint64_t* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// Every thread waits for the copy (bounded): false in every thread when any
+// thread's wait expired.  inject != 0 (failure injection, asmg_params::
+// inject_timeout) takes the expired path without polling.
+__device__ __forceinline__ bool tile_arrived(uint64_t* bar, uint32_t parity, int inject) {
+  return __syncthreads_and(!inject && mbar_wait_bounded(smem_addr(bar), parity));
+}
+
+// after an expired wait: record it and give the copy a second bounded wait
+// before the block ends
+__device__ __forceinline__ void tile_expired(uint64_t* bar, uint32_t parity, int* timeout) {
+  if (threadIdx.x == 0) atomicExch(timeout, 1);
+  mbar_wait_bounded(smem_addr(bar), parity);
+  __syncthreads();
+}
+
+// The entries of one row (up to W) in registers, and its product with the
+// values in shared memory at `u`, summed in stored order.  Entries beyond the
+// slice's width are zeros at offset 0 (their products leave the sum as it is),
+// so the common widths run without a test per entry: a test, its branch and
+// their waits cost more than the multiply-add.
+// A0: entries multiplied whatever the width; the rest in groups of two.
+template <class T, class V, int W>
+struct TileRow {
+  uint32_t c[(W + 1) / 2];
+  T v[W];
+  __device__ __forceinline__ void load(const uint32_t* words, const T* val, const TileSlice& h, int lane) {
+#pragma unroll
+    for (int e = 0; e < (W + 1) / 2; ++e) c[e] = 2 * e < h.w ? words[(h.words + e) * 32 + lane] : 0u;
+#pragma unroll
+    for (int e = 0; e < W; ++e) v[e] = e < h.w ? val[(h.vals + e) * 32 + lane] : (T)0;
+  }
+  __device__ __forceinline__ T term(const char* u, int e, T acc) const {
+    return acc + v[e] * *reinterpret_cast<const T*>(u + ((e & 1) ? c[e / 2] >> 16 : c[e / 2] & 0xffffu));
+  }
+};
+template <class T, int W>
+struct TileRow<T, bf16v, W> {
+  uint32_t c[W];
+  __device__ __forceinline__ void load(const uint32_t* words, const T*, const TileSlice& h, int lane) {
+#pragma unroll
+    for (int e = 0; e < W; ++e) c[e] = e < h.w ? words[(h.words + e) * 32 + lane] : 0u;
+  }
+  __device__ __forceinline__ T term(const char* u, int e, T acc) const {
+    return acc + (T)__uint_as_float(c[e] & 0xffff0000u) * *reinterpret_cast<const T*>(u + (c[e] & 0xffffu));
+  }
+};
+template <class T, class V, int W>
+__device__ __forceinline__ T tile_dot(const TileRow<T, V, W>& row, const char* u, int w) {
+  constexpr int A0 = W <= 8 ? 6 : 8;
   T acc = 0;
-  int e = 0;
-  for (; e + 4 <= w; e += 4) {
-    const int q = b + (e << 5) + lane;
-    const int c0 = col[q], c1 = col[q + 32], c2 = col[q + 64], c3 = col[q + 96];
-    const T v0 = (T)val_of(val[q]), v1 = (T)val_of(val[q + 32]), v2 = (T)val_of(val[q + 64]),
-            v3 = (T)val_of(val[q + 96]);
-    const T x0 = Ul[c0], x1 = Ul[c1], x2 = Ul[c2], x3 = Ul[c3];
-    acc += v0 * x0;
-    acc += v1 * x1;
-    acc += v2 * x2;
-    acc += v3 * x3;
-  }
-  for (; e < w; ++e) {
-    const int q = b + (e << 5) + lane;
-    acc += (T)val_of(val[q]) * Ul[col[q]];
-  }
+#pragma unroll
+  for (int e = 0; e < A0; ++e) acc = row.term(u, e, acc);
+#pragma unroll
+  for (int e = A0; e < W; e += 2)
+    if (w > e) {
+      acc = row.term(u, e, acc);
+      acc = row.term(u, e + 1, acc);
+    }
   return acc;
 }
 
-// the staged block of a tile (TileLayout) and, after it, U (local rows and
-// outside values) and F
-template <class T, class V>
-struct TileSmem {
-  const int32_t* soff;
-  const uint16_t* col;
-  const V* val;
-  const T* dinv;
-  const int32_t* lsm;
-  const int32_t* laux;
-  const int32_t* ext;
-  T *Ul, *Fl;
+// the thread's rows of a tile, from the staged block
+template <class T, class V, int S, int W>
+struct TileRows {
+  int wc[S];        // slice: width | colour class << 8 (-1 << 8: empty)
+  TileRow<T, V, W> row[S];
+  T di[S];
+  int32_t g[S], ax[S];  // SM row (own k, halo -2 - k, padding -1), aux ID
+  __device__ __forceinline__ void load(const unsigned char* blob, const TileHead& h, const TileLayout& lay) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const TileSlice* hdr = reinterpret_cast<const TileSlice*>(blob);
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      wc[s] = -256;
+      g[s] = -1;
+      if (s < h.slots) {
+        const TileSlice sl = hdr[s * TILE_WARPS + warp];
+        wc[s] = sl.w | (int)sl.colour << 8;
+        row[s].load(reinterpret_cast<const uint32_t*>(blob + lay.words), reinterpret_cast<const T*>(blob + lay.val), sl,
+                    lane);
+        di[s] = reinterpret_cast<const T*>(blob + lay.dinv)[s * TILE_THREADS + tid];
+        g[s] = reinterpret_cast<const int32_t*>(blob + lay.lsm)[s * TILE_THREADS + tid];
+        ax[s] = reinterpret_cast<const int32_t*>(blob + lay.laux)[s * TILE_THREADS + tid];
+      }
+    }
+  }
+  // one colour phase: u += (f - A u) / a_ii on the thread's rows of class c
+  __device__ __forceinline__ void phase(int c, T* Ul, const T (&f)[S], T (&u)[S]) const {
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (wc[s] >> 8 == c) {
+        const T acc = tile_dot(row[s], reinterpret_cast<const char*>(Ul), wc[s] & 255);
+        u[s] += (f[s] - acc) * di[s];
+        Ul[s * TILE_THREADS + threadIdx.x] = u[s];
+      }
+  }
 };
 
-template <class T, class V>
-__device__ __forceinline__ TileSmem<T, V> tile_smem(unsigned char* raw, int64_t maxblob, int maxloc, int maxext,
-                                                    int nl, int nx) {
-  TileSmem<T, V> t;
-  t.soff = reinterpret_cast<const int32_t*>(raw);
-  const TileLayout lay = tile_layout(nl, t.soff[nl >> 5], nx, (int64_t)sizeof(T), (int64_t)sizeof(V));
-  t.col = reinterpret_cast<const uint16_t*>(raw + lay.col);
-  t.val = reinterpret_cast<const V*>(raw + lay.val);
-  t.dinv = reinterpret_cast<const T*>(raw + lay.dinv);
-  t.lsm = reinterpret_cast<const int32_t*>(raw + lay.lsm);
-  t.laux = reinterpret_cast<const int32_t*>(raw + lay.laux);
-  t.ext = reinterpret_cast<const int32_t*>(raw + lay.ext);
-  t.Ul = reinterpret_cast<T*>(raw + maxblob);
-  t.Fl = t.Ul + maxloc + maxext;
-  return t;
+// blocks per SM the kernels are compiled for: the most whose registers hold the
+// rows (a few spilled words cost less than a fourth block gives, BF16: level of
+// 3.46 M rows 115 us with three blocks, 80 us with four)
+template <class T, class V, int S, int W>
+constexpr int tile_min_blocks() {
+  if (sizeof(T) == 8) return W > 8 ? (S > 2 ? 1 : 2) : S > 2 ? 2 : 3;
+  return W > 8 ? 2 : S == 4 && !std::is_same<V, bf16v>::value ? 3 : 4;
 }
 
 // pre-sweeps: us (the level's own correction, SM order) starts at 0; the
-// first sweep saves F on the tile's own rows in fs.  The block is copied in
-// while the previous kernel finishes.
-template <class T, class V>
-__global__ void __launch_bounds__(TILE_TPB) k_tile_down(const int64_t* __restrict__ loc_off,
-                                                        const int64_t* __restrict__ blob_off,
-                                                        const unsigned char* __restrict__ blob,
-                                                        const int32_t* __restrict__ phase, int ncol, int64_t maxblob,
-                                                        int maxloc, const T* __restrict__ F, T* __restrict__ fs,
-                                                        T* __restrict__ us, int nu, int* timeout, int inject) {
+// first sweep saves F on the tile's own rows in fs
+template <class T, class V, int S, int W>
+__global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W>())
+    k_tile_down(TileView<T> t, int ncol, int64_t vals, const T* __restrict__ F, T* __restrict__ fs,
+                T* __restrict__ us, int nu, int* timeout, int inject) {
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ __align__(8) uint64_t bar;
-  const int64_t base = loc_off[blockIdx.x];
-  const int nl = (int)(loc_off[blockIdx.x + 1] - base);
-  const int64_t b0 = blob_off[blockIdx.x];
-  const uint32_t bytes = (uint32_t)(blob_off[blockIdx.x + 1] - b0);
-  const int32_t* ph = phase + (int64_t)blockIdx.x * (ncol + 1);
-  tile_stage(smraw, blob + b0, bytes, &bar);
+  T* Ul = reinterpret_cast<T*>(smraw);
+  unsigned char* blob = smraw + vals;
+  const int tid = threadIdx.x;
+  int64_t tile = blockIdx.x;
+  TileHead h = t.head[tile];
+  if (tid == 0) {
+    tile_bar_init(&bar);
+    tile_fetch(blob, t.blob, h, &bar);
+  }
+  __syncthreads();  // the barrier is initialised before any thread polls it
+  // the first tile's rows are in registers before the wait on the previous kernel
+  TileRows<T, V, S, W> R;
+  uint32_t parity = 0;
+  bool ok = tile_arrived(&bar, parity, inject);
+  if (ok) R.load(blob, h, tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T)));
   pdl_wait();
-  if (tile_staged(&bar, timeout, inject)) {
-    TileSmem<T, V> t = tile_smem<T, V>(smraw, maxblob, maxloc, 0, nl, 0);
-    for (int k = threadIdx.x; k < nl; k += blockDim.x) {
-      const int32_t g = t.lsm[k];
-      T f = 0;
-      if (g != -1) {
-        f = F[t.laux[k]];
-        if (g >= 0) fs[g] = f;
-      }
-      t.Fl[k] = f;
-      t.Ul[k] = 0;
+  while (ok) {
+    T f[S], u[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      f[s] = R.g[s] != -1 ? F[R.ax[s]] : (T)0;
+      u[s] = 0;
+      Ul[s * TILE_THREADS + tid] = 0;
     }
-    __syncthreads();
+    const uint32_t mask = h.cmask;
+    tile += gridDim.x;
+    const bool more = tile < t.ntiles;
+    if (more) h = t.head[tile];
+    __syncthreads();  // values in place, the block read by all
+    if (tid == 0 && more) tile_fetch(blob, t.blob, h, &bar);
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (R.g[s] >= 0) fs[R.g[s]] = f[s];
     for (int sw = 0; sw < nu; ++sw)
       for (int c = 0; c < ncol; ++c) {
-        for (int k = ph[c] + threadIdx.x; k < ph[c + 1]; k += blockDim.x) {
-          const T acc = tile_row_dot<T, V>(k, t.soff, t.col, t.val, t.Ul);
-          t.Ul[k] += (t.Fl[k] - acc) * t.dinv[k];
-        }
+        if (!((mask >> min(c, 31)) & 1u)) continue;  // no row of this class in the tile
+        R.phase(c, Ul, f, u);
         __syncthreads();
       }
-    for (int k = threadIdx.x; k < nl; k += blockDim.x) {
-      const int32_t g = t.lsm[k];
-      if (g >= 0) us[g] = t.Ul[k];
-    }
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (R.g[s] >= 0) us[R.g[s]] = u[s];
+    if (!more) return;
+    parity ^= 1;
+    ok = tile_arrived(&bar, parity, inject);
+    if (ok) R.load(blob, h, tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T)));
   }
+  tile_expired(&bar, parity, timeout);
 }
 
 // start of the up path of a tiled level: the prolongation of the coarse
 // correction (I_l: new nodes take the mean of their parents) plus the level's
 // saved correction, and the saved rhs, written for every SM row to each place
 // the row holds in the post-sweep tiles (own and halo copies; TileSweeps::
-// pos).  U itself is not written, so the tiles can copy their start values in
+// pos).  U itself is not written, so the tiles can read their start values
 // while other tiles write their results to U.
 template <class T>
 __global__ void k_up_init(int64_t nsm, const int32_t* __restrict__ rows, const int32_t* __restrict__ par0,
@@ -489,65 +543,66 @@ __global__ void k_up_init(int64_t nsm, const int32_t* __restrict__ rows, const i
 }
 
 // post-sweeps (backward colour order) from the start values and saved rhs
-// that k_up_init wrote in tile order: both arrive by bulk copy after the
-// wait on the previous kernel, the tile's block before it; the columns
+// that k_up_init wrote in tile order (`per` local rows a tile); the columns
 // outside N~_l (the tile's outside values) are read from U once; the tile's
 // own rows are written to U
-template <class T, class V>
-__global__ void __launch_bounds__(TILE_TPB) k_tile_up(const int64_t* __restrict__ loc_off,
-                                                      const int64_t* __restrict__ blob_off,
-                                                      const unsigned char* __restrict__ blob,
-                                                      const int64_t* __restrict__ ext_off,
-                                                      const int32_t* __restrict__ phase, int ncol, int64_t maxblob,
-                                                      int maxloc, int maxext, const T* __restrict__ ust,
-                                                      const T* __restrict__ fsl, T* U, int nu, int* timeout,
-                                                      int inject) {
+template <class T, class V, int S, int W>
+__global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W>())
+    k_tile_up(TileView<T> t, int ncol, int64_t vals, const T* __restrict__ ust, const T* __restrict__ fsl, T* U,
+              int nu, int* timeout, int inject) {
   extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ __align__(8) uint64_t bar, bar2;
-  const int64_t base = loc_off[blockIdx.x];
-  const int nl = (int)(loc_off[blockIdx.x + 1] - base);
-  const int64_t b0 = blob_off[blockIdx.x];
-  const uint32_t bytes = (uint32_t)(blob_off[blockIdx.x + 1] - b0);
-  const int nx = (int)(ext_off[blockIdx.x + 1] - ext_off[blockIdx.x]);
-  const int32_t* ph = phase + (int64_t)blockIdx.x * (ncol + 1);
-  T* Ul = reinterpret_cast<T*>(smraw + maxblob);
-  T* Fl = Ul + maxloc + maxext;
-  if (threadIdx.x == 0) {
-    // initialised before tile_stage's fence.mbarrier_init, which covers it
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar2)) : "memory");
+  __shared__ __align__(8) uint64_t bar;
+  T* Ul = reinterpret_cast<T*>(smraw);
+  unsigned char* blob = smraw + vals;
+  const int tid = threadIdx.x;
+  int64_t tile = blockIdx.x;
+  TileHead h = t.head[tile];
+  if (tid == 0) {
+    tile_bar_init(&bar);
+    tile_fetch(blob, t.blob, h, &bar);
   }
-  tile_stage(smraw, blob + b0, bytes, &bar);
+  __syncthreads();  // the barrier is initialised before any thread polls it
+  // the first tile's rows are in registers before the wait on the previous kernel
+  TileRows<T, V, S, W> R;
+  TileLayout lay = tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T));
+  uint32_t parity = 0;
+  bool ok = tile_arrived(&bar, parity, inject);
+  if (ok) R.load(blob, h, lay);
   pdl_wait();
-  if (threadIdx.x == 0) {
-    const uint32_t b2 = smem_addr(&bar2), vb = (uint32_t)((int64_t)nl * sizeof(T));
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b2), "r"(2 * vb) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(Ul)),
-                 "l"(ust + base), "r"(vb), "r"(b2)
-                 : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(Fl)),
-                 "l"(fsl + base), "r"(vb), "r"(b2)
-                 : "memory");
-  }
-  const bool ok1 = tile_staged(&bar, timeout, inject);
-  // the outside values, once the block (which holds their IDs) is in place
-  TileSmem<T, V> t = tile_smem<T, V>(smraw, maxblob, maxloc, maxext, nl, nx);
-  if (ok1)
-    for (int e = threadIdx.x; e < nx; e += blockDim.x) t.Ul[nl + e] = U[t.ext[e]];
-  const bool ok2 = tile_staged(&bar2, timeout, inject || !ok1);
-  if (ok1 && ok2) {
+  while (ok) {
+    const int64_t base = tile * (S * TILE_THREADS) + tid;
+    T f[S], u[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      u[s] = ust[base + s * TILE_THREADS];
+      f[s] = fsl[base + s * TILE_THREADS];
+    }
+    const int32_t* ext = reinterpret_cast<const int32_t*>(blob + lay.ext);
+    for (int e = tid; e < h.nx; e += TILE_THREADS) Ul[S * TILE_THREADS + e] = U[ext[e]];
+#pragma unroll
+    for (int s = 0; s < S; ++s) Ul[s * TILE_THREADS + tid] = u[s];
+    const uint32_t mask = h.cmask;
+    tile += gridDim.x;
+    const bool more = tile < t.ntiles;
+    if (more) h = t.head[tile];
+    __syncthreads();  // values in place, the block read by all
+    if (tid == 0 && more) tile_fetch(blob, t.blob, h, &bar);
     for (int sw = 0; sw < nu; ++sw)
       for (int c = ncol - 1; c >= 0; --c) {
-        for (int k = ph[c] + threadIdx.x; k < ph[c + 1]; k += blockDim.x) {
-          const T acc = tile_row_dot<T, V>(k, t.soff, t.col, t.val, t.Ul);
-          t.Ul[k] += (t.Fl[k] - acc) * t.dinv[k];
-        }
+        if (!((mask >> min(c, 31)) & 1u)) continue;
+        R.phase(c, Ul, f, u);
         __syncthreads();
       }
-    for (int k = threadIdx.x; k < nl; k += blockDim.x)
-      if (t.lsm[k] >= 0) U[t.laux[k]] = t.Ul[k];
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (R.g[s] >= 0) U[R.ax[s]] = u[s];
+    if (!more) return;
+    lay = tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T));
+    parity ^= 1;
+    ok = tile_arrived(&bar, parity, inject);
+    if (ok) R.load(blob, h, lay);
   }
+  tile_expired(&bar, parity, timeout);
 }
 
 // ------------------------------------------- near-boundary solve (Alg. 3)
@@ -1080,6 +1135,21 @@ int64_t small_bytes(const Prec<T>& P, int first, int count, int nu, bool down) {
   return by;
 }
 
+// f(slots, width) with the tile kernel's compile-time sizes for a level's tiles
+template <class T, class V, class F>
+void tile_dispatch(const TileSweeps<T>& Tl, F f) {
+  auto by_width = [&](auto sl) {
+    if (Tl.width <= 8)
+      f(sl, std::integral_constant<int, 8>{});
+    else
+      f(sl, std::integral_constant<int, TILE_MAXW>{});
+  };
+  if (Tl.slots == 1) by_width(std::integral_constant<int, 1>{});
+  if (Tl.slots == 2) by_width(std::integral_constant<int, 2>{});
+  if (Tl.slots == 3) by_width(std::integral_constant<int, 3>{});
+  if (Tl.slots == 4) by_width(std::integral_constant<int, 4>{});
+}
+
 // the slot's timeout flag (PcgScalars::timeout, device memory)
 int* timeout_flag(Slot& S) {
   return reinterpret_cast<int*>(reinterpret_cast<char*>(S.scal.p) + offsetof(PcgScalars, timeout));
@@ -1111,10 +1181,13 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
       const TileSweeps<T>& Tl = L.tdown;
       const int64_t by = Tl.nnz_real * (sv + 2) + (Tl.interior + Tl.halo) * (8 + 2 * sz) + Tl.interior * (4 + sz);
       LAUNCH(ASMG_PROF_AUX_GS, by,
-             launch_smem(h.prm.use_pdl, k_tile_down<T, V>, Tl.ntiles, Tl.tpb, Tl.smem(), s, Tl.loc_off.p,
-                         Tl.blob_off.p, (const unsigned char*)Tl.blob.p, Tl.phase.p, L.ncolours, Tl.maxblob,
-                         Tl.maxloc, (const T*)SP.F.p, SP.fs[li].p, SP.us[li].p, npre, timeout_flag(S),
-                         h.prm.inject_timeout));
+             tile_dispatch<T, V>(Tl, [&](auto sl, auto w) {
+               constexpr int SL = decltype(sl)::value, W = decltype(w)::value;
+               launch_smem(h.prm.use_pdl, k_tile_down<T, V, SL, W>,
+                           std::min<int64_t>(Tl.ntiles, NSM * tile_min_blocks<T, V, SL, W>()), TILE_THREADS, Tl.smem(), s,
+                           Tl.view(), L.ncolours, Tl.smem_values(), (const T*)SP.F.p, SP.fs[li].p, SP.us[li].p, npre,
+                           timeout_flag(S), h.prm.inject_timeout);
+             }));
       ++launches;
     }
     // pre-sweeps on us (SM order); the first also saves F on N~_l for the
@@ -1170,10 +1243,13 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
                     (const T*)SP.fs[li].p, SP.ust[li].p, SP.fsl[li].p));
       const int64_t by = Tl.nnz_real * (sv + 2) + (Tl.interior + Tl.halo) * (8 + 3 * sz) + Tl.interior * (4 + sz);
       LAUNCH(ASMG_PROF_AUX_GS, by,
-             launch_smem(h.prm.use_pdl, k_tile_up<T, V>, Tl.ntiles, Tl.tpb, Tl.smem(), s, Tl.loc_off.p, Tl.blob_off.p,
-                         (const unsigned char*)Tl.blob.p, Tl.ext_off.p, Tl.phase.p, L.ncolours, Tl.maxblob,
-                         Tl.maxloc, Tl.maxext, (const T*)SP.ust[li].p, (const T*)SP.fsl[li].p, SP.U.p, npost,
-                         timeout_flag(S), h.prm.inject_timeout));
+             tile_dispatch<T, V>(Tl, [&](auto sl, auto w) {
+               constexpr int SL = decltype(sl)::value, W = decltype(w)::value;
+               launch_smem(h.prm.use_pdl, k_tile_up<T, V, SL, W>,
+                           std::min<int64_t>(Tl.ntiles, NSM * tile_min_blocks<T, V, SL, W>()), TILE_THREADS, Tl.smem(), s,
+                           Tl.view(), L.ncolours, Tl.smem_values(), (const T*)SP.ust[li].p, (const T*)SP.fsl[li].p,
+                           SP.U.p, npost, timeout_flag(S), h.prm.inject_timeout);
+             }));
       launches += 2;
       continue;
     }
@@ -1510,15 +1586,23 @@ void setup_small(Prec<T>& P) {
   P.n_bottom = nb;
   const int smem = (int)small_smem<T>();
   // the attribute belongs to the kernel, not to this handle: every handle sets
-  // the same bound, for tiles the largest a tile may use
+  // the same bound
   auto attrs = [&](auto vtag) {
     using V = decltype(vtag);
     ASMG_CUDA(cudaFuncSetAttribute(k_small_down<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     ASMG_CUDA(cudaFuncSetAttribute(k_small_up<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ASMG_CUDA(
-        cudaFuncSetAttribute(k_tile_down<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_LIMIT));
-    ASMG_CUDA(
-        cudaFuncSetAttribute(k_tile_up<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_LIMIT));
+    for (int slots = 1; slots <= TILE_SLOTS_MAX; ++slots)
+      for (int width : {8, TILE_MAXW}) {
+        TileSweeps<T> Tl;
+        Tl.slots = slots;
+        Tl.width = width;
+        tile_dispatch<T, V>(Tl, [&](auto sl, auto w) {
+          ASMG_CUDA(cudaFuncSetAttribute(k_tile_down<T, V, decltype(sl)::value, decltype(w)::value>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX));
+          ASMG_CUDA(cudaFuncSetAttribute(k_tile_up<T, V, decltype(sl)::value, decltype(w)::value>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX));
+        });
+      }
   };
   attrs(T{});
   if constexpr (std::is_same<T, float>::value) attrs(bf16v{});
