@@ -68,6 +68,7 @@ int64_t pad32(int64_t n) { return (n + 31) / 32 * 32; }
 constexpr int TILE_ROWS_2COL = 256;
 constexpr double TILE_OWN_DOWN = 0.5, TILE_OWN_UP = 0.375;
 constexpr double TILE_MAX_HALO = 1.5;
+constexpr int64_t TILE_MIN_ROWS = 64;  // smoothing rows of a tiled level (below, the fused runs hold every level)
 
 // f(begin, end) over contiguous ranges of [0, n) on host threads
 template <class F>
@@ -118,14 +119,15 @@ HostCSR select_rows(const HostCSR& A, const std::vector<int64_t>& sel, const std
   return B;
 }
 
-// Shared-memory form of a small level: local numbering (smoothing nodes in
-// colour order first, then the other rows of E_l), 16-bit local columns.
+// The form of a small level that the fused runs take (small_run.h): local
+// numbering (smoothing nodes in colour order first, then the other rows of
+// E_l), 16-bit local columns.
 template <class T>
 void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<uint8_t>& inset,
                  const std::vector<int64_t>& sel, const std::vector<int64_t>& rsel, const std::vector<T>& dinv_pad,
                  const std::vector<int32_t>& pid, const std::vector<int32_t>& pptr, const std::vector<int32_t>& child,
-                 bool bf16, AuxLevelDev<T>& D, cudaStream_t s) {
-  SmallLevelDev<T>& S = D.small;
+                 AuxLevelDev<T>& D) {
+  SmallLevel<T>& S = D.small;
   S.ok = false;
   std::vector<int32_t> gid;
   std::vector<T> dinv;
@@ -142,7 +144,7 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
   for (int64_t r : rsel)
     if (r >= 0 && !inset[r]) gid.push_back((int32_t)r);
   const int mE = (int)gid.size();
-  if (mE > SMALL_LMAX || D.ncolours > SMALL_MAXC) return;
+  if (mE > small_lmax<T>() || D.ncolours > SMALL_MAXC) return;
   std::unordered_map<int32_t, int32_t> loc;
   loc.reserve(mE * 2);
   for (int k = 0; k < mE; ++k) loc[gid[k]] = k;
@@ -196,36 +198,30 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
     }
     rp_ptr.push_back((int32_t)rp_child.size());
   }
+  auto longest = [](const std::vector<int32_t>& ptr) {
+    int32_t w = 0;
+    for (size_t k = 1; k < ptr.size(); ++k) w = std::max(w, ptr[k] - ptr[k - 1]);
+    return w;
+  };
+  if (longest(sm_ptr) > SMALL_MAXW || longest(rs_ptr) > SMALL_MAXW) return;
   S.mS = mS;
   S.mE = mE;
   S.ncol = D.ncolours;
-  S.nnew = (int)nn_id.size();
-  S.npar = (int)rp_id.size();
-  S.nnz_sm = (int64_t)sm_col.size();
-  S.nnz_rs = (int64_t)rs_col.size();
-  S.nchild = (int64_t)rp_child.size();
-  S.cs = cs;
-  S.gid.upload(gid, s);
-  S.sm_ptr.upload(sm_ptr, s);
-  S.sm_col.upload(sm_col, s);
-  S.sm_val.upload(sm_val, s);
-  S.dinv.upload(dinv, s);
-  S.rs_ptr.upload(rs_ptr, s);
-  S.rs_col.upload(rs_col, s);
-  S.rs_val.upload(rs_val, s);
-  if (bf16) {
-    std::vector<bf16v> a(sm_val.size()), b(rs_val.size());
-    for (size_t k = 0; k < a.size(); ++k) a[k].bits = bf16_bits((float)sm_val[k]);
-    for (size_t k = 0; k < b.size(); ++k) b[k].bits = bf16_bits((float)rs_val[k]);
-    S.sm_v16.upload(a, s);
-    S.rs_v16.upload(b, s);
-  }
-  S.nn_id.upload(nn_id, s);
-  S.nn_p0.upload(nn_p0, s);
-  S.nn_p1.upload(nn_p1, s);
-  S.rp_id.upload(rp_id, s);
-  S.rp_ptr.upload(rp_ptr, s);
-  S.rp_child.upload(rp_child, s);
+  S.cs = std::move(cs);
+  S.gid = std::move(gid);
+  S.sm_ptr = std::move(sm_ptr);
+  S.sm_col = std::move(sm_col);
+  S.sm_val = std::move(sm_val);
+  S.dinv = std::move(dinv);
+  S.rs_ptr = std::move(rs_ptr);
+  S.rs_col = std::move(rs_col);
+  S.rs_val = std::move(rs_val);
+  S.nn_id = std::move(nn_id);
+  S.nn_p0 = std::move(nn_p0);
+  S.nn_p1 = std::move(nn_p1);
+  S.rp_id = std::move(rp_id);
+  S.rp_ptr = std::move(rp_ptr);
+  S.rp_child = std::move(rp_child);
   S.ok = true;
 }
 
@@ -662,9 +658,8 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
   D.sm_dinv.upload(dinv, s);
   // temporal blocking of the level's sweeps (TileSweeps), with the default own
   // rows per tile and a halo of at most TILE_MAX_HALO times the own rows, or the
-  // requested rows and any halo; the level needs at least two tiles and every
-  // new node must be a smoothing row (k_up_init prolongs through the smoothing
-  // rows)
+  // requested rows and any halo; every new node must be a smoothing row
+  // (k_up_init prolongs through the smoothing rows)
   D.tiled = false;
   if (prm.tile_rows >= 0 && prm.nu_post >= 1) {
     bool ok = true;
@@ -674,7 +669,7 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
     const int cap = TILE_SLOTS_MAX * TILE_THREADS;
     const int rd = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN_DOWN);
     const int ru = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN_UP);
-    if (ok && D.nsm_real >= 2 * (int64_t)std::max(rd, ru)) {
+    if (ok && D.nsm_real >= TILE_MIN_ROWS) {
       // the two directions are built at the same time, each on half the host threads
       TileSweeps<T> td, tu;
       const unsigned half = std::max(1u, std::thread::hardware_concurrency() / 2);
@@ -760,7 +755,7 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
   build_nb_dev<T>(L, Arows, pos, D, s);
   // a level with a near-boundary solve keeps its own launches (the solve sits
   // between the coarse correction and the post-smoothing)
-  if (D.nb.m == 0) build_small<T>(L, Arows, inset, sel, rsel, dinv, pid, pptr, child, bf16, D, s);
+  if (D.nb.m == 0) build_small<T>(L, Arows, inset, sel, rsel, dinv, pid, pptr, child, D);
   else D.small.ok = false;
 }
 

@@ -42,7 +42,8 @@ struct Prec {
   DBuf<T> dinv_f;
   Sell<T> P, PT;               // Scott-Zhang transfer and its transpose
   std::vector<AuxLevelDev<T>> lev;  // levels c+1..J (index 0 = c+1)
-  int n_deep = 0, n_bottom = 0;  // fused small-level runs (top of the hierarchy, bottom)
+  SmallRun<T> deep, bot;         // fused small-level runs (top of the hierarchy, bottom)
+  SmallRun<T> deep_k, bot_k;     // the same for KRHS interleaved columns
 };
 
 // Per-solve work state in precision T.
@@ -52,7 +53,7 @@ struct SlotPrec {
   std::vector<DBuf<T>> fs, us;      // per level: saved rhs / pre-smoothed values on N~_l
   std::vector<DBuf<double>> nbr, nbs;  // per level: near-boundary rhs / solution pools (mixed boundaries)
   std::vector<DBuf<T>> ust, fsl;    // per level with tiled post-sweeps: start values and saved rhs in tile order
-  DBuf<SmallDesc<T>> deep_desc, bot_desc;
+  DBuf<T> deep_fs, deep_us, bot_fs, bot_us;  // the same for the levels of the fused runs
 };
 
 // Everything one solve writes: several slots let independent right-hand
@@ -90,8 +91,7 @@ template <class T>
 struct MultiPrec {
   DBuf<T> uf, rho, F, U;                  // [rows][KRHS]
   std::vector<DBuf<T>> fs, us;            // per level [nsm][KRHS]
-  DBuf<SmallDesc<T>> deep_desc, bot_desc;
-  int n_deep = 0, n_bottom = 0;           // fused small-level runs for KRHS columns
+  DBuf<T> deep_fs, deep_us, bot_fs, bot_us;  // the same for the levels of the fused runs
 };
 
 struct MultiSlot {

@@ -252,47 +252,55 @@ HostCSR assemble_simplices(int dim, int64_t n, const double* dP, const int32_t* 
 std::vector<int32_t> jp_colour_gpu(const HostCSR& A, const std::vector<uint8_t>& inset,
                                    const std::vector<uint64_t>& prio_key, cudaStream_t s);
 
-// A level small enough to run inside one thread block with its rhs and
-// correction in shared memory (see k_small_down / k_small_up).  Local node
-// k < mS is the k-th smoothing node (colour order); mS <= k < mE are the other
-// nodes of the rows E_l.  Column indices are local (16 bit).
-constexpr int SMALL_LMAX = 8192;
-constexpr int SMALL_MAXC = 24;
+// A level small enough to run inside one thread block (small_run.h), in host
+// memory.  Local node k < mS is the k-th smoothing node (colour order); mS <= k
+// < mE are the other nodes of the rows E_l.  Columns, parents and children are
+// local nodes.
+// Most rows: one per thread; in FP64 half of that, as one SM's FP64 units (2 FMA
+// a cycle) bound a run (65^2 FP64 with its 992-row level fused 834 us per
+// solve, tiled 776 us; 331^2 mixed 1,626 and 1,632 us)
 template <class T>
-struct SmallDesc {
-  int mS, mE, ncol, nnew, npar;
-  int nnz_sm, nnz_rs, nchild;  // entries of the smoothing / residual rows, children of the restriction
-  int cs[SMALL_MAXC + 1];
-  const int32_t* gid;
-  const int32_t* sm_ptr;
-  const uint16_t* sm_col;
-  const T* sm_val;
-  const bf16v* sm_v16;  // the same values in BF16 (level_bf16), else null
-  const T* dinv;
-  const int32_t* rs_ptr;
-  const uint16_t* rs_col;
-  const T* rs_val;
-  const bf16v* rs_v16;
-  const uint16_t* nn_id;
-  const int32_t* nn_p0;
-  const int32_t* nn_p1;
-  const uint16_t* rp_id;
-  const int32_t* rp_ptr;
-  const uint16_t* rp_child;
-  T* fs;
-  T* us;
+constexpr int small_lmax() {
+  return sizeof(T) == 8 ? 512 : 1024;
+}
+constexpr int SMALL_MAXC = 24;
+constexpr int SMALL_MAXW = 16;                 // longest row
+constexpr int SMALL_NONE = 0xffff;             // no parent (Dirichlet)
+constexpr int64_t SMALL_SMEM_MAX = 200 * 1024; // shared memory of a run
+
+template <class T>
+struct SmallLevel {
+  bool ok = false;  // the level fits
+  int mS = 0, mE = 0, ncol = 0;
+  std::vector<int> cs;                        // colour class starts
+  std::vector<int32_t> gid;                   // aux IDs
+  std::vector<int32_t> sm_ptr, rs_ptr, rp_ptr, nn_p0, nn_p1;
+  std::vector<uint16_t> sm_col, rs_col, nn_id, rp_id, rp_child;
+  std::vector<T> sm_val, dinv, rs_val;
+};
+
+// one level of a run: sizes, and byte offsets within the run's block of its
+// union rows, diagonal inverses, ELL rows (mSp / mEp rows per column, widths
+// wsm / wrs), new nodes and restriction; sm0: its first row in the run's fs, us
+struct SmallHead {
+  int32_t mS, mE, ncol, nnew, npar, sm0, mSp, mEp, wsm, wrs;
+  int32_t cs[SMALL_MAXC + 1];
+  int32_t o_row, o_dinv, o_smc, o_smv, o_nn, o_rsc, o_rsv, o_rid, o_rptr, o_rch;
+};
+
+inline __host__ __device__ int64_t small_pad16(int64_t b) { return (b + 15) / 16 * 16; }
+
+struct SmallRunView {
+  const unsigned char* blob = nullptr;  // SmallHead [nlev], then the arrays; the first up_bytes serve the way up
+  int32_t bytes = 0, up_bytes = 0;
+  int32_t nlev = 0, nunion = 0, nsm = 0, o_gid = 0;
 };
 
 template <class T>
-struct SmallLevelDev {
-  bool ok = false;  // level fits the small-level kernels
-  int mS = 0, mE = 0, ncol = 0, nnew = 0, npar = 0;
-  int64_t nnz_sm = 0, nnz_rs = 0, nchild = 0;
-  std::vector<int> cs;
-  DBuf<int32_t> gid, sm_ptr, rs_ptr, nn_p0, nn_p1, rp_ptr;
-  DBuf<uint16_t> sm_col, rs_col, nn_id, rp_id, rp_child;
-  DBuf<T> sm_val, dinv, rs_val;
-  DBuf<bf16v> sm_v16, rs_v16;  // level_bf16: sm_val / rs_val in BF16
+struct SmallRun {
+  SmallRunView v;
+  int width = 0, threads = 0;
+  DBuf<unsigned char> blob;
 };
 
 // Temporal blocking of the sweeps of one auxiliary level (Algorithm 2's
@@ -433,7 +441,7 @@ struct AuxLevelDev {
   int64_t npar = 0, nchild = 0;
   DBuf<int32_t> rp_id;           // parents receiving restricted residuals
   DBuf<int32_t> rp_ptr, rp_child;
-  SmallLevelDev<T> small;        // shared-memory form, when the level is small
+  SmallLevel<T> small;           // shared-memory form, when the level is small
   // temporal blocking (tiled = 1): pre-sweeps in one launch (k_tile_down), and
   // after k_up_init, post-sweeps in one launch (k_tile_up)
   bool tiled = false;                // tiles built for both directions

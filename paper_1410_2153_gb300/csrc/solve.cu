@@ -28,6 +28,7 @@
 
 #include "handle.h"
 #include "kernels.h"
+#include "small_run.h"
 
 namespace asmg {
 
@@ -734,133 +735,6 @@ __global__ void __launch_bounds__(NB_TPB) k_nb_solve(int R, const int32_t* __res
   for (int64_t q = threadIdx.x; q < m; q += blockDim.x) U[aux[q]] += (T)sol[q];
 }
 
-// ---------------------------------------------------- small levels, fused
-// A run of small levels in one thread block.  Per level the rhs F and the
-// correction U of the rows E_l, and the row pointers of its smoothing and
-// residual rows, live in shared memory; colour phases are separated by
-// __syncthreads instead of kernel boundaries.  The steps are those of
-// k_gs_aux / k_resid_aux / k_restrict_aux (down) and k_prolong_aux /
-// k_addsaved_aux / k_gs_aux (up).
-constexpr int SMALL_TPB = 1024;
-constexpr int SMALL_B = 8;  // row entries loaded in one batch
-
-template <class T>
-constexpr size_t small_smem() {
-  return 2 * SMALL_LMAX * sizeof(T) + 2 * (SMALL_LMAX + 1) * sizeof(int32_t);
-}
-
-// acc - sum_p val[p] * x[col[p]] over p0 <= p < p1, the first SMALL_B
-// entries loaded together (ascending p, as a plain loop would add them)
-template <class T, class V>
-__device__ __forceinline__ T small_row(T acc, int p0, int p1, const V* __restrict__ val,
-                                       const uint16_t* __restrict__ col, const T* x) {
-  T v[SMALL_B];
-  uint16_t c[SMALL_B];
-#pragma unroll
-  for (int q = 0; q < SMALL_B; ++q)
-    if (p0 + q < p1) {
-      v[q] = (T)val_of(val[p0 + q]);
-      c[q] = col[p0 + q];
-    }
-#pragma unroll
-  for (int q = 0; q < SMALL_B; ++q)
-    if (p0 + q < p1) acc -= v[q] * x[c[q]];
-  for (int p = p0 + SMALL_B; p < p1; ++p) acc -= (T)val_of(val[p]) * x[col[p]];
-  return acc;
-}
-
-template <class T, class V>
-__global__ void __launch_bounds__(SMALL_TPB, 1)
-    k_small_down(const SmallDesc<T>* __restrict__ D, int nlev, T* F, int nu) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* Ul = reinterpret_cast<T*>(smraw);
-  T* Fl = Ul + SMALL_LMAX;
-  int32_t* Psm = reinterpret_cast<int32_t*>(Fl + SMALL_LMAX);
-  int32_t* Prs = Psm + SMALL_LMAX + 1;
-  if (nlev > 0) small_prefetch<T, V>(D, true);
-  pdl_wait();
-  for (int d = 0; d < nlev; ++d) {
-    const SmallDesc<T>& L = D[d];
-    const int mS = L.mS, mE = L.mE;
-    if (d + 1 < nlev) small_prefetch<T, V>(D + d + 1, true);
-    for (int k = threadIdx.x; k <= mE; k += blockDim.x) {
-      if (k < mE) {
-        const T f = F[L.gid[k]];
-        Fl[k] = f;
-        Ul[k] = 0;
-        if (k < mS) L.fs[k] = f;
-      }
-      if (k <= mS) Psm[k] = L.sm_ptr[k];
-      Prs[k] = L.rs_ptr[k];
-    }
-    __syncthreads();
-    for (int sw = 0; sw < nu; ++sw)
-      for (int c = 0; c < L.ncol; ++c) {
-        for (int k = L.cs[c] + threadIdx.x; k < L.cs[c + 1]; k += blockDim.x) {
-          const T acc = small_row(Fl[k], Psm[k], Psm[k + 1], sm_vals(L, (const V*)nullptr), L.sm_col, Ul);
-          Ul[k] += acc * L.dinv[k];
-        }
-        __syncthreads();
-      }
-    for (int k = threadIdx.x; k < mE; k += blockDim.x) Fl[k] = small_row(Fl[k], Prs[k], Prs[k + 1], rs_vals(L, (const V*)nullptr), L.rs_col, Ul);
-    __syncthreads();
-    for (int t = threadIdx.x; t < L.npar; t += blockDim.x) {
-      T acc = 0;
-      for (int p = L.rp_ptr[t]; p < L.rp_ptr[t + 1]; ++p) acc += Fl[L.rp_child[p]];
-      Fl[L.rp_id[t]] += (T)0.5 * acc;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < mE; k += blockDim.x) {
-      F[L.gid[k]] = Fl[k];
-      if (k < mS) L.us[k] = Ul[k];
-    }
-    __syncthreads();
-  }
-}
-
-template <class T, class V>
-__global__ void __launch_bounds__(SMALL_TPB, 1)
-    k_small_up(const SmallDesc<T>* __restrict__ D, int nlev, T* U, int nu) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* Ul = reinterpret_cast<T*>(smraw);
-  T* Fl = Ul + SMALL_LMAX;
-  int32_t* Psm = reinterpret_cast<int32_t*>(Fl + SMALL_LMAX);
-  if (nlev > 0) small_prefetch<T, V>(D + nlev - 1, false);
-  pdl_wait();
-  for (int d = nlev - 1; d >= 0; --d) {
-    const SmallDesc<T>& L = D[d];
-    const int mS = L.mS, mE = L.mE;
-    if (d > 0) small_prefetch<T, V>(D + d - 1, false);
-    for (int k = threadIdx.x; k < mE; k += blockDim.x) {
-      Ul[k] = U[L.gid[k]];
-      if (k < mS) Fl[k] = L.fs[k];
-      if (k <= mS) Psm[k] = L.sm_ptr[k];
-    }
-    if (mS == mE && threadIdx.x == 0) Psm[mS] = L.sm_ptr[mS];
-    __syncthreads();
-    for (int t = threadIdx.x; t < L.nnew; t += blockDim.x) {
-      const int32_t a = L.nn_p0[t], b = L.nn_p1[t];
-      T v = 0;
-      if (a >= 0) v += Ul[a];
-      if (b >= 0) v += Ul[b];
-      Ul[L.nn_id[t]] = (T)0.5 * v;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < mS; k += blockDim.x) Ul[k] += L.us[k];
-    __syncthreads();
-    for (int sw = 0; sw < nu; ++sw)
-      for (int c = L.ncol - 1; c >= 0; --c) {
-        for (int k = L.cs[c] + threadIdx.x; k < L.cs[c + 1]; k += blockDim.x) {
-          const T acc = small_row(Fl[k], Psm[k], Psm[k + 1], sm_vals(L, (const V*)nullptr), L.sm_col, Ul);
-          Ul[k] += acc * L.dinv[k];
-        }
-        __syncthreads();
-      }
-    for (int k = threadIdx.x; k < mS; k += blockDim.x) U[L.gid[k]] = Ul[k];
-    __syncthreads();
-  }
-}
-
 // ------------------------------------------------------------------ PCG
 __device__ __forceinline__ void set_cond(PcgScalars* sc, int cond, cudaGraphConditionalHandle hnd, int use_hnd) {
   sc->cond = cond;
@@ -1119,20 +993,12 @@ SlotPrec<double>& slotprec<double>(Slot& S) { return S.s64; }
 template <>
 SlotPrec<float>& slotprec<float>(Slot& S) { return S.s32; }
 
-template <class T, class V>
-int64_t small_bytes(const Prec<T>& P, int first, int count, int nu, bool down) {
-  const int64_t sz = sizeof(T), sv = sizeof(V);
-  int64_t by = 0;
-  for (int k = 0; k < count; ++k) {
-    const SmallLevelDev<T>& S = P.lev[first + k].small;
-    by += nu * (S.nnz_sm * (2 + sv) + (int64_t)S.mS * (4 + sz));
-    if (down)
-      by += (int64_t)S.mE * (4 + 2 * sz) + (int64_t)S.mS * 2 * sz + S.nnz_rs * (2 + sv) + (int64_t)S.mE * 4 +
-            (int64_t)S.npar * 10 + S.nchild * 2;
-    else
-      by += (int64_t)S.mE * (4 + sz) + (int64_t)S.mS * 3 * sz + (int64_t)S.nnew * 10;
-  }
-  return by;
+// compulsory bytes of a fused run: its block, the union's values and the
+// smoothing rows' saved values
+template <class T>
+int64_t small_bytes(const SmallRun<T>& R, bool down) {
+  const int64_t sz = sizeof(T);
+  return (down ? R.v.bytes : R.v.up_bytes) + 2 * sz * (R.v.nunion + R.v.nsm);
 }
 
 // f(slots, width) with the tile kernel's compile-time sizes for a level's tiles
@@ -1164,11 +1030,10 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
   const int64_t sz = sizeof(T), sv = sizeof(V);
   const int npre = h.prm.nu_pre, npost = h.prm.nu_post;
   const int nlev = (int)P.lev.size();
-  const int ndeep = P.n_deep, nbot = P.n_bottom;  // fused runs at the top and at the bottom
-  const size_t smem = small_smem<T>();
+  const int ndeep = P.deep.v.nlev, nbot = P.bot.v.nlev;  // fused runs at the top and at the bottom
   if (ndeep) {
-    LAUNCH(ASMG_PROF_AUX_SMALL, (small_bytes<T, V>(P, nlev - ndeep, ndeep, npre, true)),
-           launch_smem(h.prm.use_pdl, k_small_down<T, V>, 1, SMALL_TPB, smem, s, SP.deep_desc.p, ndeep, SP.F.p, npre));
+    LAUNCH(ASMG_PROF_AUX_SMALL, small_bytes(P.deep, true),
+           small::launch_down<T, V, 1>(h.prm.use_pdl, P.deep, SP.F.p, SP.deep_fs.p, SP.deep_us.p, npre, s));
     ++launches;
   }
   for (int li = nlev - 1 - ndeep; li >= nbot; --li) {
@@ -1215,8 +1080,8 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
   }
   g_prof_level = -1;
   if (nbot) {
-    LAUNCH(ASMG_PROF_AUX_SMALL, (small_bytes<T, V>(P, 0, nbot, npre, true)),
-           launch_smem(h.prm.use_pdl, k_small_down<T, V>, 1, SMALL_TPB, smem, s, SP.bot_desc.p, nbot, SP.F.p, npre));
+    LAUNCH(ASMG_PROF_AUX_SMALL, small_bytes(P.bot, true),
+           small::launch_down<T, V, 1>(h.prm.use_pdl, P.bot, SP.F.p, SP.bot_fs.p, SP.bot_us.p, npre, s));
     ++launches;
   }
   if (h.nc > 0) {
@@ -1225,8 +1090,8 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
     ++launches;
   }
   if (nbot) {
-    LAUNCH(ASMG_PROF_AUX_SMALL, (small_bytes<T, V>(P, 0, nbot, npost, false)),
-           launch_smem(h.prm.use_pdl, k_small_up<T, V>, 1, SMALL_TPB, smem, s, SP.bot_desc.p, nbot, SP.U.p, npost));
+    LAUNCH(ASMG_PROF_AUX_SMALL, small_bytes(P.bot, false),
+           small::launch_up<T, V, 1>(h.prm.use_pdl, P.bot, SP.U.p, SP.bot_fs.p, SP.bot_us.p, npost, s));
     ++launches;
   }
   for (int li = nbot; li <= nlev - 1 - ndeep; ++li) {
@@ -1286,8 +1151,8 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
   }
   g_prof_level = -1;
   if (ndeep) {
-    LAUNCH(ASMG_PROF_AUX_SMALL, (small_bytes<T, V>(P, nlev - ndeep, ndeep, npost, false)),
-           launch_smem(h.prm.use_pdl, k_small_up<T, V>, 1, SMALL_TPB, smem, s, SP.deep_desc.p, ndeep, SP.U.p, npost));
+    LAUNCH(ASMG_PROF_AUX_SMALL, small_bytes(P.deep, false),
+           small::launch_up<T, V, 1>(h.prm.use_pdl, P.deep, SP.U.p, SP.deep_fs.p, SP.deep_us.p, npost, s));
     ++launches;
   }
   return launches;
@@ -1571,26 +1436,17 @@ int profile_solve(asmg_s& h, double rtol, cudaStream_t s, double* out, double* o
   return its;
 }
 
-// The fused runs: the longest run of small levels from the finest level down
-// and from the coarsest V-cycle level up (a level is small when its rows E_l
-// fit SMALL_LMAX); their descriptors live in device memory.
+// The fused small-level runs, for one and for KRHS right-hand sides, and the
+// kernels' shared-memory limits.
 template <class T>
-void setup_small(Prec<T>& P) {
-  const int nlev = (int)P.lev.size();
-  int nd = 0;
-  while (nd < nlev && P.lev[nlev - 1 - nd].small.ok) ++nd;
-  int nb = 0;
-  if (nd < nlev)
-    while (nb < nlev - nd && P.lev[nb].small.ok) ++nb;
-  P.n_deep = nd;
-  P.n_bottom = nb;
-  const int smem = (int)small_smem<T>();
+void setup_small(Prec<T>& P, bool bf16, cudaStream_t s) {
+  small::build_runs(P, bf16, 1, P.deep, P.bot, s);
+  small::build_runs(P, bf16, KRHS, P.deep_k, P.bot_k, s);
   // the attribute belongs to the kernel, not to this handle: every handle sets
   // the same bound
   auto attrs = [&](auto vtag) {
     using V = decltype(vtag);
-    ASMG_CUDA(cudaFuncSetAttribute(k_small_down<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ASMG_CUDA(cudaFuncSetAttribute(k_small_up<T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    small::set_smem_limits<T, V, 1>();
     for (int slots = 1; slots <= TILE_SLOTS_MAX; ++slots)
       for (int width : {8, TILE_MAXW}) {
         TileSweeps<T> Tl;
@@ -1608,9 +1464,7 @@ void setup_small(Prec<T>& P) {
   if constexpr (std::is_same<T, float>::value) attrs(bf16v{});
 }
 
-// Work state of one solve in precision T: vectors, per-level saved values,
-// descriptors of the fused small-level runs (they point at this slot's
-// saved values).
+// Work state of one solve in precision T: vectors and per-level saved values.
 template <class T>
 void alloc_slot_prec(asmg_s& h, Prec<T>& P, SlotPrec<T>& SP, cudaStream_t s) {
   SP.uf.alloc(h.npad);
@@ -1660,44 +1514,8 @@ void alloc_slot_prec(asmg_s& h, Prec<T>& P, SlotPrec<T>& SP, cudaStream_t s) {
       SP.nbs[li].zero(s);
     }
   }
-  auto desc = [&](int li) {
-    AuxLevelDev<T>& L = P.lev[li];
-    SmallDesc<T> d;
-    SmallLevelDev<T>& M = L.small;
-    d.mS = M.mS;
-    d.mE = M.mE;
-    d.ncol = M.ncol;
-    d.nnew = M.nnew;
-    d.npar = M.npar;
-    d.nnz_sm = (int)M.nnz_sm;
-    d.nnz_rs = (int)M.nnz_rs;
-    d.nchild = (int)M.nchild;
-    for (int c = 0; c <= SMALL_MAXC; ++c) d.cs[c] = c <= M.ncol ? M.cs[c] : M.mS;
-    d.gid = M.gid.p;
-    d.sm_ptr = M.sm_ptr.p;
-    d.sm_col = M.sm_col.p;
-    d.sm_val = M.sm_val.p;
-    d.sm_v16 = M.sm_v16.p;
-    d.dinv = M.dinv.p;
-    d.rs_ptr = M.rs_ptr.p;
-    d.rs_col = M.rs_col.p;
-    d.rs_val = M.rs_val.p;
-    d.rs_v16 = M.rs_v16.p;
-    d.nn_id = M.nn_id.p;
-    d.nn_p0 = M.nn_p0.p;
-    d.nn_p1 = M.nn_p1.p;
-    d.rp_id = M.rp_id.p;
-    d.rp_ptr = M.rp_ptr.p;
-    d.rp_child = M.rp_child.p;
-    d.fs = SP.fs[li].p;
-    d.us = SP.us[li].p;
-    return d;
-  };
-  std::vector<SmallDesc<T>> deep, bot;
-  for (int k = 0; k < P.n_deep; ++k) deep.push_back(desc(nlev - 1 - k));  // finest first (down order)
-  for (int k = P.n_bottom - 1; k >= 0; --k) bot.push_back(desc(k));
-  SP.deep_desc.upload(deep, s);
-  SP.bot_desc.upload(bot, s);
+  for (DBuf<T>* v : {&SP.deep_fs, &SP.deep_us}) v->alloc(std::max(P.deep.v.nsm, 1));
+  for (DBuf<T>* v : {&SP.bot_fs, &SP.bot_us}) v->alloc(std::max(P.bot.v.nsm, 1));
 }
 
 // Schedule of the auxiliary levels (the autotuner, tile_rows = 0): each
@@ -1715,7 +1533,7 @@ void autotune_levels(asmg_s& h, cudaStream_t s) {
   Slot& S = *h.slots[0];
   const int nlev = (int)P.lev.size();
   std::vector<int> cand;
-  for (int li = P.n_bottom; li <= nlev - 1 - P.n_deep; ++li)
+  for (int li = P.bot.v.nlev; li <= nlev - 1 - P.deep.v.nlev; ++li)
     if (P.lev[li].tiled) cand.push_back(li);
   if (cand.empty()) return;
   cudaStream_t cs;
@@ -1811,7 +1629,7 @@ template <class T>
 void drop_unused_tiles(Prec<T>& P) {
   const int nlev = (int)P.lev.size();
   for (int li = 0; li < nlev; ++li)
-    if (li < P.n_bottom || li > nlev - 1 - P.n_deep) {
+    if (li < P.bot.v.nlev || li > nlev - 1 - P.deep.v.nlev) {
       P.lev[li].tiled = P.lev[li].tiled_down = P.lev[li].tiled_up = false;
       P.lev[li].tdown = TileSweeps<T>();
       P.lev[li].tup = TileSweeps<T>();
@@ -1820,10 +1638,10 @@ void drop_unused_tiles(Prec<T>& P) {
 
 void setup_solve(asmg_s& h, cudaStream_t s) {
   if (h.prm.precision == ASMG_MIXED) {
-    setup_small(h.p32);
+    setup_small(h.p32, h.prm.level_bf16 == 1, s);
     drop_unused_tiles(h.p32);
   } else {
-    setup_small(h.p64);
+    setup_small(h.p64, false, s);
     drop_unused_tiles(h.p64);
   }
   h.slots.clear();

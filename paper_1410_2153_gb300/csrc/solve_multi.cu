@@ -12,8 +12,8 @@
 // its own test (converged, iteration cap, breakdown): it then keeps alpha = 0,
 // so its x and r no longer change, and the loop runs while any column is
 // active.  The fused small-level kernels hold KRHS columns in shared memory,
-// so a run of small levels is shorter here (SMALL_LMAX / KRHS rows per level
-// in FP32); such a level's arithmetic then follows the per-level kernels.
+// so a run of small levels may be shorter here; the other levels' arithmetic
+// follows the per-level kernels.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -23,6 +23,7 @@
 
 #include "handle.h"
 #include "kernels.h"
+#include "small_run.h"
 
 namespace asmg {
 
@@ -394,193 +395,6 @@ __global__ void k_coarse_k(int64_t nc, const int32_t* __restrict__ cid, const do
   }
 }
 
-// ---------------------------------------------------- small levels, fused
-// As k_small_down / k_small_up of solve.cu with KRHS columns per row in
-// shared memory; the levels of a run have at most small_lmax_k<T>() rows.
-constexpr int SMALL_TPB_K = 1024;
-constexpr int SMALL_B_K = 8;
-
-template <class T>
-__host__ __device__ constexpr int small_lmax_k() {
-  return sizeof(T) == 4 ? 4096 : 2048;
-}
-
-template <class T>
-constexpr size_t small_smem_k() {
-  return 2 * (size_t)small_lmax_k<T>() * K * sizeof(T) + 2 * (size_t)(small_lmax_k<T>() + 1) * sizeof(int32_t);
-}
-
-// acc[j] - sum_p val[p] x[col[p]][j] over p0 <= p < p1 (the order of small_row)
-template <class T, class V>
-__device__ __forceinline__ void small_row_k(T (&acc)[K], int p0, int p1, const V* __restrict__ val,
-                                            const uint16_t* __restrict__ col, const T* x) {
-  T v[SMALL_B_K];
-  uint16_t c[SMALL_B_K];
-#pragma unroll
-  for (int q = 0; q < SMALL_B_K; ++q)
-    if (p0 + q < p1) {
-      v[q] = (T)val_of(val[p0 + q]);
-      c[q] = col[p0 + q];
-    }
-#pragma unroll
-  for (int q = 0; q < SMALL_B_K; ++q)
-    if (p0 + q < p1) {
-#pragma unroll
-      for (int j = 0; j < K; ++j) acc[j] -= v[q] * x[(int)c[q] * K + j];
-    }
-  for (int p = p0 + SMALL_B_K; p < p1; ++p) {
-    const T a = (T)val_of(val[p]);
-    const int cc = col[p];
-#pragma unroll
-    for (int j = 0; j < K; ++j) acc[j] -= a * x[cc * K + j];
-  }
-}
-
-template <class T, class V>
-__global__ void __launch_bounds__(SMALL_TPB_K, 1)
-    k_small_down_k(const SmallDesc<T>* __restrict__ D, int nlev, T* F, int nu) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int LM = small_lmax_k<T>();
-  T* Ul = reinterpret_cast<T*>(smraw);
-  T* Fl = Ul + LM * K;
-  int32_t* Psm = reinterpret_cast<int32_t*>(Fl + LM * K);
-  int32_t* Prs = Psm + LM + 1;
-  if (nlev > 0) small_prefetch<T, V>(D, true);
-  pdl_wait();
-  for (int d = 0; d < nlev; ++d) {
-    const SmallDesc<T>& L = D[d];
-    const int mS = L.mS, mE = L.mE;
-    if (d + 1 < nlev) small_prefetch<T, V>(D + d + 1, true);
-    for (int k = threadIdx.x; k <= mE; k += blockDim.x) {
-      if (k < mE) {
-        const VK<T> f = ldk<T>(F + (int64_t)L.gid[k] * K);
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-          Fl[k * K + j] = f.v[j];
-          Ul[k * K + j] = 0;
-        }
-        if (k < mS) stk<T>(L.fs + (int64_t)k * K, f);
-      }
-      if (k <= mS) Psm[k] = L.sm_ptr[k];
-      Prs[k] = L.rs_ptr[k];
-    }
-    __syncthreads();
-    for (int sw = 0; sw < nu; ++sw)
-      for (int c = 0; c < L.ncol; ++c) {
-        for (int k = L.cs[c] + threadIdx.x; k < L.cs[c + 1]; k += blockDim.x) {
-          T acc[K];
-#pragma unroll
-          for (int j = 0; j < K; ++j) acc[j] = Fl[k * K + j];
-          small_row_k(acc, Psm[k], Psm[k + 1], sm_vals(L, (const V*)nullptr), L.sm_col, Ul);
-          const T di = L.dinv[k];
-#pragma unroll
-          for (int j = 0; j < K; ++j) Ul[k * K + j] += acc[j] * di;
-        }
-        __syncthreads();
-      }
-    for (int k = threadIdx.x; k < mE; k += blockDim.x) {
-      T acc[K];
-#pragma unroll
-      for (int j = 0; j < K; ++j) acc[j] = Fl[k * K + j];
-      small_row_k(acc, Prs[k], Prs[k + 1], rs_vals(L, (const V*)nullptr), L.rs_col, Ul);
-#pragma unroll
-      for (int j = 0; j < K; ++j) Fl[k * K + j] = acc[j];
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < L.npar; t += blockDim.x) {
-      T acc[K];
-#pragma unroll
-      for (int j = 0; j < K; ++j) acc[j] = 0;
-      for (int p = L.rp_ptr[t]; p < L.rp_ptr[t + 1]; ++p)
-#pragma unroll
-        for (int j = 0; j < K; ++j) acc[j] += Fl[(int)L.rp_child[p] * K + j];
-      const int pr = L.rp_id[t];
-#pragma unroll
-      for (int j = 0; j < K; ++j) Fl[pr * K + j] += (T)0.5 * acc[j];
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < mE; k += blockDim.x) {
-      VK<T> f, u;
-#pragma unroll
-      for (int j = 0; j < K; ++j) {
-        f.v[j] = Fl[k * K + j];
-        u.v[j] = Ul[k * K + j];
-      }
-      stk<T>(F + (int64_t)L.gid[k] * K, f);
-      if (k < mS) stk<T>(L.us + (int64_t)k * K, u);
-    }
-    __syncthreads();
-  }
-}
-
-template <class T, class V>
-__global__ void __launch_bounds__(SMALL_TPB_K, 1)
-    k_small_up_k(const SmallDesc<T>* __restrict__ D, int nlev, T* U, int nu) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int LM = small_lmax_k<T>();
-  T* Ul = reinterpret_cast<T*>(smraw);
-  T* Fl = Ul + LM * K;
-  int32_t* Psm = reinterpret_cast<int32_t*>(Fl + LM * K);
-  if (nlev > 0) small_prefetch<T, V>(D + nlev - 1, false);
-  pdl_wait();
-  for (int d = nlev - 1; d >= 0; --d) {
-    const SmallDesc<T>& L = D[d];
-    const int mS = L.mS, mE = L.mE;
-    if (d > 0) small_prefetch<T, V>(D + d - 1, false);
-    for (int k = threadIdx.x; k < mE; k += blockDim.x) {
-      const VK<T> u = ldk<T>(U + (int64_t)L.gid[k] * K);
-#pragma unroll
-      for (int j = 0; j < K; ++j) Ul[k * K + j] = u.v[j];
-      if (k < mS) {
-        const VK<T> f = ldk<T>(L.fs + (int64_t)k * K);
-#pragma unroll
-        for (int j = 0; j < K; ++j) Fl[k * K + j] = f.v[j];
-      }
-      if (k <= mS) Psm[k] = L.sm_ptr[k];
-    }
-    if (mS == mE && threadIdx.x == 0) Psm[mS] = L.sm_ptr[mS];
-    __syncthreads();
-    for (int t = threadIdx.x; t < L.nnew; t += blockDim.x) {
-      const int32_t a = L.nn_p0[t], b = L.nn_p1[t];
-      const int me = L.nn_id[t];
-#pragma unroll
-      for (int j = 0; j < K; ++j) {
-        T v = 0;
-        if (a >= 0) v += Ul[a * K + j];
-        if (b >= 0) v += Ul[b * K + j];
-        Ul[me * K + j] = (T)0.5 * v;
-      }
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < mS; k += blockDim.x) {
-      const VK<T> s = ldk<T>(L.us + (int64_t)k * K);
-#pragma unroll
-      for (int j = 0; j < K; ++j) Ul[k * K + j] += s.v[j];
-    }
-    __syncthreads();
-    for (int sw = 0; sw < nu; ++sw)
-      for (int c = L.ncol - 1; c >= 0; --c) {
-        for (int k = L.cs[c] + threadIdx.x; k < L.cs[c + 1]; k += blockDim.x) {
-          T acc[K];
-#pragma unroll
-          for (int j = 0; j < K; ++j) acc[j] = Fl[k * K + j];
-          small_row_k(acc, Psm[k], Psm[k + 1], sm_vals(L, (const V*)nullptr), L.sm_col, Ul);
-          const T di = L.dinv[k];
-#pragma unroll
-          for (int j = 0; j < K; ++j) Ul[k * K + j] += acc[j] * di;
-        }
-        __syncthreads();
-      }
-    for (int k = threadIdx.x; k < mS; k += blockDim.x) {
-      VK<T> u;
-#pragma unroll
-      for (int j = 0; j < K; ++j) u.v[j] = Ul[k * K + j];
-      stk<T>(U + (int64_t)L.gid[k] * K, u);
-    }
-    __syncthreads();
-  }
-}
-
 // ------------------------------------------------------------------ PCG
 __device__ __forceinline__ void set_cond_k(MultiScalars* sc, int cond, cudaGraphConditionalHandle hnd, int use_hnd) {
   sc->cond = cond;
@@ -843,9 +657,8 @@ void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
   const bool pdl = h.prm.use_pdl;
   const int npre = h.prm.nu_pre, npost = h.prm.nu_post;
   const int nlev = (int)P.lev.size();
-  const int ndeep = M.n_deep, nbot = M.n_bottom;
-  const size_t smem = small_smem_k<T>();
-  if (ndeep) launch_smem(pdl, k_small_down_k<T, V>, 1, SMALL_TPB_K, smem, s, M.deep_desc.p, ndeep, M.F.p, npre);
+  const int ndeep = P.deep_k.v.nlev, nbot = P.bot_k.v.nlev;
+  if (ndeep) small::launch_down<T, V, K>(pdl, P.deep_k, M.F.p, M.deep_fs.p, M.deep_us.p, npre, s);
   for (int li = nlev - 1 - ndeep; li >= nbot; --li) {
     AuxLevelDev<T>& L = P.lev[li];
     auto SMd = view(L.SMd);
@@ -862,10 +675,10 @@ void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
     launch(pdl, k_restrict_aux_k<T>, nblk(L.npar, rows_tpb(L.npar)), rows_tpb(L.npar), s, L.npar, L.rp_id.p,
            L.rp_ptr.p, L.rp_child.p, M.F.p);
   }
-  if (nbot) launch_smem(pdl, k_small_down_k<T, V>, 1, SMALL_TPB_K, smem, s, M.bot_desc.p, nbot, M.F.p, npre);
+  if (nbot) small::launch_down<T, V, K>(pdl, P.bot_k, M.F.p, M.bot_fs.p, M.bot_us.p, npre, s);
   if (h.nc > 0)
     launch(pdl, k_coarse_k<T>, nblk(h.nc * 32), TPB, s, h.nc, h.d_cid.p, h.d_cinv.p, (const T*)M.F.p, M.U.p);
-  if (nbot) launch_smem(pdl, k_small_up_k<T, V>, 1, SMALL_TPB_K, smem, s, M.bot_desc.p, nbot, M.U.p, npost);
+  if (nbot) small::launch_up<T, V, K>(pdl, P.bot_k, M.U.p, M.bot_fs.p, M.bot_us.p, npost, s);
   for (int li = nbot; li <= nlev - 1 - ndeep; ++li) {
     AuxLevelDev<T>& L = P.lev[li];
     auto SM = view(L.SM);
@@ -882,7 +695,7 @@ void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
                L.sm_dinv.p, L.sm_rows.p, (const T*)M.fs[li].p, M.U.p);
       }
   }
-  if (ndeep) launch_smem(pdl, k_small_up_k<T, V>, 1, SMALL_TPB_K, smem, s, M.deep_desc.p, ndeep, M.U.p, npost);
+  if (ndeep) small::launch_up<T, V, K>(pdl, P.deep_k, M.U.p, M.deep_fs.p, M.deep_us.p, npost, s);
 }
 
 // z = B_co r for KRHS columns (Algorithm 1, multiplicative, Gauss-Seidel)
@@ -956,8 +769,7 @@ void enqueue_init_k(asmg_s& h, MultiSlot& S, double rtol, cudaStream_t s, cudaGr
   ASMG_CUDA(cudaGetLastError());
 }
 
-// Work state for KRHS columns in precision T, and the fused small-level runs
-// whose levels fit small_lmax_k<T>() rows.
+// Work state for KRHS columns in precision T.
 template <class T>
 void alloc_multi_prec(asmg_s& h, MultiPrec<T>& M, cudaStream_t s) {
   Prec<T>& P = prec_of<T>(h);
@@ -980,62 +792,10 @@ void alloc_multi_prec(asmg_s& h, MultiPrec<T>& M, cudaStream_t s) {
     M.fs[li].zero(s);
     M.us[li].zero(s);
   }
-  auto fits = [&](int li) {
-    const SmallLevelDev<T>& q = P.lev[li].small;
-    return q.ok && q.mE <= small_lmax_k<T>();
-  };
-  int nd = 0;
-  while (nd < nlev && fits(nlev - 1 - nd)) ++nd;
-  int nb = 0;
-  if (nd < nlev)
-    while (nb < nlev - nd && fits(nb)) ++nb;
-  M.n_deep = nd;
-  M.n_bottom = nb;
-  auto desc = [&](int li) {
-    AuxLevelDev<T>& L = P.lev[li];
-    SmallLevelDev<T>& S = L.small;
-    SmallDesc<T> d;
-    d.mS = S.mS;
-    d.mE = S.mE;
-    d.ncol = S.ncol;
-    d.nnew = S.nnew;
-    d.npar = S.npar;
-    d.nnz_sm = (int)S.nnz_sm;
-    d.nnz_rs = (int)S.nnz_rs;
-    d.nchild = (int)S.nchild;
-    for (int c = 0; c <= SMALL_MAXC; ++c) d.cs[c] = c <= S.ncol ? S.cs[c] : S.mS;
-    d.gid = S.gid.p;
-    d.sm_ptr = S.sm_ptr.p;
-    d.sm_col = S.sm_col.p;
-    d.sm_val = S.sm_val.p;
-    d.sm_v16 = S.sm_v16.p;
-    d.dinv = S.dinv.p;
-    d.rs_ptr = S.rs_ptr.p;
-    d.rs_col = S.rs_col.p;
-    d.rs_val = S.rs_val.p;
-    d.rs_v16 = S.rs_v16.p;
-    d.nn_id = S.nn_id.p;
-    d.nn_p0 = S.nn_p0.p;
-    d.nn_p1 = S.nn_p1.p;
-    d.rp_id = S.rp_id.p;
-    d.rp_ptr = S.rp_ptr.p;
-    d.rp_child = S.rp_child.p;
-    d.fs = M.fs[li].p;
-    d.us = M.us[li].p;
-    return d;
-  };
-  std::vector<SmallDesc<T>> deep, bot;
-  for (int k = 0; k < nd; ++k) deep.push_back(desc(nlev - 1 - k));
-  for (int k = nb - 1; k >= 0; --k) bot.push_back(desc(k));
-  M.deep_desc.upload(deep, s);
-  M.bot_desc.upload(bot, s);
-  const int smem = (int)small_smem_k<T>();
-  ASMG_CUDA(cudaFuncSetAttribute(k_small_down_k<T, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  ASMG_CUDA(cudaFuncSetAttribute(k_small_up_k<T, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  if constexpr (std::is_same<T, float>::value) {
-    ASMG_CUDA(cudaFuncSetAttribute(k_small_down_k<T, bf16v>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ASMG_CUDA(cudaFuncSetAttribute(k_small_up_k<T, bf16v>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  }
+  for (DBuf<T>* v : {&M.deep_fs, &M.deep_us}) v->alloc(std::max(P.deep_k.v.nsm, 1) * K);
+  for (DBuf<T>* v : {&M.bot_fs, &M.bot_us}) v->alloc(std::max(P.bot_k.v.nsm, 1) * K);
+  small::set_smem_limits<T, T, K>();
+  if constexpr (std::is_same<T, float>::value) small::set_smem_limits<T, bf16v, K>();
 }
 
 void build_graph_k(asmg_s& h, MultiSlot& S, double rtol) {
