@@ -190,97 +190,159 @@ HostCSR coo_to_csr(int64_t m, DBuf<uint64_t>& key, DBuf<double>& val, int64_t nr
   return A;
 }
 
+// |T| / 12 (triangles) or |T| / 20 (tetrahedra): the weights of the mass
+// product.  Kept per element: recomputing each around every vertex reads its
+// coordinates again and divides in FP64 (2 FMA a cycle and SM) 6 times in 2D,
+// 24 times in 3D.
+__global__ void k_elem_mass(int64_t ne, const double* __restrict__ X, const int32_t* __restrict__ E,
+                            double* __restrict__ w) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= ne) return;
+  const int32_t v0 = E[3 * t], v1 = E[3 * t + 1], v2 = E[3 * t + 2];
+  const double area = 0.5 * ((X[2 * v1] - X[2 * v0]) * (X[2 * v2 + 1] - X[2 * v0 + 1]) -
+                             (X[2 * v2] - X[2 * v0]) * (X[2 * v1 + 1] - X[2 * v0 + 1]));
+  w[t] = area / 12.0;
+}
+
+__global__ void k_elem_mass3(int64_t ne, const double* __restrict__ X, const int32_t* __restrict__ E,
+                             double* __restrict__ w) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= ne) return;
+  double P[4][3];
+  for (int k = 0; k < 4; ++k)
+    for (int r = 0; r < 3; ++r) P[k][r] = X[3 * (int64_t)E[4 * t + k] + r];
+  double e[3][3];
+  for (int k = 0; k < 3; ++k)
+    for (int r = 0; r < 3; ++r) e[k][r] = P[k + 1][r] - P[0][r];
+  const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
+                     e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
+                     e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
+  w[t] = det / 120.0;
+}
+
 // consistent P1 mass matrix applied to nodal values, gathered per vertex:
 // b_v = sum over the elements T around v (ascending element index) of
-// |T|/12 (f_v + sum_j f_j) in 2D, |T|/20 (f_v + sum_j f_j) in 3D.  Each sum
-// runs in a fixed order, so the result is the same bit for bit on every run
-// (no atomics).  v2e: element indices around each vertex (CSR by vertex).
+// w_T (f_v + sum_j f_j), 0 at vertices without a row.  Each sum runs in a
+// fixed order, so the result is the same bit for bit on every run (no
+// atomics).  v2e: element indices around each vertex (CSR by vertex).
+template <int NV>
 __global__ void k_mass_gather(int64_t nv, const int64_t* __restrict__ v2e_ptr, const int32_t* __restrict__ v2e,
-                              const double* __restrict__ X, const int32_t* __restrict__ E,
-                              const double* __restrict__ f, double* __restrict__ b) {
+                              const double* __restrict__ w, const int32_t* __restrict__ E,
+                              const int32_t* __restrict__ rowv, const double* __restrict__ f,
+                              double* __restrict__ b) {
   const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (v >= nv) return;
   double acc = 0;
-  const double fv = f[v];
-  for (int64_t p = v2e_ptr[v]; p < v2e_ptr[v + 1]; ++p) {
-    const int64_t t = v2e[p];
-    const int32_t v0 = E[3 * t], v1 = E[3 * t + 1], v2 = E[3 * t + 2];
-    const double area = 0.5 * ((X[2 * v1] - X[2 * v0]) * (X[2 * v2 + 1] - X[2 * v0 + 1]) -
-                               (X[2 * v2] - X[2 * v0]) * (X[2 * v1 + 1] - X[2 * v0 + 1]));
-    const double sum = f[v0] + f[v1] + f[v2];
-    acc += area / 12.0 * (sum + fv);
+  if (rowv[v] >= 0) {
+    const double fv = f[v];
+    const int64_t p1 = v2e_ptr[v + 1];
+    for (int64_t p = v2e_ptr[v]; p < p1; ++p) {
+      const int64_t t = v2e[p];
+      int32_t q[NV];
+      if constexpr (NV == 4) {
+        const int4 e = *reinterpret_cast<const int4*>(E + 4 * t);
+        q[0] = e.x;
+        q[1] = e.y;
+        q[2] = e.z;
+        q[3] = e.w;
+      } else {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) q[k] = E[NV * t + k];
+      }
+      double sum = f[q[0]];
+#pragma unroll
+      for (int k = 1; k < NV; ++k) sum += f[q[k]];
+      acc += w[t] * (sum + fv);
+    }
   }
   b[v] = acc;
 }
 
-__global__ void k_mass_gather3(int64_t nv, const int64_t* __restrict__ v2e_ptr, const int32_t* __restrict__ v2e,
-                               const double* __restrict__ X, const int32_t* __restrict__ E,
-                               const double* __restrict__ f, double* __restrict__ b) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= nv) return;
-  double acc = 0;
-  const double fv = f[v];
-  for (int64_t p = v2e_ptr[v]; p < v2e_ptr[v + 1]; ++p) {
-    const int64_t t = v2e[p];
-    int32_t w[4];
-    double P[4][3];
-    for (int k = 0; k < 4; ++k) {
-      w[k] = E[4 * t + k];
-      for (int r = 0; r < 3; ++r) P[k][r] = X[3 * (int64_t)w[k] + r];
+// Element stiffness for a = 1 without its first row and column (rows sum to
+// 0): entries (i, j), 1 <= i <= j <= d, one array of ne after another.
+template <int D>
+__device__ __forceinline__ void elem_stiffness(int64_t t, const double* __restrict__ X, const int32_t* __restrict__ E,
+                                               double (&k)[D * (D + 1) / 2]) {
+  if constexpr (D == 2) {
+    double x[3], y[3], K[3][3];
+    for (int q = 0; q < 3; ++q) {
+      const int32_t v = E[3 * t + q];
+      x[q] = X[2 * (int64_t)v];
+      y[q] = X[2 * (int64_t)v + 1];
     }
-    double e[3][3];
-    for (int k = 0; k < 3; ++k)
-      for (int r = 0; r < 3; ++r) e[k][r] = P[k + 1][r] - P[0][r];
-    const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
-                       e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
-                       e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
-    const double sum = f[w[0]] + f[w[1]] + f[w[2]] + f[w[3]];
-    acc += det / 120.0 * (sum + fv);  // |T| / 20
+    tri_K(x, y, 1.0, K);
+    k[0] = K[1][1];
+    k[1] = K[1][2];
+    k[2] = K[2][2];
+  } else {
+    double P[4][3], K[4][4];
+    for (int q = 0; q < 4; ++q)
+      for (int r = 0; r < 3; ++r) P[q][r] = X[3 * (int64_t)E[4 * t + q] + r];
+    tet_K(P, 1.0, K);
+    k[0] = K[1][1];
+    k[1] = K[1][2];
+    k[2] = K[1][3];
+    k[3] = K[2][2];
+    k[4] = K[2][3];
+    k[5] = K[3][3];
   }
-  b[v] = acc;
+}
+
+template <int D>
+__global__ void k_elem_stiffness(int64_t ne, const double* __restrict__ X, const int32_t* __restrict__ E,
+                                 double* __restrict__ K) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= ne) return;
+  double k[D * (D + 1) / 2];
+  elem_stiffness<D>(t, X, E, k);
+#pragma unroll
+  for (int q = 0; q < D * (D + 1) / 2; ++q) K[q * ne + t] = k[q];
 }
 
 // dL/da_e = -lambda_e^T K_e^(1) u_e, times scale[e] when scale is given
-// (scale = a: the derivative with respect to g_e for a = exp(g))
-__global__ void k_elem_grad3(int64_t ne, const double* __restrict__ X, const int32_t* __restrict__ E,
-                             const double* __restrict__ u, const double* __restrict__ lam,
-                             const double* __restrict__ scale, double* __restrict__ g) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= ne) return;
-  double P[4][3], ue[4], le[4];
-  for (int k = 0; k < 4; ++k) {
-    int32_t v = E[4 * t + k];
-    for (int r = 0; r < 3; ++r) P[k][r] = X[3 * (int64_t)v + r];
-    ue[k] = u[v];
-    le[k] = lam[v];
-  }
-  double K[4][4];
-  tet_K(P, 1.0, K);
-  double s = 0;
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) s += le[i] * K[i][j] * ue[j];
-  g[t] = scale ? -(scale[t] * s) : -s;
-}
-
-// dL/da_e = -lambda_e^T K_e^(1) u_e (times scale[e] when given), triangles
+// (scale = a: the derivative with respect to g_e for a = exp(g)), from the
+// differences to the element's first vertex.  Kst: the stored stiffness, or
+// NULL to compute it here.  In FP64 the chip does 2 FMA a cycle and SM, so
+// forming the tetrahedron's stiffness each time bounded the call: 1.57 M
+// tetrahedra 390 us.
+template <int D>
 __global__ void k_elem_grad(int64_t ne, const double* __restrict__ X, const int32_t* __restrict__ E,
-                            const double* __restrict__ u, const double* __restrict__ lam,
+                            const double* __restrict__ Kst, const double2* __restrict__ pair,
                             const double* __restrict__ scale, double* __restrict__ g) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= ne) return;
-  double x[3], y[3], ue[3], le[3];
-  for (int k = 0; k < 3; ++k) {
-    int32_t v = E[3 * t + k];
-    x[k] = X[2 * v];
-    y[k] = X[2 * v + 1];
-    ue[k] = u[v];
-    le[k] = lam[v];
+  double k[D * (D + 1) / 2];
+  if (Kst) {
+#pragma unroll
+    for (int q = 0; q < D * (D + 1) / 2; ++q) k[q] = __ldcs(Kst + q * ne + t);
+  } else {
+    elem_stiffness<D>(t, X, E, k);
   }
-  double K[3][3];
-  tri_K(x, y, 1.0, K);
-  double s = 0;
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) s += le[i] * K[i][j] * ue[j];
+  int32_t v[D + 1];
+  if constexpr (D == 3) {
+    const int4 e = *reinterpret_cast<const int4*>(E + 4 * t);
+    v[0] = e.x;
+    v[1] = e.y;
+    v[2] = e.z;
+    v[3] = e.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q <= D; ++q) v[q] = E[(D + 1) * t + q];
+  }
+  const double2 p0 = pair[v[0]];
+  double du[D], dl[D];
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    const double2 p = pair[v[q + 1]];
+    du[q] = p.x - p0.x;
+    dl[q] = p.y - p0.y;
+  }
+  double s;
+  if constexpr (D == 2)
+    s = du[0] * (k[0] * dl[0] + k[1] * dl[1]) + du[1] * (k[1] * dl[0] + k[2] * dl[1]);
+  else
+    s = du[0] * (k[0] * dl[0] + k[1] * dl[1] + k[2] * dl[2]) + du[1] * (k[1] * dl[0] + k[3] * dl[1] + k[4] * dl[2]) +
+        du[2] * (k[2] * dl[0] + k[4] * dl[1] + k[5] * dl[2]);
   g[t] = scale ? -(scale[t] * s) : -s;
 }
 
@@ -394,21 +456,38 @@ HostCSR assemble_mesh(int dim, int64_t ne, const double* dX, const int32_t* dE, 
   return coo_to_csr(m, key, val, nfree, s);
 }
 
-void mass_apply_gpu(int dim, int64_t nv, const int64_t* v2e_ptr, const int32_t* v2e, const double* dX,
-                    const int32_t* dE, const double* df, double* db, cudaStream_t s) {
+void element_mass_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, double* w, cudaStream_t s) {
   if (dim == 2)
-    k_mass_gather<<<nblk(nv), 256, 0, s>>>(nv, v2e_ptr, v2e, dX, dE, df, db);
+    k_elem_mass<<<nblk(ne), 256, 0, s>>>(ne, dX, dE, w);
   else
-    k_mass_gather3<<<nblk(nv), 256, 0, s>>>(nv, v2e_ptr, v2e, dX, dE, df, db);
+    k_elem_mass3<<<nblk(ne), 256, 0, s>>>(ne, dX, dE, w);
   ASMG_CUDA(cudaGetLastError());
 }
 
-void element_grad_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, const double* du, const double* dl,
-                      const double* dscale, double* dg, cudaStream_t s) {
+void mass_apply_gpu(int dim, int64_t nv, const int64_t* v2e_ptr, const int32_t* v2e, const double* w,
+                    const int32_t* dE, const int32_t* row_of_vertex, const double* df, double* db, cudaStream_t s) {
   if (dim == 2)
-    k_elem_grad<<<nblk(ne), 256, 0, s>>>(ne, dX, dE, du, dl, dscale, dg);
+    k_mass_gather<3><<<nblk(nv), 256, 0, s>>>(nv, v2e_ptr, v2e, w, dE, row_of_vertex, df, db);
   else
-    k_elem_grad3<<<nblk(ne), 256, 0, s>>>(ne, dX, dE, du, dl, dscale, dg);
+    k_mass_gather<4><<<nblk(nv), 256, 0, s>>>(nv, v2e_ptr, v2e, w, dE, row_of_vertex, df, db);
+  ASMG_CUDA(cudaGetLastError());
+}
+
+void element_stiffness_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, double* K, cudaStream_t s) {
+  if (dim == 2)
+    k_elem_stiffness<2><<<nblk(ne), 256, 0, s>>>(ne, dX, dE, K);
+  else
+    k_elem_stiffness<3><<<nblk(ne), 256, 0, s>>>(ne, dX, dE, K);
+  ASMG_CUDA(cudaGetLastError());
+}
+
+void element_grad_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, const double* K, const double* pair,
+                      const double* dscale, double* dg, cudaStream_t s) {
+  const double2* p = reinterpret_cast<const double2*>(pair);
+  if (dim == 2)
+    k_elem_grad<2><<<nblk(ne), 256, 0, s>>>(ne, dX, dE, K, p, dscale, dg);
+  else
+    k_elem_grad<3><<<nblk(ne), 256, 0, s>>>(ne, dX, dE, K, p, dscale, dg);
   ASMG_CUDA(cudaGetLastError());
 }
 

@@ -55,6 +55,29 @@ void copy_out(double* dst, const double* src, int64_t n, cudaStream_t s) {
   ASMG_CUDA(cudaMemcpyAsync(dst, src, 8 * n, is_device(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
 }
 
+// A device array the kernels read or write in place: memory of the current
+// device, aligned for its type.  Anything else (host, managed or another
+// device's memory) goes through the handle's staging arrays.
+bool in_place(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  int dev = -1;
+  ASMG_CUDA(cudaGetDevice(&dev));
+  return a.type == cudaMemoryTypeDevice && a.device == dev && (uintptr_t)p % sizeof(double) == 0;
+}
+
+// The caller's input array where kernels can read it: itself, or a staged copy.
+// Calls on device arrays spent much of their time in these copies (graded
+// 1025^2, one operator product and one load vector: see amg_spmv).
+const double* input(const double* user, double* stage, int64_t n, cudaStream_t s) {
+  if (in_place(user)) return user;
+  copy_in(stage, user, n, s);
+  return stage;
+}
+
 int64_t pad32(int64_t n) { return (n + 31) / 32 * 32; }
 
 // Temporally blocked sweeps (asmg_params::tile_rows = 0): own rows per tile on
@@ -1237,6 +1260,7 @@ int amg_setup(int dim, int64_t nv, const double* vertices, int64_t ne, const int
   // load the allocation-free entry point's module (and so its fixed scratch
   // array) on this device now, so that its calls never create memory
   noalloc_scratch_for_current_device();
+  h->pinned.alloc(READBACK_SCALARS + 8 * (size_t)READBACK_HIST);
   h->stats.t_total = now() - t0;
   *out = h.release();
   return ASMG_OK;
@@ -1274,6 +1298,12 @@ struct asmg_batch_s {
   bool multi = false;  // right-hand sides in groups of KRHS columns (SpMM form), one graph branch per group
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  // per branch its vertex arrays of this call: `per` right-hand sides, then
+  // `per` solutions (NULL: an unused column, right-hand side 0); and the
+  // branches' scalars read back
+  int per = 1;
+  DBuf<double*> tab;
+  PinnedBuf tab_host, back;
   ~asmg_batch_s() {
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
@@ -1308,6 +1338,11 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
       while ((int)h->slots.size() < 1 + nrhs) add_slot(*h, s);
     }
   }
+  B->per = B->multi ? KRHS : 1;
+  const int nbranch = nprob * (B->multi ? ngroups : nrhs);
+  B->tab.alloc(2 * (int64_t)B->per * nbranch);
+  B->tab_host.alloc(sizeof(double*) * (size_t)B->tab.n);
+  B->back.alloc(READBACK_SCALARS * (size_t)nbranch);
   ASMG_CUDA(cudaGraphCreate(&B->graph, 0));
   cudaStream_t cs;
   ASMG_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -1319,8 +1354,9 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
         asmg_s& h = *B->H[p];
         MultiSlot& S = B->mslot(p, g);
         ASMG_CUDA(cudaStreamBeginCaptureToGraph(cs, B->graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        gather_multi(h, S.vb.p, S.b.p, cs);
-        gather_multi(h, S.vu.p, S.x.p, cs);
+        double* const* tab = B->tab.p + 2 * KRHS * (int64_t)(p * ngroups + g);
+        gather_multi_tab(h, tab, S.b.p, cs);
+        gather_multi_tab(h, tab + KRHS, S.x.p, cs);
         cudaStreamCaptureStatus st;
         const cudaGraphNode_t* leaf = nullptr;
         size_t nleaf = 0;
@@ -1330,7 +1366,7 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
         ASMG_CUDA(cudaStreamEndCapture(cs, &gg));
         cudaGraphNode_t wnode = capture_solve_multi(h, S, rtol, B->graph, leaves.data(), leaves.size());
         ASMG_CUDA(cudaStreamBeginCaptureToGraph(cs, B->graph, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
-        scatter_multi(h, S.x.p, S.vu.p, cs);
+        scatter_multi_tab(h, S.x.p, tab + KRHS, cs);
         ASMG_CUDA(cudaStreamEndCapture(cs, &gg));
       }
   }
@@ -1338,10 +1374,11 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
     for (int j = 0; j < nrhs; ++j) {
       asmg_s& h = *B->H[p];
       Slot& S = B->slot(p, j);
-      // gather the staged rhs / initial guess (a root of its own branch)
+      // gather the rhs / initial guess (a root of its own branch)
       ASMG_CUDA(cudaStreamBeginCaptureToGraph(cs, B->graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-      gather_rows(h, S.vb.p, S.b.p, cs);
-      gather_rows(h, S.vu.p, S.x.p, cs);
+      double* const* tab = B->tab.p + 2 * (int64_t)(p * nrhs + j);
+      gather_rows_tab(h, tab, S.b.p, cs);
+      gather_rows_tab(h, tab + 1, S.x.p, cs);
       cudaStreamCaptureStatus st;
       const cudaGraphNode_t* leaf = nullptr;
       size_t nleaf = 0;
@@ -1351,7 +1388,7 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
       ASMG_CUDA(cudaStreamEndCapture(cs, &gg));
       cudaGraphNode_t wnode = capture_solve(h, S, rtol, B->graph, leaves.data(), leaves.size());
       ASMG_CUDA(cudaStreamBeginCaptureToGraph(cs, B->graph, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
-      scatter_rows(h, S.x.p, false, S.vu.p, cs);
+      scatter_rows_tab(h, S.x.p, tab + 1, cs);
       ASMG_CUDA(cudaStreamEndCapture(cs, &gg));
     }
   ASMG_CUDA(cudaStreamDestroy(cs));
@@ -1369,76 +1406,67 @@ int amg_batch_solve(asmg_batch B, const double* const* bs, double* const* us, in
   const int np = (int)B->H.size(), nr = B->nrhs;
   for (int k = 0; k < np * nr; ++k)
     if (!bs[k] || !us[k]) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null array in batch");
-  if (B->multi) {
-    const int ngroups = (nr + KRHS - 1) / KRHS;
-    for (int p = 0; p < np; ++p)
-      for (int g = 0; g < ngroups; ++g) {
-        MultiSlot& S = B->mslot(p, g);
-        const int64_t nv = B->H[p]->mesh.nv;
-        for (int c = 0; c < KRHS; ++c) {
-          const int j = g * KRHS + c;
-          if (j < nr) {
-            copy_in(S.vb.p + c * nv, bs[p * nr + j], nv, s);
-            copy_in(S.vu.p + c * nv, us[p * nr + j], nv, s);
-          } else {
-            // unused column: zero right-hand side, converged from the start
-            ASMG_CUDA(cudaMemsetAsync(S.vb.p + c * nv, 0, 8 * nv, s));
-            ASMG_CUDA(cudaMemsetAsync(S.vu.p + c * nv, 0, 8 * nv, s));
-          }
-        }
-      }
-    ASMG_CUDA(cudaGraphLaunch(B->exec, s));
-    std::vector<MultiScalars> sc((size_t)np * ngroups);
-    for (int p = 0; p < np; ++p)
-      for (int g = 0; g < ngroups; ++g) {
-        MultiSlot& S = B->mslot(p, g);
-        const int64_t nv = B->H[p]->mesh.nv;
-        for (int c = 0; c < KRHS && g * KRHS + c < nr; ++c) copy_out(us[p * nr + g * KRHS + c], S.vu.p + c * nv, nv, s);
-        ASMG_CUDA(cudaMemcpyAsync(&sc[p * ngroups + g], S.scal.p, sizeof(MultiScalars), cudaMemcpyDeviceToHost, s));
-      }
-    ASMG_CUDA(cudaStreamSynchronize(s));
-    int worst = ASMG_OK;
-    for (int p = 0; p < np; ++p)
-      for (int j = 0; j < nr; ++j) {
-        const MultiScalars& m = sc[p * ngroups + j / KRHS];
-        const int c = j % KRHS;
-        iterations[p * nr + j] = m.k[c];
-        const int st = m.status[c] == 0                    ? ASMG_OK
-                       : m.status[c] == ASMG_ERR_BREAKDOWN ? ASMG_ERR_BREAKDOWN
-                       : m.status[c] == ASMG_ERR_TIMEOUT   ? ASMG_ERR_TIMEOUT
-                                                           : ASMG_NOT_CONVERGED;
-        if (status) status[p * nr + j] = st;
-        if (st < 0 || (worst == ASMG_OK && st != ASMG_OK)) worst = st;
-      }
-    if (worst == ASMG_ERR_BREAKDOWN) g_err = "PCG breakdown in a batched solve";
-    return worst;
-  }
+  // the branches read and write the caller's device arrays through the table;
+  // other arrays are staged
+  const int ngroups = B->multi ? (nr + KRHS - 1) / KRHS : nr;
+  double** tab = static_cast<double**>(B->tab_host.p);
+  struct Out {
+    double *user, *stage;
+    int64_t n;
+  };
+  std::vector<Out> staged;
   for (int p = 0; p < np; ++p)
-    for (int j = 0; j < nr; ++j) {
-      Slot& S = B->slot(p, j);
+    for (int g = 0; g < ngroups; ++g) {
       const int64_t nv = B->H[p]->mesh.nv;
-      copy_in(S.vb.p, bs[p * nr + j], nv, s);
-      copy_in(S.vu.p, us[p * nr + j], nv, s);
+      double* vb = B->multi ? B->mslot(p, g).vb.p : B->slot(p, g).vb.p;
+      double* vu = B->multi ? B->mslot(p, g).vu.p : B->slot(p, g).vu.p;
+      double** t = tab + 2 * (int64_t)B->per * (p * ngroups + g);
+      for (int c = 0; c < B->per; ++c) {
+        const int j = g * B->per + c;
+        t[c] = t[B->per + c] = nullptr;
+        if (j >= nr) continue;
+        const double* b = bs[p * nr + j];
+        double* u = us[p * nr + j];
+        t[c] = const_cast<double*>(input(b, vb + c * nv, nv, s));
+        t[B->per + c] = const_cast<double*>(input(u, vu + c * nv, nv, s));
+        if (t[B->per + c] != u) staged.push_back({u, vu + c * nv, nv});
+      }
     }
+  ASMG_CUDA(cudaMemcpyAsync(B->tab.p, tab, sizeof(double*) * (size_t)B->tab.n, cudaMemcpyHostToDevice, s));
   ASMG_CUDA(cudaGraphLaunch(B->exec, s));
-  std::vector<PcgScalars> sc((size_t)np * nr);
+  char* back = static_cast<char*>(B->back.p);
   for (int p = 0; p < np; ++p)
-    for (int j = 0; j < nr; ++j) {
-      Slot& S = B->slot(p, j);
-      copy_out(us[p * nr + j], S.vu.p, B->H[p]->mesh.nv, s);
-      ASMG_CUDA(cudaMemcpyAsync(&sc[p * nr + j], S.scal.p, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
+    for (int g = 0; g < ngroups; ++g) {
+      char* dst = back + READBACK_SCALARS * (size_t)(p * ngroups + g);
+      if (B->multi)
+        ASMG_CUDA(cudaMemcpyAsync(dst, B->mslot(p, g).scal.p, sizeof(MultiScalars), cudaMemcpyDeviceToHost, s));
+      else
+        ASMG_CUDA(cudaMemcpyAsync(dst, B->slot(p, g).scal.p, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
     }
+  for (const Out& o : staged) copy_out(o.user, o.stage, o.n, s);
   ASMG_CUDA(cudaStreamSynchronize(s));
   int worst = ASMG_OK;
-  for (size_t k = 0; k < sc.size(); ++k) {
-    iterations[k] = sc[k].k;
-    const int st = sc[k].status == 0                    ? ASMG_OK
-                   : sc[k].status == ASMG_ERR_BREAKDOWN ? ASMG_ERR_BREAKDOWN
-                   : sc[k].status == ASMG_ERR_TIMEOUT   ? ASMG_ERR_TIMEOUT
-                                                        : ASMG_NOT_CONVERGED;
-    if (status) status[k] = st;
-    if (st < 0 || (worst == ASMG_OK && st != ASMG_OK)) worst = st;
-  }
+  for (int p = 0; p < np; ++p)
+    for (int j = 0; j < nr; ++j) {
+      const char* src = back + READBACK_SCALARS * (size_t)(p * ngroups + j / B->per);
+      int k, code;
+      if (B->multi) {
+        const MultiScalars& m = *reinterpret_cast<const MultiScalars*>(src);
+        k = m.k[j % KRHS];
+        code = m.status[j % KRHS];
+      } else {
+        const PcgScalars& m = *reinterpret_cast<const PcgScalars*>(src);
+        k = m.k;
+        code = m.status;
+      }
+      iterations[p * nr + j] = k;
+      const int st = code == 0                    ? ASMG_OK
+                     : code == ASMG_ERR_BREAKDOWN ? ASMG_ERR_BREAKDOWN
+                     : code == ASMG_ERR_TIMEOUT   ? ASMG_ERR_TIMEOUT
+                                                  : ASMG_NOT_CONVERGED;
+      if (status) status[p * nr + j] = st;
+      if (st < 0 || (worst == ASMG_OK && st != ASMG_OK)) worst = st;
+    }
   if (worst == ASMG_ERR_BREAKDOWN) g_err = "PCG breakdown in a batched solve";
   if (worst == ASMG_ERR_TIMEOUT) g_err = "a bounded device wait expired in a batched solve";
   return worst;
@@ -1461,8 +1489,7 @@ int amg_profile(asmg_handle h, const double* b, double rtol, double* out, int* i
   cudaStream_t s = (cudaStream_t)stream;
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv;
-  copy_in(S0.vb.p, b, nv, s);
-  gather_rows(*h, S0.vb.p, S0.b.p, s);
+  gather_rows(*h, input(b, S0.vb.p, nv, s), S0.b.p, s);
   S0.x.zero(s);
   *iterations = profile_solve(*h, rtol, s, out);
   return ASMG_OK;
@@ -1477,8 +1504,7 @@ int amg_profile_levels(asmg_handle h, const double* b, double rtol, double* out,
   cudaStream_t s = (cudaStream_t)stream;
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv;
-  copy_in(S0.vb.p, b, nv, s);
-  gather_rows(*h, S0.vb.p, S0.b.p, s);
+  gather_rows(*h, input(b, S0.vb.p, nv, s), S0.b.p, s);
   S0.x.zero(s);
   *iterations = profile_solve(*h, rtol, s, out, out_levels, nlev);
   return ASMG_OK;
@@ -1493,20 +1519,26 @@ int amg_solve(asmg_handle h, const double* b, double* u, double rtol, int* itera
   cudaStream_t s = (cudaStream_t)stream;
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv;
-  copy_in(S0.vb.p, b, nv, s);
-  copy_in(S0.vu.p, u, nv, s);
-  gather_rows(*h, S0.vb.p, S0.b.p, s);
-  gather_rows(*h, S0.vu.p, S0.x.p, s);
+  const bool direct = in_place(u);
+  gather_rows(*h, input(b, S0.vb.p, nv, s), S0.b.p, s);
+  gather_rows(*h, input(u, S0.vu.p, nv, s), S0.x.p, s);
   run_solve(*h, S0, rtol, s);
-  scatter_rows(*h, S0.x.p, false, S0.vu.p, s);
-  copy_out(u, S0.vu.p, nv, s);
-  PcgScalars sc;
+  scatter_rows(*h, S0.x.p, false, direct ? u : S0.vu.p, s);
+  if (!direct) copy_out(u, S0.vu.p, nv, s);
+  // the scalars and the start of the history come back together, in pinned memory
+  PcgScalars& sc = *static_cast<PcgScalars*>(h->pinned.p);
+  double* hist = reinterpret_cast<double*>(static_cast<char*>(h->pinned.p) + READBACK_SCALARS);
+  const int nh = std::min(h->prm.max_iter + 1, READBACK_HIST);
   ASMG_CUDA(cudaMemcpyAsync(&sc, S0.scal.p, sizeof sc, cudaMemcpyDeviceToHost, s));
+  if (res_history) ASMG_CUDA(cudaMemcpyAsync(hist, S0.hist.p, 8 * (size_t)nh, cudaMemcpyDeviceToHost, s));
   ASMG_CUDA(cudaStreamSynchronize(s));
   *iterations = sc.k;
   if (res_history) {
-    ASMG_CUDA(cudaMemcpyAsync(res_history, S0.hist.p, 8 * (size_t)(sc.k + 1), cudaMemcpyDeviceToHost, s));
-    ASMG_CUDA(cudaStreamSynchronize(s));
+    std::memcpy(res_history, hist, 8 * (size_t)std::min(sc.k + 1, nh));
+    if (sc.k + 1 > nh) {
+      ASMG_CUDA(cudaMemcpyAsync(res_history + nh, S0.hist.p + nh, 8 * (size_t)(sc.k + 1 - nh), cudaMemcpyDeviceToHost, s));
+      ASMG_CUDA(cudaStreamSynchronize(s));
+    }
   }
   if (sc.status == ASMG_ERR_BREAKDOWN) {
     g_err = "PCG breakdown: <p, A p> or <r, z> not positive";
@@ -1533,21 +1565,13 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
   if (h->mslots.empty()) add_multi_slot(*h, s);
   MultiSlot& S = *h->mslots[0];
   const int64_t nv = h->mesh.nv;
-  for (int c = 0; c < KRHS; ++c) {
-    if (c < k) {
-      copy_in(S.vb.p + c * nv, b + c * nv, nv, s);
-      copy_in(S.vu.p + c * nv, u + c * nv, nv, s);
-    } else {
-      ASMG_CUDA(cudaMemsetAsync(S.vb.p + c * nv, 0, 8 * nv, s));
-      ASMG_CUDA(cudaMemsetAsync(S.vu.p + c * nv, 0, 8 * nv, s));
-    }
-  }
-  gather_multi(*h, S.vb.p, S.b.p, s);
-  gather_multi(*h, S.vu.p, S.x.p, s);
+  const bool direct = in_place(u);
+  gather_multi(*h, input(b, S.vb.p, k * nv, s), k, S.b.p, s);
+  gather_multi(*h, input(u, S.vu.p, k * nv, s), k, S.x.p, s);
   run_solve_multi(*h, S, rtol, s);
-  scatter_multi(*h, S.x.p, S.vu.p, s);
-  for (int c = 0; c < k; ++c) copy_out(u + c * nv, S.vu.p + c * nv, nv, s);
-  MultiScalars sc;
+  scatter_multi(*h, S.x.p, k, direct ? u : S.vu.p, s);
+  if (!direct) copy_out(u, S.vu.p, k * nv, s);
+  MultiScalars& sc = *static_cast<MultiScalars*>(h->pinned.p);
   ASMG_CUDA(cudaMemcpyAsync(&sc, S.scal.p, sizeof sc, cudaMemcpyDeviceToHost, s));
   ASMG_CUDA(cudaStreamSynchronize(s));
   const int64_t hl = h->prm.max_iter + 1;
@@ -1564,7 +1588,7 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
       ASMG_CUDA(cudaMemcpyAsync(res_history + c * hl, S.hist.p + c * hl, 8 * (size_t)(sc.k[c] + 1),
                                 cudaMemcpyDeviceToHost, s));
   }
-  ASMG_CUDA(cudaStreamSynchronize(s));
+  if (res_history) ASMG_CUDA(cudaStreamSynchronize(s));
   if (worst == ASMG_ERR_BREAKDOWN) g_err = "PCG breakdown in a column of a multiple solve";
   return worst;
   API_END
@@ -1589,12 +1613,15 @@ int amg_mass_apply(asmg_handle h, const double* f, double* bout, void* stream) {
       for (int k = 0; k < nvert; ++k) el[fill[m.E[e * nvert + k]]++] = (int32_t)e;
     h->d_v2e_ptr.upload(ptr, s);
     h->d_v2e.upload(el, s);
+    h->d_elem_mass.alloc(m.ne);
+    element_mass_gpu(m.dim, m.ne, h->dX.p, h->dE.p, h->d_elem_mass.p, s);
   }
-  copy_in(S0.vb.p, f, nv, s);
-  mass_apply_gpu(h->mesh.dim, nv, h->d_v2e_ptr.p, h->d_v2e.p, h->dX.p, h->dE.p, S0.vb.p, S0.vu.p, s);
-  gather_rows(*h, S0.vu.p, S0.q.p, s);
-  scatter_rows(*h, S0.q.p, false, S0.vu.p, s);  // zero at Dirichlet vertices
-  copy_out(bout, S0.vu.p, nv, s);
+  // the result goes straight to the caller's array unless it overlaps the input
+  const bool overlap = (uintptr_t)f < (uintptr_t)(bout + nv) && (uintptr_t)bout < (uintptr_t)(f + nv);
+  double* out = in_place(bout) && !overlap ? bout : S0.vu.p;
+  mass_apply_gpu(h->mesh.dim, nv, h->d_v2e_ptr.p, h->d_v2e.p, h->d_elem_mass.p, h->dE.p, h->d_row_of_vertex.p,
+                 input(f, S0.vb.p, nv, s), out, s);
+  if (out != bout) copy_out(bout, out, nv, s);
   ASMG_CUDA(cudaStreamSynchronize(s));
   return ASMG_OK;
   API_END
@@ -1606,17 +1633,18 @@ int amg_precond_apply(asmg_handle h, const double* r, double* z, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv;
-  copy_in(S0.vb.p, r, nv, s);
-  gather_rows(*h, S0.vb.p, S0.r.p, s);
+  gather_rows(*h, input(r, S0.vb.p, nv, s), S0.r.p, s);
   int* tflag = reinterpret_cast<int*>(reinterpret_cast<char*>(S0.scal.p) + offsetof(PcgScalars, timeout));
   ASMG_CUDA(cudaMemsetAsync(tflag, 0, sizeof(int), s));
   precond_apply(*h, S0.r.p, s);
+  const bool direct = in_place(z);
+  double* out = direct ? z : S0.vu.p;
   if (h->prm.precision == ASMG_MIXED)
-    scatter_rows(*h, S0.s32.uf.p, true, S0.vu.p, s);
+    scatter_rows(*h, S0.s32.uf.p, true, out, s);
   else
-    scatter_rows(*h, S0.s64.uf.p, false, S0.vu.p, s);
-  copy_out(z, S0.vu.p, nv, s);
-  int tout = 0;
+    scatter_rows(*h, S0.s64.uf.p, false, out, s);
+  if (!direct) copy_out(z, out, nv, s);
+  int& tout = *static_cast<int*>(h->pinned.p);
   ASMG_CUDA(cudaMemcpyAsync(&tout, tflag, sizeof(int), cudaMemcpyDeviceToHost, s));
   ASMG_CUDA(cudaStreamSynchronize(s));
   if (tout) ASMG_FAIL(ASMG_ERR_TIMEOUT, "a bounded device wait expired (a tile's shared-memory copy did not complete)");
@@ -1630,11 +1658,11 @@ int amg_spmv(asmg_handle h, const double* x, double* y, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv;
-  copy_in(S0.vb.p, x, nv, s);
-  gather_rows(*h, S0.vb.p, S0.p.p, s);
+  const bool direct = in_place(y);
+  gather_rows(*h, input(x, S0.vb.p, nv, s), S0.p.p, s);
   spmv64(*h, S0.p.p, S0.q.p, s);
-  scatter_rows(*h, S0.q.p, false, S0.vu.p, s);
-  copy_out(y, S0.vu.p, nv, s);
+  scatter_rows(*h, S0.q.p, false, direct ? y : S0.vu.p, s);
+  if (!direct) copy_out(y, S0.vu.p, nv, s);
   ASMG_CUDA(cudaStreamSynchronize(s));
   return ASMG_OK;
   API_END
@@ -1648,22 +1676,32 @@ void element_grad_common(asmg_handle h, const double* u, const double* lambda, d
                          cudaStream_t s) {
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv, ne = h->mesh.ne;
-  // Dirichlet entries are treated as 0: gather/scatter through the free rows
-  copy_in(S0.vb.p, u, nv, s);
-  gather_rows(*h, S0.vb.p, S0.p.p, s);
-  scatter_rows(*h, S0.p.p, false, S0.vb.p, s);
-  copy_in(S0.vu.p, lambda, nv, s);
-  gather_rows(*h, S0.vu.p, S0.q.p, s);
-  scatter_rows(*h, S0.q.p, false, S0.vu.p, s);
+  if (!h->d_elem_stiff.p && !h->elem_stiff_tried) {
+    // element stiffness (a = 1), kept for the handle's life where memory allows:
+    // recomputing it bounds the gradient by the FP64 units
+    h->elem_stiff_tried = true;
+    try {
+      h->d_elem_stiff.alloc(ne * (h->mesh.dim == 2 ? 3 : 6));
+      element_stiffness_gpu(h->mesh.dim, ne, h->dX.p, h->dE.p, h->d_elem_stiff.p, s);
+    } catch (const Error& e) {
+      h->d_elem_stiff.release();
+      if (e.code != ASMG_ERR_OOM) throw;
+      cudaGetLastError();
+    }
+  }
+  // (u, lambda) per vertex, Dirichlet entries 0
+  if (!h->d_pair.p) h->d_pair.alloc(2 * nv);
+  mask_pair(*h, input(u, S0.vb.p, nv, s), input(lambda, S0.vu.p, nv, s), h->d_pair.p, s);
   DBuf<double> dg;
-  const bool dev = is_device(g);
+  const bool dev = in_place(g);
   double* out = g;
   if (!dev) {
     dg.alloc(ne);
     out = dg.p;
   }
-  element_grad_gpu(h->mesh.dim, ne, h->dX.p, h->dE.p, S0.vb.p, S0.vu.p, log_coeff ? h->dCoeff.p : nullptr, out, s);
-  if (!dev) ASMG_CUDA(cudaMemcpyAsync(g, dg.p, 8 * ne, cudaMemcpyDeviceToHost, s));
+  element_grad_gpu(h->mesh.dim, ne, h->dX.p, h->dE.p, h->d_elem_stiff.p, h->d_pair.p,
+                   log_coeff ? h->dCoeff.p : nullptr, out, s);
+  if (!dev) copy_out(g, dg.p, ne, s);
   ASMG_CUDA(cudaStreamSynchronize(s));
 }
 

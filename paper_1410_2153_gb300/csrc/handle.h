@@ -27,6 +27,21 @@ const bf16v* sell_vals(const Sell<T>& S, const bf16v*) {
   return S.v16.p;
 }
 
+// Page-locked host memory: a copy into it does not pass through the driver's
+// staging.
+struct PinnedBuf {
+  void* p = nullptr;
+  PinnedBuf() = default;
+  PinnedBuf(const PinnedBuf&) = delete;
+  PinnedBuf& operator=(const PinnedBuf&) = delete;
+  ~PinnedBuf() {
+    if (p) cudaFreeHost(p);
+  }
+  void alloc(size_t bytes) { ASMG_CUDA(cudaHostAlloc(&p, bytes, cudaHostAllocDefault)); }
+};
+constexpr size_t READBACK_SCALARS = 512;  // bytes for a solve's scalars, then READBACK_HIST residual norms
+constexpr int READBACK_HIST = 512;
+
 // Scalars of the PCG recurrences, device resident.
 struct PcgScalars {
   double rz;      // <r_k, z_k>
@@ -111,6 +126,8 @@ struct MultiSlot {
   }
 };
 
+static_assert(sizeof(MultiScalars) <= READBACK_SCALARS && sizeof(PcgScalars) <= READBACK_SCALARS, "readback size");
+
 }  // namespace asmg
 
 struct asmg_s {
@@ -120,6 +137,11 @@ struct asmg_s {
   asmg::DBuf<int32_t> dE;
   asmg::DBuf<int64_t> d_v2e_ptr;  // elements around each vertex (CSR, ascending element), for the mass product
   asmg::DBuf<int32_t> d_v2e;
+  asmg::DBuf<double> d_elem_mass;   // [ne] |T| / 12 (triangles), |T| / 20 (tetrahedra), built with d_v2e
+  asmg::DBuf<double> d_elem_stiff;  // element stiffness for a = 1 (see element_stiffness_gpu), for the gradients
+  bool elem_stiff_tried = false;    // its allocation was tried (without it the gradients recompute it)
+  asmg::DBuf<double> d_pair;        // [nv][2] u and lambda, for the gradients
+  asmg::PinnedBuf pinned;           // what a call reads back from the device
   asmg::TreeResult tree;
   asmg::AuxHost aux;
 
@@ -173,16 +195,26 @@ void scatter_rows(asmg_s& h, const void* src, bool src_float, double* vdst, cuda
 // solve_multi.cu
 bool multi_supported(const asmg_s& h);
 MultiSlot& add_multi_slot(asmg_s& h, cudaStream_t s);
-void gather_multi(asmg_s& h, const double* vsrc, double* dst, cudaStream_t s);
-void scatter_multi(asmg_s& h, const double* src, double* vdst, cudaStream_t s);
+// k columns at vsrc + c nv (the others 0) -> interleaved rows, and back
+void gather_multi(asmg_s& h, const double* vsrc, int k, double* dst, cudaStream_t s);
+void scatter_multi(asmg_s& h, const double* src, int k, double* vdst, cudaStream_t s);
+// the same through device tables of vertex arrays: KRHS entries, NULL for an
+// unused column (one entry for gather_rows_tab / scatter_rows_tab)
+void gather_multi_tab(asmg_s& h, double* const* tab, double* dst, cudaStream_t s);
+void scatter_multi_tab(asmg_s& h, const double* src, double* const* tab, cudaStream_t s);
+void gather_rows_tab(asmg_s& h, double* const* tab, double* dst, cudaStream_t s);
+void scatter_rows_tab(asmg_s& h, const double* src, double* const* tab, cudaStream_t s);
 void run_solve_multi(asmg_s& h, MultiSlot& S, double rtol, cudaStream_t s);
 cudaGraphNode_t capture_solve_multi(asmg_s& h, MultiSlot& S, double rtol, cudaGraph_t g, const cudaGraphNode_t* deps,
                                     size_t ndeps);
 // assemble.cu
 HostCSR assemble_mesh(int dim, int64_t ne, const double* dX, const int32_t* dE, const int32_t* dFree,
                       const double* dCoef, int64_t nfree, cudaStream_t s);
-void mass_apply_gpu(int dim, int64_t nv, const int64_t* v2e_ptr, const int32_t* v2e, const double* dX,
-                    const int32_t* dE, const double* df, double* db, cudaStream_t s);
-void element_grad_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, const double* du, const double* dl,
+void element_mass_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, double* w, cudaStream_t s);
+void mass_apply_gpu(int dim, int64_t nv, const int64_t* v2e_ptr, const int32_t* v2e, const double* w,
+                    const int32_t* dE, const int32_t* row_of_vertex, const double* df, double* db, cudaStream_t s);
+void element_stiffness_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, double* K, cudaStream_t s);
+void mask_pair(asmg_s& h, const double* u, const double* lambda, double* pair, cudaStream_t s);
+void element_grad_gpu(int dim, int64_t ne, const double* dX, const int32_t* dE, const double* K, const double* pair,
                       const double* dscale, double* dg, cudaStream_t s);
 }  // namespace asmg

@@ -68,19 +68,6 @@ void launch(bool pdl, void (*kern)(KArgs...), int64_t grid, int block, cudaStrea
   ASMG_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
 }
 
-template <class T, class X>
-__device__ __forceinline__ T sell_dot(int64_t row, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
-                                      const T* __restrict__ val, const X* x) {
-  const int64_t sl = row >> 5, lane = row & 31;
-  const int64_t b = __ldg(off + sl), w = (__ldg(off + sl + 1) - b) >> 5;
-  T s = 0;
-  for (int64_t k = 0; k < w; ++k) {
-    const int64_t e = b + (k << 5) + lane;
-    s += __ldg(val + e) * (T)x[__ldg(col + e)];
-  }
-  return s;
-}
-
 // Programmatic dependent launch: every solve kernel first loads what was
 // written at setup (matrix rows, index lists), then waits for the preceding
 // kernel (griddepcontrol.wait) and at once lets the next kernel launch

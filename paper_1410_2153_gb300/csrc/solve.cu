@@ -919,6 +919,24 @@ __global__ void k_gather(int64_t n, const int32_t* __restrict__ vrow, const doub
   dst[i] = v >= 0 ? src[v] : 0.0;
 }
 
+// the same with the vertex array's address in device memory (batched solves:
+// the graph stays, the caller's arrays change)
+__global__ void k_gather_tab1(int64_t n, const int32_t* __restrict__ vrow, double* const* __restrict__ tab,
+                              double* __restrict__ dst) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int32_t v = vrow[i];
+  dst[i] = v >= 0 ? tab[0][v] : 0.0;
+}
+
+__global__ void k_scatter_tab1(int64_t nv, const int32_t* __restrict__ rowv, const double* __restrict__ src,
+                               double* const* __restrict__ tab) {
+  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (v >= nv) return;
+  const int32_t r = rowv[v];
+  tab[0][v] = r >= 0 ? src[r] : 0.0;
+}
+
 template <class S>
 __global__ void k_scatter(int64_t nv, const int32_t* __restrict__ rowv, const S* __restrict__ src,
                           double* __restrict__ dst) {
@@ -1290,11 +1308,35 @@ void gather_rows(asmg_s& h, const double* vsrc, double* dst, cudaStream_t s) {
   ASMG_CUDA(cudaGetLastError());
 }
 
+void gather_rows_tab(asmg_s& h, double* const* tab, double* dst, cudaStream_t s) {
+  launch(false, k_gather_tab1, nblk(h.npad), TPB, s, h.npad, h.d_vertex_of_row.p, tab, dst);
+  ASMG_CUDA(cudaGetLastError());
+}
+
+void scatter_rows_tab(asmg_s& h, const double* src, double* const* tab, cudaStream_t s) {
+  launch(false, k_scatter_tab1, nblk(h.mesh.nv), TPB, s, h.mesh.nv, h.d_row_of_vertex.p, src, tab);
+  ASMG_CUDA(cudaGetLastError());
+}
+
 void scatter_rows(asmg_s& h, const void* src, bool src_float, double* vdst, cudaStream_t s) {
   if (src_float)
     launch(false, k_scatter<float>, nblk(h.mesh.nv), TPB, s, h.mesh.nv, h.d_row_of_vertex.p, (const float*)src, vdst);
   else
     launch(false, k_scatter<double>, nblk(h.mesh.nv), TPB, s, h.mesh.nv, h.d_row_of_vertex.p, (const double*)src, vdst);
+  ASMG_CUDA(cudaGetLastError());
+}
+
+// (u, lambda) of every vertex side by side, 0 at Dirichlet vertices
+__global__ void k_mask_pair(int64_t nv, const int32_t* __restrict__ rowv, const double* __restrict__ u,
+                            const double* __restrict__ lambda, double2* __restrict__ pair) {
+  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (v >= nv) return;
+  pair[v] = rowv[v] >= 0 ? make_double2(u[v], lambda[v]) : make_double2(0.0, 0.0);
+}
+
+void mask_pair(asmg_s& h, const double* u, const double* lambda, double* pair, cudaStream_t s) {
+  launch(false, k_mask_pair, nblk(h.mesh.nv), TPB, s, h.mesh.nv, h.d_row_of_vertex.p, u, lambda,
+         reinterpret_cast<double2*>(pair));
   ASMG_CUDA(cudaGetLastError());
 }
 
@@ -1306,9 +1348,13 @@ void precond_apply(asmg_s& h, const double* r_perm, cudaStream_t s) {
     enqueue_precond<double>(h, S, r_perm, s);
 }
 
+// y = A x, a row's entries loaded into registers at once
 __global__ void k_spmv64(int64_t n, SellView<double> A, const double* __restrict__ x, double* __restrict__ y) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) y[i] = sell_dot<double, double>(i, A.off, A.col, A.val, x);
+  if (i >= n) return;
+  Row<double> row;
+  row_load(row, i, A.off, A.col, A.val);
+  y[i] = row_dot(row, A.col, A.val, x);
 }
 
 void spmv64(asmg_s& h, const double* x, double* y, cudaStream_t s) {

@@ -593,19 +593,19 @@ __global__ void k_axpy_norm_k(int64_t n, const double* __restrict__ p, const dou
   }
 }
 
-// vertex-major columns [KRHS][nv] <-> permuted interleaved rows [npad][KRHS]
-__global__ void k_gather_k(int64_t n, int64_t nv, const int32_t* __restrict__ vrow, const double* __restrict__ src,
-                           double* __restrict__ dst) {
+// vertex-major columns [k][nv] <-> permuted interleaved rows [npad][KRHS]
+__global__ void k_gather_k(int64_t n, int64_t nv, int k, const int32_t* __restrict__ vrow,
+                           const double* __restrict__ src, double* __restrict__ dst) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int32_t v = vrow[i];
   VK<double> o;
 #pragma unroll
-  for (int j = 0; j < K; ++j) o.v[j] = v >= 0 ? src[(int64_t)j * nv + v] : 0.0;
+  for (int j = 0; j < K; ++j) o.v[j] = v >= 0 && j < k ? src[(int64_t)j * nv + v] : 0.0;
   stk<double>(dst + i * K, o);
 }
 
-__global__ void k_scatter_k(int64_t nv, const int32_t* __restrict__ rowv, const double* __restrict__ src,
+__global__ void k_scatter_k(int64_t nv, int k, const int32_t* __restrict__ rowv, const double* __restrict__ src,
                             double* __restrict__ dst) {
   const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (v >= nv) return;
@@ -613,11 +613,42 @@ __global__ void k_scatter_k(int64_t nv, const int32_t* __restrict__ rowv, const 
   if (r >= 0) {
     const VK<double> x = ldk<double>(src + (int64_t)r * K);
 #pragma unroll
-    for (int j = 0; j < K; ++j) dst[(int64_t)j * nv + v] = x.v[j];
+    for (int j = 0; j < K; ++j)
+      if (j < k) dst[(int64_t)j * nv + v] = x.v[j];
   } else {
 #pragma unroll
-    for (int j = 0; j < K; ++j) dst[(int64_t)j * nv + v] = 0.0;
+    for (int j = 0; j < K; ++j)
+      if (j < k) dst[(int64_t)j * nv + v] = 0.0;
   }
+}
+
+// the same through a table of K vertex arrays (NULL: an unused column)
+__global__ void k_gather_tab(int64_t n, const int32_t* __restrict__ vrow, double* const* __restrict__ tab,
+                             double* __restrict__ dst) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int32_t v = vrow[i];
+  VK<double> o;
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    const double* src = tab[j];
+    o.v[j] = v >= 0 && src ? src[v] : 0.0;
+  }
+  stk<double>(dst + i * K, o);
+}
+
+__global__ void k_scatter_tab(int64_t nv, const int32_t* __restrict__ rowv, const double* __restrict__ src,
+                              double* const* __restrict__ tab) {
+  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (v >= nv) return;
+  const int32_t r = rowv[v];
+  VK<double> x;
+#pragma unroll
+  for (int j = 0; j < K; ++j) x.v[j] = 0;
+  if (r >= 0) x = ldk<double>(src + (int64_t)r * K);
+#pragma unroll
+  for (int j = 0; j < K; ++j)
+    if (tab[j]) tab[j][v] = x.v[j];
 }
 
 // --------------------------------------------------------- enqueueing
@@ -843,13 +874,23 @@ MultiSlot& add_multi_slot(asmg_s& h, cudaStream_t s) {
   return S;
 }
 
-void gather_multi(asmg_s& h, const double* vsrc, double* dst, cudaStream_t s) {
-  launch(false, k_gather_k, nblk(h.npad), TPB, s, h.npad, h.mesh.nv, h.d_vertex_of_row.p, vsrc, dst);
+void gather_multi(asmg_s& h, const double* vsrc, int k, double* dst, cudaStream_t s) {
+  launch(false, k_gather_k, nblk(h.npad), TPB, s, h.npad, h.mesh.nv, k, h.d_vertex_of_row.p, vsrc, dst);
   ASMG_CUDA(cudaGetLastError());
 }
 
-void scatter_multi(asmg_s& h, const double* src, double* vdst, cudaStream_t s) {
-  launch(false, k_scatter_k, nblk(h.mesh.nv), TPB, s, h.mesh.nv, h.d_row_of_vertex.p, src, vdst);
+void scatter_multi(asmg_s& h, const double* src, int k, double* vdst, cudaStream_t s) {
+  launch(false, k_scatter_k, nblk(h.mesh.nv), TPB, s, h.mesh.nv, k, h.d_row_of_vertex.p, src, vdst);
+  ASMG_CUDA(cudaGetLastError());
+}
+
+void gather_multi_tab(asmg_s& h, double* const* tab, double* dst, cudaStream_t s) {
+  launch(false, k_gather_tab, nblk(h.npad), TPB, s, h.npad, h.d_vertex_of_row.p, tab, dst);
+  ASMG_CUDA(cudaGetLastError());
+}
+
+void scatter_multi_tab(asmg_s& h, const double* src, double* const* tab, cudaStream_t s) {
+  launch(false, k_scatter_tab, nblk(h.mesh.nv), TPB, s, h.mesh.nv, h.d_row_of_vertex.p, src, tab);
   ASMG_CUDA(cudaGetLastError());
 }
 
