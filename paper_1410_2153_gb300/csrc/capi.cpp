@@ -1590,6 +1590,7 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
   }
   if (res_history) ASMG_CUDA(cudaStreamSynchronize(s));
   if (worst == ASMG_ERR_BREAKDOWN) g_err = "PCG breakdown in a column of a multiple solve";
+  if (worst == ASMG_ERR_TIMEOUT) g_err = "a bounded device wait expired in a multiple solve";
   return worst;
   API_END
 }

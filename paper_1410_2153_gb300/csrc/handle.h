@@ -106,6 +106,7 @@ template <class T>
 struct MultiPrec {
   DBuf<T> uf, rho, F, U;                  // [rows][KRHS]
   std::vector<DBuf<T>> fs, us;            // per level [nsm][KRHS]
+  std::vector<DBuf<T>> ust, fsl;          // per level with tiled post-sweeps [nloc][KRHS]
   DBuf<T> deep_fs, deep_us, bot_fs, bot_us;  // the same for the levels of the fused runs
 };
 
@@ -141,6 +142,7 @@ struct asmg_s {
   asmg::DBuf<double> d_elem_stiff;  // element stiffness for a = 1 (see element_stiffness_gpu), for the gradients
   bool elem_stiff_tried = false;    // its allocation was tried (without it the gradients recompute it)
   asmg::DBuf<double> d_pair;        // [nv][2] u and lambda, for the gradients
+  std::vector<uint8_t> sched;       // per level the tiled directions the autotuner chose (1 down, 2 up)
   asmg::PinnedBuf pinned;           // what a call reads back from the device
   asmg::TreeResult tree;
   asmg::AuxHost aux;

@@ -393,9 +393,8 @@ struct TileSweeps {
   DBuf<int64_t> pos_ptr;         // [nsm + 1]
   DBuf<int32_t> pos;             // positions in [0, nloc)
   TileView<T> view() const { return TileView<T>{head.p, blob.p, ntiles}; }
-  // values (rows and outside values), then the block
-  int64_t smem_values() const { return ((int64_t)(slots * TILE_THREADS + maxext) * (int64_t)sizeof(T) + 15) / 16 * 16; }
-  size_t smem() const { return (size_t)(smem_values() + maxblob); }
+  // shared memory of a launch with one column: values (rows and outside values), then the block
+  int64_t smem() const { return ((int64_t)(slots * TILE_THREADS + maxext) * (int64_t)sizeof(T) + 127) / 128 * 128 + maxblob; }
 };
 
 // The exact near-boundary solve of Algorithm 3 on the device: the block

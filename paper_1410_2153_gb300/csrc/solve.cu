@@ -29,6 +29,7 @@
 #include "handle.h"
 #include "kernels.h"
 #include "small_run.h"
+#include "tiles.h"
 
 namespace asmg {
 
@@ -271,339 +272,6 @@ __global__ void k_coarse(int64_t nc, const int32_t* __restrict__ cid, const doub
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) U[cid[row]] = (T)s;
   }
-}
-
-// ------------------------------------------- tiled sweeps (one launch each)
-// One thread block per tile (see TileSweeps), a persistent grid over the
-// tiles: the tile's rows -- its own rows of N~_l plus the halo its sweeps read
-// -- are held in registers for all nu sweeps, one row per slot and thread; the
-// rows' values live in shared memory and the colour phases are separated by
-// __syncthreads.  A tile's block of setup data arrives by one bulk copy
-// (cp.async.bulk, completion on an mbarrier): the first before the wait on the
-// previous kernel, each further one while the block sweeps the tile before.
-// Each row is updated with the same arithmetic, over the same stored entries
-// in the same order, as k_gs_aux_down / k_gs_aux do; the entries a tile leaves
-// out are exactly those whose value cannot reach the tile's own rows' results,
-// so those results equal the class-by-class launches bit for bit.  Halo
-// results are discarded.
-//
-// What bounds them is instructions and waits per colour phase, not the bytes:
-// with the rows read from shared memory entry by entry a level of 3.46 M rows
-// in five classes (graded 2049^2, BF16) took 118 us a direction at 18% of the
-// DRAM rate; with the rows in registers, no test per entry and four blocks per
-// SM it takes 78 us (graded 2049^2 solve 254.7 -> 231.6 ms, graded 513^2 FP64
-// 40.3 -> 38.2 ms, 331^2 mixed 2.04 -> 1.98 ms).
-
-// bound on the wait for a bulk copy (SM clock cycles, about 1 s): when it
-// expires the block records the timeout, waits once more (bounded) for its
-// copy to land, and ends
-constexpr long long TILE_WAIT_CYCLES = 2000000000LL;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// bounded wait for the mbarrier's phase of the given parity
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > TILE_WAIT_CYCLES) return false;
-  return true;
-}
-
-// one thread: arm the barrier and start the copy of a tile's block; the block's
-// earlier reads of the same shared memory came before a __syncthreads
-__device__ __forceinline__ void tile_fetch(void* dst, const unsigned char* blob, const TileHead& h, uint64_t* bar) {
-  const uint32_t b = smem_addr(bar);
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"((uint32_t)h.bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_addr(dst)),
-               "l"(blob + h.off), "r"((uint32_t)h.bytes), "r"(b)
-               : "memory");
-}
-
-__device__ __forceinline__ void tile_bar_init(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// Every thread waits for the copy (bounded): false in every thread when any
-// thread's wait expired.  inject != 0 (failure injection, asmg_params::
-// inject_timeout) takes the expired path without polling.
-__device__ __forceinline__ bool tile_arrived(uint64_t* bar, uint32_t parity, int inject) {
-  return __syncthreads_and(!inject && mbar_wait_bounded(smem_addr(bar), parity));
-}
-
-// after an expired wait: record it and give the copy a second bounded wait
-// before the block ends
-__device__ __forceinline__ void tile_expired(uint64_t* bar, uint32_t parity, int* timeout) {
-  if (threadIdx.x == 0) atomicExch(timeout, 1);
-  mbar_wait_bounded(smem_addr(bar), parity);
-  __syncthreads();
-}
-
-// The entries of one row (up to W) in registers, and its product with the
-// values in shared memory at `u`, summed in stored order.  Entries beyond the
-// slice's width are zeros at offset 0 (their products leave the sum as it is),
-// so the common widths run without a test per entry: a test, its branch and
-// their waits cost more than the multiply-add.
-// A0: entries multiplied whatever the width; the rest in groups of two.
-template <class T, class V, int W>
-struct TileRow {
-  uint32_t c[(W + 1) / 2];
-  T v[W];
-  __device__ __forceinline__ void load(const uint32_t* words, const T* val, const TileSlice& h, int lane) {
-#pragma unroll
-    for (int e = 0; e < (W + 1) / 2; ++e) c[e] = 2 * e < h.w ? words[(h.words + e) * 32 + lane] : 0u;
-#pragma unroll
-    for (int e = 0; e < W; ++e) v[e] = e < h.w ? val[(h.vals + e) * 32 + lane] : (T)0;
-  }
-  __device__ __forceinline__ T term(const char* u, int e, T acc) const {
-    return acc + v[e] * *reinterpret_cast<const T*>(u + ((e & 1) ? c[e / 2] >> 16 : c[e / 2] & 0xffffu));
-  }
-};
-template <class T, int W>
-struct TileRow<T, bf16v, W> {
-  uint32_t c[W];
-  __device__ __forceinline__ void load(const uint32_t* words, const T*, const TileSlice& h, int lane) {
-#pragma unroll
-    for (int e = 0; e < W; ++e) c[e] = e < h.w ? words[(h.words + e) * 32 + lane] : 0u;
-  }
-  __device__ __forceinline__ T term(const char* u, int e, T acc) const {
-    return acc + (T)__uint_as_float(c[e] & 0xffff0000u) * *reinterpret_cast<const T*>(u + (c[e] & 0xffffu));
-  }
-};
-template <class T, class V, int W>
-__device__ __forceinline__ T tile_dot(const TileRow<T, V, W>& row, const char* u, int w) {
-  constexpr int A0 = W <= 8 ? 6 : 8;
-  T acc = 0;
-#pragma unroll
-  for (int e = 0; e < A0; ++e) acc = row.term(u, e, acc);
-#pragma unroll
-  for (int e = A0; e < W; e += 2)
-    if (w > e) {
-      acc = row.term(u, e, acc);
-      acc = row.term(u, e + 1, acc);
-    }
-  return acc;
-}
-
-// the thread's rows of a tile, from the staged block
-template <class T, class V, int S, int W>
-struct TileRows {
-  int wc[S];        // slice: width | colour class << 8 (-1 << 8: empty)
-  TileRow<T, V, W> row[S];
-  T di[S];
-  int32_t g[S], ax[S];  // SM row (own k, halo -2 - k, padding -1), aux ID
-  __device__ __forceinline__ void load(const unsigned char* blob, const TileHead& h, const TileLayout& lay) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const TileSlice* hdr = reinterpret_cast<const TileSlice*>(blob);
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      wc[s] = -256;
-      g[s] = -1;
-      if (s < h.slots) {
-        const TileSlice sl = hdr[s * TILE_WARPS + warp];
-        wc[s] = sl.w | (int)sl.colour << 8;
-        row[s].load(reinterpret_cast<const uint32_t*>(blob + lay.words), reinterpret_cast<const T*>(blob + lay.val), sl,
-                    lane);
-        di[s] = reinterpret_cast<const T*>(blob + lay.dinv)[s * TILE_THREADS + tid];
-        g[s] = reinterpret_cast<const int32_t*>(blob + lay.lsm)[s * TILE_THREADS + tid];
-        ax[s] = reinterpret_cast<const int32_t*>(blob + lay.laux)[s * TILE_THREADS + tid];
-      }
-    }
-  }
-  // one colour phase: u += (f - A u) / a_ii on the thread's rows of class c
-  __device__ __forceinline__ void phase(int c, T* Ul, const T (&f)[S], T (&u)[S]) const {
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-      if (wc[s] >> 8 == c) {
-        const T acc = tile_dot(row[s], reinterpret_cast<const char*>(Ul), wc[s] & 255);
-        u[s] += (f[s] - acc) * di[s];
-        Ul[s * TILE_THREADS + threadIdx.x] = u[s];
-      }
-  }
-};
-
-// blocks per SM the kernels are compiled for: the most whose registers hold the
-// rows (a few spilled words cost less than a fourth block gives, BF16: level of
-// 3.46 M rows 115 us with three blocks, 80 us with four)
-template <class T, class V, int S, int W>
-constexpr int tile_min_blocks() {
-  if (sizeof(T) == 8) return W > 8 ? (S > 2 ? 1 : 2) : S > 2 ? 2 : 3;
-  return W > 8 ? 2 : S == 4 && !std::is_same<V, bf16v>::value ? 3 : 4;
-}
-
-// pre-sweeps: us (the level's own correction, SM order) starts at 0; the
-// first sweep saves F on the tile's own rows in fs
-template <class T, class V, int S, int W>
-__global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W>())
-    k_tile_down(TileView<T> t, int ncol, int64_t vals, const T* __restrict__ F, T* __restrict__ fs,
-                T* __restrict__ us, int nu, int* timeout, int inject) {
-  extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ __align__(8) uint64_t bar;
-  T* Ul = reinterpret_cast<T*>(smraw);
-  unsigned char* blob = smraw + vals;
-  const int tid = threadIdx.x;
-  int64_t tile = blockIdx.x;
-  TileHead h = t.head[tile];
-  if (tid == 0) {
-    tile_bar_init(&bar);
-    tile_fetch(blob, t.blob, h, &bar);
-  }
-  __syncthreads();  // the barrier is initialised before any thread polls it
-  // the first tile's rows are in registers before the wait on the previous kernel
-  TileRows<T, V, S, W> R;
-  uint32_t parity = 0;
-  bool ok = tile_arrived(&bar, parity, inject);
-  if (ok) R.load(blob, h, tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T)));
-  pdl_wait();
-  while (ok) {
-    T f[S], u[S];
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      f[s] = R.g[s] != -1 ? F[R.ax[s]] : (T)0;
-      u[s] = 0;
-      Ul[s * TILE_THREADS + tid] = 0;
-    }
-    const uint32_t mask = h.cmask;
-    tile += gridDim.x;
-    const bool more = tile < t.ntiles;
-    if (more) h = t.head[tile];
-    __syncthreads();  // values in place, the block read by all
-    if (tid == 0 && more) tile_fetch(blob, t.blob, h, &bar);
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-      if (R.g[s] >= 0) fs[R.g[s]] = f[s];
-    for (int sw = 0; sw < nu; ++sw)
-      for (int c = 0; c < ncol; ++c) {
-        if (!((mask >> min(c, 31)) & 1u)) continue;  // no row of this class in the tile
-        R.phase(c, Ul, f, u);
-        __syncthreads();
-      }
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-      if (R.g[s] >= 0) us[R.g[s]] = u[s];
-    if (!more) return;
-    parity ^= 1;
-    ok = tile_arrived(&bar, parity, inject);
-    if (ok) R.load(blob, h, tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T)));
-  }
-  tile_expired(&bar, parity, timeout);
-}
-
-// start of the up path of a tiled level: the prolongation of the coarse
-// correction (I_l: new nodes take the mean of their parents) plus the level's
-// saved correction, and the saved rhs, written for every SM row to each place
-// the row holds in the post-sweep tiles (own and halo copies; TileSweeps::
-// pos).  U itself is not written, so the tiles can read their start values
-// while other tiles write their results to U.
-template <class T>
-__global__ void k_up_init(int64_t nsm, const int32_t* __restrict__ rows, const int32_t* __restrict__ par0,
-                          const int32_t* __restrict__ par1, const int64_t* __restrict__ pos_ptr,
-                          const int32_t* __restrict__ pos, const T* __restrict__ U, const T* __restrict__ us,
-                          const T* __restrict__ fs, T* __restrict__ ust, T* __restrict__ fsl) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int32_t i = -1, a = -3, b = -3;
-  int64_t p0 = 0, p1 = 0;
-  if (k < nsm) {
-    i = rows[k];
-    a = par0[k];
-    b = par1[k];
-    p0 = pos_ptr[k];
-    p1 = pos_ptr[k + 1];
-  }
-  pdl_wait();
-  if (i >= 0) {
-    T v;
-    if (a == -3) {
-      v = U[i];
-    } else {
-      T p = 0;
-      if (a >= 0) p += U[a];
-      if (b >= 0) p += U[b];
-      v = (T)0.5 * p;
-    }
-    v = v + us[k];
-    const T f = fs[k];
-    for (int64_t q = p0; q < p1; ++q) {
-      const int32_t o = pos[q];
-      ust[o] = v;
-      fsl[o] = f;
-    }
-  }
-}
-
-// post-sweeps (backward colour order) from the start values and saved rhs
-// that k_up_init wrote in tile order (`per` local rows a tile); the columns
-// outside N~_l (the tile's outside values) are read from U once; the tile's
-// own rows are written to U
-template <class T, class V, int S, int W>
-__global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W>())
-    k_tile_up(TileView<T> t, int ncol, int64_t vals, const T* __restrict__ ust, const T* __restrict__ fsl, T* U,
-              int nu, int* timeout, int inject) {
-  extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ __align__(8) uint64_t bar;
-  T* Ul = reinterpret_cast<T*>(smraw);
-  unsigned char* blob = smraw + vals;
-  const int tid = threadIdx.x;
-  int64_t tile = blockIdx.x;
-  TileHead h = t.head[tile];
-  if (tid == 0) {
-    tile_bar_init(&bar);
-    tile_fetch(blob, t.blob, h, &bar);
-  }
-  __syncthreads();  // the barrier is initialised before any thread polls it
-  // the first tile's rows are in registers before the wait on the previous kernel
-  TileRows<T, V, S, W> R;
-  TileLayout lay = tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T));
-  uint32_t parity = 0;
-  bool ok = tile_arrived(&bar, parity, inject);
-  if (ok) R.load(blob, h, lay);
-  pdl_wait();
-  while (ok) {
-    const int64_t base = tile * (S * TILE_THREADS) + tid;
-    T f[S], u[S];
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      u[s] = ust[base + s * TILE_THREADS];
-      f[s] = fsl[base + s * TILE_THREADS];
-    }
-    const int32_t* ext = reinterpret_cast<const int32_t*>(blob + lay.ext);
-    for (int e = tid; e < h.nx; e += TILE_THREADS) Ul[S * TILE_THREADS + e] = U[ext[e]];
-#pragma unroll
-    for (int s = 0; s < S; ++s) Ul[s * TILE_THREADS + tid] = u[s];
-    const uint32_t mask = h.cmask;
-    tile += gridDim.x;
-    const bool more = tile < t.ntiles;
-    if (more) h = t.head[tile];
-    __syncthreads();  // values in place, the block read by all
-    if (tid == 0 && more) tile_fetch(blob, t.blob, h, &bar);
-    for (int sw = 0; sw < nu; ++sw)
-      for (int c = ncol - 1; c >= 0; --c) {
-        if (!((mask >> min(c, 31)) & 1u)) continue;
-        R.phase(c, Ul, f, u);
-        __syncthreads();
-      }
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-      if (R.g[s] >= 0) U[R.ax[s]] = u[s];
-    if (!more) return;
-    lay = tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T));
-    parity ^= 1;
-    ok = tile_arrived(&bar, parity, inject);
-    if (ok) R.load(blob, h, lay);
-  }
-  tile_expired(&bar, parity, timeout);
 }
 
 // ------------------------------------------- near-boundary solve (Alg. 3)
@@ -1019,21 +687,6 @@ int64_t small_bytes(const SmallRun<T>& R, bool down) {
   return (down ? R.v.bytes : R.v.up_bytes) + 2 * sz * (R.v.nunion + R.v.nsm);
 }
 
-// f(slots, width) with the tile kernel's compile-time sizes for a level's tiles
-template <class T, class V, class F>
-void tile_dispatch(const TileSweeps<T>& Tl, F f) {
-  auto by_width = [&](auto sl) {
-    if (Tl.width <= 8)
-      f(sl, std::integral_constant<int, 8>{});
-    else
-      f(sl, std::integral_constant<int, TILE_MAXW>{});
-  };
-  if (Tl.slots == 1) by_width(std::integral_constant<int, 1>{});
-  if (Tl.slots == 2) by_width(std::integral_constant<int, 2>{});
-  if (Tl.slots == 3) by_width(std::integral_constant<int, 3>{});
-  if (Tl.slots == 4) by_width(std::integral_constant<int, 4>{});
-}
-
 // the slot's timeout flag (PcgScalars::timeout, device memory)
 int* timeout_flag(Slot& S) {
   return reinterpret_cast<int*>(reinterpret_cast<char*>(S.scal.p) + offsetof(PcgScalars, timeout));
@@ -1064,13 +717,8 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
       const TileSweeps<T>& Tl = L.tdown;
       const int64_t by = Tl.nnz_real * (sv + 2) + (Tl.interior + Tl.halo) * (8 + 2 * sz) + Tl.interior * (4 + sz);
       LAUNCH(ASMG_PROF_AUX_GS, by,
-             tile_dispatch<T, V>(Tl, [&](auto sl, auto w) {
-               constexpr int SL = decltype(sl)::value, W = decltype(w)::value;
-               launch_smem(h.prm.use_pdl, k_tile_down<T, V, SL, W>,
-                           std::min<int64_t>(Tl.ntiles, NSM * tile_min_blocks<T, V, SL, W>()), TILE_THREADS, Tl.smem(), s,
-                           Tl.view(), L.ncolours, Tl.smem_values(), (const T*)SP.F.p, SP.fs[li].p, SP.us[li].p, npre,
-                           timeout_flag(S), h.prm.inject_timeout);
-             }));
+             (tiles::launch_down<T, V, 1>(h.prm.use_pdl, Tl, L.ncolours, SP.F.p, SP.fs[li].p, SP.us[li].p, npre,
+                                          timeout_flag(S), h.prm.inject_timeout, s)));
       ++launches;
     }
     // pre-sweeps on us (SM order); the first also saves F on N~_l for the
@@ -1121,18 +769,13 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
       LAUNCH(ASMG_PROF_AUX_TRANSFER,
              L.nsm_real * (28 + 3 * sz) + L.nnew * 2 * sz + (L.nsm_real - L.nnew) * sz +
                  (Tl.interior + Tl.halo) * (4 + 2 * sz),
-             launch(h.prm.use_pdl, k_up_init<T>, nblk(L.nsm, rows_tpb(L.nsm)), rows_tpb(L.nsm), s, L.nsm, L.sm_rows.p,
+             launch(h.prm.use_pdl, tiles::k_up_init<T, 1>, nblk(L.nsm, rows_tpb(L.nsm)), rows_tpb(L.nsm), s, L.nsm, L.sm_rows.p,
                     L.sm_par0.p, L.sm_par1.p, Tl.pos_ptr.p, Tl.pos.p, (const T*)SP.U.p, (const T*)SP.us[li].p,
                     (const T*)SP.fs[li].p, SP.ust[li].p, SP.fsl[li].p));
       const int64_t by = Tl.nnz_real * (sv + 2) + (Tl.interior + Tl.halo) * (8 + 3 * sz) + Tl.interior * (4 + sz);
       LAUNCH(ASMG_PROF_AUX_GS, by,
-             tile_dispatch<T, V>(Tl, [&](auto sl, auto w) {
-               constexpr int SL = decltype(sl)::value, W = decltype(w)::value;
-               launch_smem(h.prm.use_pdl, k_tile_up<T, V, SL, W>,
-                           std::min<int64_t>(Tl.ntiles, NSM * tile_min_blocks<T, V, SL, W>()), TILE_THREADS, Tl.smem(), s,
-                           Tl.view(), L.ncolours, Tl.smem_values(), (const T*)SP.ust[li].p, (const T*)SP.fsl[li].p,
-                           SP.U.p, npost, timeout_flag(S), h.prm.inject_timeout);
-             }));
+             (tiles::launch_up<T, V, 1>(h.prm.use_pdl, Tl, L.ncolours, SP.ust[li].p, SP.fsl[li].p, SP.U.p, npost,
+                                        timeout_flag(S), h.prm.inject_timeout, s)));
       launches += 2;
       continue;
     }
@@ -1493,18 +1136,7 @@ void setup_small(Prec<T>& P, bool bf16, cudaStream_t s) {
   auto attrs = [&](auto vtag) {
     using V = decltype(vtag);
     small::set_smem_limits<T, V, 1>();
-    for (int slots = 1; slots <= TILE_SLOTS_MAX; ++slots)
-      for (int width : {8, TILE_MAXW}) {
-        TileSweeps<T> Tl;
-        Tl.slots = slots;
-        Tl.width = width;
-        tile_dispatch<T, V>(Tl, [&](auto sl, auto w) {
-          ASMG_CUDA(cudaFuncSetAttribute(k_tile_down<T, V, decltype(sl)::value, decltype(w)::value>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX));
-          ASMG_CUDA(cudaFuncSetAttribute(k_tile_up<T, V, decltype(sl)::value, decltype(w)::value>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX));
-        });
-      }
+    tiles::set_smem_limits<T, V, 1>();
   };
   attrs(T{});
   if constexpr (std::is_same<T, float>::value) attrs(bf16v{});
@@ -1564,6 +1196,11 @@ void alloc_slot_prec(asmg_s& h, Prec<T>& P, SlotPrec<T>& SP, cudaStream_t s) {
   for (DBuf<T>* v : {&SP.bot_fs, &SP.bot_us}) v->alloc(std::max(P.bot.v.nsm, 1));
 }
 
+// A level of at most this many tiles always runs them: they are one wave of
+// blocks, about the time of one or two of the class launches they replace
+// (level of 16,129 rows on graded 2049^2: 8 us against 4 launches a direction).
+constexpr int64_t TILE_ALWAYS = 2 * NSM;
+
 // Schedule of the auxiliary levels (the autotuner, tile_rows = 0): each
 // direction of a level that has tiles runs either its temporally blocked
 // sweeps or its launches per colour class and sweep, with the same results.
@@ -1571,8 +1208,7 @@ void alloc_slot_prec(asmg_s& h, Prec<T>& P, SlotPrec<T>& SP, cudaStream_t s) {
 // captured as a CUDA graph and timed (median of 3 runs of 5 launches) with
 // every level tiled both ways, then for each level in turn the post-sweeps
 // and then the pre-sweeps are switched to class launches, each switch kept
-// when it is faster by more than 0.5% (and 2 us).  Tiles of a direction left
-// untiled are freed.
+// when it is faster by more than 0.5% (and 2 us).
 template <class T>
 void autotune_levels(asmg_s& h, cudaStream_t s) {
   Prec<T>& P = prec<T>(h);
@@ -1580,7 +1216,7 @@ void autotune_levels(asmg_s& h, cudaStream_t s) {
   const int nlev = (int)P.lev.size();
   std::vector<int> cand;
   for (int li = P.bot.v.nlev; li <= nlev - 1 - P.deep.v.nlev; ++li)
-    if (P.lev[li].tiled) cand.push_back(li);
+    if (P.lev[li].tiled && std::max(P.lev[li].tdown.ntiles, P.lev[li].tup.ntiles) > TILE_ALWAYS) cand.push_back(li);
   if (cand.empty()) return;
   cudaStream_t cs;
   ASMG_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -1629,16 +1265,45 @@ void autotune_levels(asmg_s& h, cudaStream_t s) {
   ASMG_CUDA(cudaEventDestroy(e0));
   ASMG_CUDA(cudaEventDestroy(e1));
   ASMG_CUDA(cudaStreamDestroy(cs));
-  for (int li : cand) {
+}
+
+// Free the tiles of directions that run class launches.
+template <class T>
+void drop_untiled(asmg_s& h) {
+  Prec<T>& P = prec<T>(h);
+  SlotPrec<T>& SP = slotprec<T>(*h.slots[0]);
+  for (size_t li = 0; li < P.lev.size(); ++li) {
     AuxLevelDev<T>& L = P.lev[li];
+    if (!L.tiled) continue;
     if (!L.tiled_down) L.tdown = TileSweeps<T>();
     if (!L.tiled_up) {
       L.tup = TileSweeps<T>();
-      slotprec<T>(S).ust[li] = DBuf<T>();
-      slotprec<T>(S).fsl[li] = DBuf<T>();
+      SP.ust[li] = DBuf<T>();
+      SP.fsl[li] = DBuf<T>();
     }
     L.tiled = L.tiled_down || L.tiled_up;
   }
+}
+
+// The handle's schedule: measured when the handle is set up, kept when its
+// coefficients change (they change neither the grids nor the work of a launch).
+template <class T>
+void schedule_levels(asmg_s& h, cudaStream_t s) {
+  Prec<T>& P = prec<T>(h);
+  const size_t nlev = P.lev.size();
+  if (h.sched.size() != nlev) {
+    autotune_levels<T>(h, s);
+    h.sched.assign(nlev, 0);
+    for (size_t li = 0; li < nlev; ++li)
+      h.sched[li] = (uint8_t)((P.lev[li].tiled_down ? 1 : 0) | (P.lev[li].tiled_up ? 2 : 0));
+  } else {
+    for (size_t li = 0; li < nlev; ++li) {
+      AuxLevelDev<T>& L = P.lev[li];
+      L.tiled_down = L.tiled_down && (h.sched[li] & 1);
+      L.tiled_up = L.tiled_up && (h.sched[li] & 2);
+    }
+  }
+  drop_untiled<T>(h);
 }
 
 Slot& add_slot(asmg_s& h, cudaStream_t s) {
@@ -1694,9 +1359,9 @@ void setup_solve(asmg_s& h, cudaStream_t s) {
   add_slot(h, s);
   if (h.prm.tile_rows == 0 && !h.prm.inject_timeout) {
     if (h.prm.precision == ASMG_MIXED)
-      autotune_levels<float>(h, s);
+      schedule_levels<float>(h, s);
     else
-      autotune_levels<double>(h, s);
+      schedule_levels<double>(h, s);
   }
 }
 

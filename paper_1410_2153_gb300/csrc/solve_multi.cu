@@ -24,6 +24,7 @@
 #include "handle.h"
 #include "kernels.h"
 #include "small_run.h"
+#include "tiles.h"
 
 namespace asmg {
 
@@ -680,6 +681,18 @@ const double* fine_dinv_of<double>(asmg_s& h) { return h.dinv64.p; }
 template <>
 const float* fine_dinv_of<float>(asmg_s& h) { return h.p32.dinv_f.p; }
 
+int* timeout_flag_k(MultiSlot& S) {
+  return reinterpret_cast<int*>(reinterpret_cast<char*>(S.scal.p) + offsetof(MultiScalars, timeout));
+}
+
+// Whether K columns run a direction's tiles.  In FP64 the columns' values of
+// more than two slots leave one block per SM: those levels keep their class
+// launches.
+template <class T>
+bool tiles_fit(const TileSweeps<T>& Tl) {
+  return tiles::Smem<T>(Tl, K).total <= tiles::SMEM_MAX_K && !(sizeof(T) == 8 && Tl.slots > 2);
+}
+
 // V: how the auxiliary-level matrices are read (T, or bf16v with level_bf16)
 template <class T, class V>
 void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
@@ -693,7 +706,11 @@ void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
   for (int li = nlev - 1 - ndeep; li >= nbot; --li) {
     AuxLevelDev<T>& L = P.lev[li];
     auto SMd = view(L.SMd);
-    for (int sweep = 0; sweep < npre; ++sweep)
+    const bool tiled = L.tiled_down && tiles_fit(L.tdown);
+    if (tiled)
+      tiles::launch_down<T, V, K>(pdl, L.tdown, L.ncolours, M.F.p, M.fs[li].p, M.us[li].p, npre, timeout_flag_k(S),
+                                  h.prm.inject_timeout, s);
+    for (int sweep = 0; sweep < (tiled ? 0 : npre); ++sweep)
       for (int c = 0; c < L.ncolours; ++c) {
         const int64_t k0 = L.cstart[c], nk = L.cstart[c + 1] - L.cstart[c];
         if (!nk) continue;
@@ -713,6 +730,15 @@ void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
   for (int li = nbot; li <= nlev - 1 - ndeep; ++li) {
     AuxLevelDev<T>& L = P.lev[li];
     auto SM = view(L.SM);
+    if (L.tiled_up && tiles_fit(L.tup)) {
+      const TileSweeps<T>& Tl = L.tup;
+      launch(pdl, tiles::k_up_init<T, K>, nblk(L.nsm, rows_tpb(L.nsm)), rows_tpb(L.nsm), s, L.nsm, L.sm_rows.p,
+             L.sm_par0.p, L.sm_par1.p, Tl.pos_ptr.p, Tl.pos.p, (const T*)M.U.p, (const T*)M.us[li].p,
+             (const T*)M.fs[li].p, M.ust[li].p, M.fsl[li].p);
+      tiles::launch_up<T, V, K>(pdl, Tl, L.ncolours, M.ust[li].p, M.fsl[li].p, M.U.p, npost, timeout_flag_k(S),
+                                h.prm.inject_timeout, s);
+      continue;
+    }
     if (L.nnew)
       launch(pdl, k_prolong_aux_k<T>, nblk(L.nnew, rows_tpb(L.nnew)), rows_tpb(L.nnew), s, L.nnew, L.nn_id.p,
              L.nn_p0.p, L.nn_p1.p, M.U.p);
@@ -817,16 +843,30 @@ void alloc_multi_prec(asmg_s& h, MultiPrec<T>& M, cudaStream_t s) {
   M.us.clear();
   M.fs.resize(nlev);
   M.us.resize(nlev);
+  M.ust.clear();
+  M.fsl.clear();
+  M.ust.resize(nlev);
+  M.fsl.resize(nlev);
   for (int li = 0; li < nlev; ++li) {
     M.fs[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1) * K);
     M.us[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1) * K);
     M.fs[li].zero(s);
     M.us[li].zero(s);
+    if (P.lev[li].tiled_up && tiles_fit(P.lev[li].tup)) {
+      M.ust[li].alloc(std::max<int64_t>(P.lev[li].tup.nloc, 1) * K);
+      M.fsl[li].alloc(std::max<int64_t>(P.lev[li].tup.nloc, 1) * K);
+      M.ust[li].zero(s);
+      M.fsl[li].zero(s);
+    }
   }
   for (DBuf<T>* v : {&M.deep_fs, &M.deep_us}) v->alloc(std::max(P.deep_k.v.nsm, 1) * K);
   for (DBuf<T>* v : {&M.bot_fs, &M.bot_us}) v->alloc(std::max(P.bot_k.v.nsm, 1) * K);
   small::set_smem_limits<T, T, K>();
-  if constexpr (std::is_same<T, float>::value) small::set_smem_limits<T, bf16v, K>();
+  tiles::set_smem_limits<T, T, K>();
+  if constexpr (std::is_same<T, float>::value) {
+    small::set_smem_limits<T, bf16v, K>();
+    tiles::set_smem_limits<T, bf16v, K>();
+  }
 }
 
 void build_graph_k(asmg_s& h, MultiSlot& S, double rtol) {
