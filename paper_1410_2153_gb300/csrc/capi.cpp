@@ -810,6 +810,47 @@ void build_prec(asmg_s& h, Prec<T>& P, const HostCSR& Aperm, const std::vector<d
     std::vector<T> d(dinv_perm.begin(), dinv_perm.end());
     P.dinv_f.upload(d, s);
   }
+  if (h.prm.smoother == 0 && h.prm.fine_sweeps == 1) {
+    // the halves of A the forward sweep from 0 and the residual after it read
+    const int ncol = (int)h.fine_cstart.size() - 1;
+    h.fine_lnnz.assign(ncol, 0);
+    auto half = [&](bool lower) {
+      HostCSR B;
+      B.nr = Aperm.nr;
+      B.nc = Aperm.nc;
+      B.ptr.assign(B.nr + 1, 0);
+      auto rows = [&](auto body) {
+        for (int c = 0; c < ncol; ++c) {
+          const int64_t r0 = h.fine_cstart[c], r1 = h.fine_cstart[c + 1];
+          host_for(r1 - r0, [&](int64_t a, int64_t b) {
+            for (int64_t i = r0 + a; i < r0 + b; ++i)
+              body(i, [&](int64_t p) { return lower ? Aperm.col[p] < r0 : Aperm.col[p] >= r1; });
+          });
+        }
+      };
+      rows([&](int64_t i, auto in) {
+        int64_t k = 0;
+        for (int64_t p = Aperm.ptr[i]; p < Aperm.ptr[i + 1]; ++p) k += in(p);
+        B.ptr[i + 1] = k;
+      });
+      for (int64_t i = 0; i < B.nr; ++i) B.ptr[i + 1] += B.ptr[i];
+      B.col.resize(B.ptr[B.nr]);
+      B.val.resize(B.ptr[B.nr]);
+      rows([&](int64_t i, auto in) {
+        int64_t q = B.ptr[i];
+        for (int64_t p = Aperm.ptr[i]; p < Aperm.ptr[i + 1]; ++p)
+          if (in(p)) {
+            B.col[q] = Aperm.col[p];
+            B.val[q++] = Aperm.val[p];
+          }
+      });
+      if (lower)
+        for (int c = 0; c < ncol; ++c) h.fine_lnnz[c] = B.ptr[h.fine_cstart[c + 1]] - B.ptr[h.fine_cstart[c]];
+      return B;
+    };
+    sell_build<T>(P.Lo, half(true), 0, s);
+    sell_build<T>(P.Up, half(false), 0, s);
+  }
   // transfer P (rows: permuted fine rows) and P^T (rows: aux nodes), built
   // by counting sort into flat CSR arrays; each row sorted by column
   const Triplets& Tp = h.aux.P;

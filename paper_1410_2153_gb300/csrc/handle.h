@@ -55,6 +55,7 @@ template <class T>
 struct Prec {
   Sell<T> Af;                  // fine smoother matrix (mixed mode only; FP64 mode uses A64)
   DBuf<T> dinv_f;
+  Sell<T> Lo, Up;              // the fine matrix's columns of earlier / later colour classes than the row's
   Sell<T> P, PT;               // Scott-Zhang transfer and its transpose
   std::vector<AuxLevelDev<T>> lev;  // levels c+1..J (index 0 = c+1)
   SmallRun<T> deep, bot;         // fused small-level runs (top of the hierarchy, bottom)
@@ -152,6 +153,7 @@ struct asmg_s {
   std::vector<int32_t> free_of_vertex, vertex_of_free, fine_colour, row_of_free;
   std::vector<int64_t> fine_cstart;      // colour blocks in permuted rows (multiples of 32)
   std::vector<int64_t> fine_cnnz, fine_crows;  // real non-zeros / rows per colour block
+  std::vector<int64_t> fine_lnnz;              // real non-zeros of Prec::Lo per colour block
   asmg::HostCSR A_host;                  // fine A, free-dof numbering (for export)
   asmg::Sell<double> A64;
   asmg::DBuf<double> dinv64;

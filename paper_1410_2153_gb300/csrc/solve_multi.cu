@@ -124,6 +124,50 @@ __global__ void k_gs_fine_k(int64_t r0, int64_t nrows, const int64_t* __restrict
   }
 }
 
+// the forward sweep from u = 0 and the residual after it, on the halves of A
+// (k_gs_first, k_resid_upper)
+template <class T>
+__global__ void k_gs_first_k(int64_t r0, int64_t nrows, const int64_t* __restrict__ off,
+                             const int32_t* __restrict__ col, const T* __restrict__ val, const T* __restrict__ dinv,
+                             const double* __restrict__ rhs, T* u) {
+  const int64_t i = r0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool act = i < r0 + nrows;
+  Row<T> row;
+  T di = 0;
+  if (act) {
+    row_load(row, i, off, col, val);
+    di = dinv[i];
+  }
+  pdl_wait();
+  if (act) {
+    T acc[K];
+    row_dot_k<T, T>(row, col, val, u, acc);
+    const VK<double> r = ldk<double>(rhs + i * K);
+    VK<T> ui;
+#pragma unroll
+    for (int j = 0; j < K; ++j) ui.v[j] = ((T)r.v[j] - acc[j]) * di;
+    stk<T>(u + i * K, ui);
+  }
+}
+
+template <class T>
+__global__ void k_resid_upper_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
+                                const T* __restrict__ val, const T* __restrict__ u, T* __restrict__ rho) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool act = i < n;
+  Row<T> row;
+  if (act) row_load(row, i, off, col, val);
+  pdl_wait();
+  if (act) {
+    T acc[K];
+    row_dot_k<T, T>(row, col, val, u, acc);
+    VK<T> o;
+#pragma unroll
+    for (int j = 0; j < K; ++j) o.v[j] = -acc[j];
+    stk<T>(rho + i * K, o);
+  }
+}
+
 template <class T>
 __global__ void k_resid_fine_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                                const T* __restrict__ val, const double* __restrict__ r, const T* __restrict__ u,
@@ -770,7 +814,7 @@ void enqueue_precond_k(asmg_s& h, MultiSlot& S, const double* r, cudaStream_t s)
   const SellView<T> A = fine_matrix<T>(h);
   const T* dinv = fine_dinv_of<T>(h);
   const bool pdl = h.prm.use_pdl;
-  ASMG_CUDA(cudaMemsetAsync(M.uf.p, 0, sizeof(T) * h.npad * K, s));
+  const bool split = h.prm.fine_sweeps == 1;
   const int ncol = (int)h.fine_cstart.size() - 1;
   auto smooth = [&](bool forward) {
     for (int m = 0; m < h.prm.fine_sweeps; ++m)
@@ -782,9 +826,25 @@ void enqueue_precond_k(asmg_s& h, MultiSlot& S, const double* r, cudaStream_t s)
                M.uf.p);
       }
   };
-  smooth(true);
+  if (split) {
+    auto Lo = view(P.Lo);
+    for (int c = 0; c < ncol; ++c) {
+      const int64_t r0 = h.fine_cstart[c], nr = h.fine_cstart[c + 1] - r0;
+      if (nr)
+        launch(pdl, k_gs_first_k<T>, nblk(nr, rows_tpb(nr)), rows_tpb(nr), s, r0, nr, Lo.off, Lo.col, Lo.val, dinv, r,
+               M.uf.p);
+    }
+  } else {
+    ASMG_CUDA(cudaMemsetAsync(M.uf.p, 0, sizeof(T) * h.npad * K, s));
+    smooth(true);
+  }
   if (h.nJ > 0) {
-    launch(pdl, k_resid_fine_k<T>, nblk(h.npad), TPB, s, h.npad, A.off, A.col, A.val, r, (const T*)M.uf.p, M.rho.p);
+    if (split) {
+      auto Up = view(P.Up);
+      launch(pdl, k_resid_upper_k<T>, nblk(h.npad), TPB, s, h.npad, Up.off, Up.col, Up.val, (const T*)M.uf.p, M.rho.p);
+    } else {
+      launch(pdl, k_resid_fine_k<T>, nblk(h.npad), TPB, s, h.npad, A.off, A.col, A.val, r, (const T*)M.uf.p, M.rho.p);
+    }
     auto PT = view(P.PT);
     launch(pdl, k_restrict_fine_k<T>, nblk(h.nJpad), TPB, s, h.nJpad, PT.off, PT.col, PT.val, (const T*)M.rho.p,
            M.F.p, M.U.p);
