@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -85,15 +86,31 @@ __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// A SELL-32 row held in registers (up to MAXW entries; longer rows read the rest later).
+// A SELL-32 row held in registers (up to N entries; longer rows read the rest later).
 constexpr int MAXW = 10;
-template <class T>
+template <class T, int N = MAXW>
 struct Row {
   int64_t b = 0, lane = 0;
   int w = 0;
-  int32_t c[MAXW];
-  T v[MAXW];
+  int32_t c[N];
+  T v[N];
 };
+
+// f(N) with the entries a row kernel holds per row.  A launch of one wave of
+// threads hides its latency by its loads in flight, one of several waves by its
+// occupancy, which the registers of a long row cost it: with 16 entries
+// throughout graded 2049^2 BF16 takes 256 ms, with 10 217.5, with 8 on launches
+// of several waves 211.6 (6 or 4 there: 212.2, 216.8; kuhn129 36.6 -> 35.7 ms);
+// with 6 throughout 331^2 mixed goes from 1.56 to 1.69 ms.
+constexpr int WIDE_W = 8;
+template <int SMALL = MAXW, class F>
+void by_rows(int64_t rows, F f) {
+  if (rows <= (int64_t)NSM * 2048)
+    f(std::integral_constant<int, SMALL>{});
+  else
+    f(std::integral_constant<int, WIDE_W>{});
+}
+constexpr int TRANSFER_W = 16;  // P and P^T rows of a small launch (10 entries on average in 2D, 15 in 3D)
 
 // Matrix values as stored (FP64, FP32 or BF16), widened to the arithmetic
 // type exactly; the ldg forms read through the read-only path, the ldcs forms
@@ -112,15 +129,15 @@ __device__ __forceinline__ double val_of(double v) { return v; }
 __device__ __forceinline__ float val_of(float v) { return v; }
 __device__ __forceinline__ float val_of(bf16v v) { return __uint_as_float((uint32_t)v.bits << 16); }
 
-template <class T, class V>
-__device__ __forceinline__ void row_load(Row<T>& R, int64_t row, const int64_t* __restrict__ off,
+template <class T, int N, class V>
+__device__ __forceinline__ void row_load(Row<T, N>& R, int64_t row, const int64_t* __restrict__ off,
                                          const int32_t* __restrict__ col, const V* __restrict__ val) {
   const int64_t sl = row >> 5;
   R.lane = row & 31;
   R.b = __ldg(off + sl);
   R.w = (int)((__ldg(off + sl + 1) - R.b) >> 5);
 #pragma unroll
-  for (int k = 0; k < MAXW; ++k)
+  for (int k = 0; k < N; ++k)
     if (k < R.w) {
       const int64_t e = R.b + ((int64_t)k << 5) + R.lane;
       R.c[k] = __ldcs(col + e);
@@ -128,14 +145,14 @@ __device__ __forceinline__ void row_load(Row<T>& R, int64_t row, const int64_t* 
     }
 }
 
-template <class T, class V, class X>
-__device__ __forceinline__ T row_dot(const Row<T>& R, const int32_t* __restrict__ col, const V* __restrict__ val,
+template <class T, int N, class V, class X>
+__device__ __forceinline__ T row_dot(const Row<T, N>& R, const int32_t* __restrict__ col, const V* __restrict__ val,
                                      const X* x) {
   T s = 0;
 #pragma unroll
-  for (int k = 0; k < MAXW; ++k)
+  for (int k = 0; k < N; ++k)
     if (k < R.w) s += R.v[k] * (T)x[R.c[k]];
-  for (int k = MAXW; k < R.w; ++k) {
+  for (int k = N; k < R.w; ++k) {
     const int64_t e = R.b + ((int64_t)k << 5) + R.lane;
     s += (T)ldg_val(val + e) * (T)x[__ldg(col + e)];
   }

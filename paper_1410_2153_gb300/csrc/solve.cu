@@ -39,12 +39,12 @@ using namespace kern;
 
 // ------------------------------------------------------------- fine grid
 // one colour of a Gauss-Seidel sweep: u_i += (rhs_i - (A u)_i) / a_ii
-template <class T, class R>
+template <class T, class R, int N>
 __global__ void k_gs_fine(int64_t r0, int64_t nrows, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                           const T* __restrict__ val, const T* __restrict__ dinv, const R* __restrict__ rhs, T* u) {
   const int64_t i = r0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool act = i < r0 + nrows;
-  Row<T> row;
+  Row<T, N> row;
   T di = 0;
   if (act) {
     row_load(row, i, off, col, val);
@@ -65,13 +65,13 @@ __global__ void k_gs_fine(int64_t r0, int64_t nrows, const int64_t* __restrict__
 // where a full sweep and a full residual read it twice, and the sweep needs no
 // cleared u.  With the first and last class's steps taken by the CG kernels:
 // 65^2 FP64 758 -> 718 us per solve, kuhn129 mixed 39.3 -> 36.6 ms.
-template <class T>
+template <class T, int N>
 __global__ void k_gs_first(int64_t r0, int64_t nrows, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                            const T* __restrict__ val, const T* __restrict__ dinv, const double* __restrict__ rhs,
                            T* u) {
   const int64_t i = r0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool act = i < r0 + nrows;
-  Row<T> row;
+  Row<T, N> row;
   T di = 0;
   if (act) {
     row_load(row, i, off, col, val);
@@ -84,12 +84,12 @@ __global__ void k_gs_first(int64_t r0, int64_t nrows, const int64_t* __restrict_
   }
 }
 
-template <class T>
+template <class T, int N>
 __global__ void k_resid_upper(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                               const T* __restrict__ val, const T* __restrict__ u, T* __restrict__ rho) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool act = i < n;
-  Row<T> row;
+  Row<T, N> row;
   if (act) row_load(row, i, off, col, val);
   pdl_wait();
   if (act) rho[i] = -row_dot(row, col, val, u);
@@ -109,13 +109,13 @@ __global__ void k_resid_fine(int64_t n, const int64_t* __restrict__ off, const i
 }
 
 // F = P^T rho on the auxiliary nodes, and U = 0 (start of the V-cycle)
-template <class T>
+template <class T, int N>
 __global__ void k_restrict_fine(int64_t nJ, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                                 const T* __restrict__ val, const T* __restrict__ rho, T* __restrict__ F,
                                 T* __restrict__ U) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool act = k < nJ;
-  Row<T> row;
+  Row<T, N> row;
   if (act) row_load(row, k, off, col, val);
   pdl_wait();
   if (act) {
@@ -125,12 +125,12 @@ __global__ void k_restrict_fine(int64_t nJ, const int64_t* __restrict__ off, con
 }
 
 // u += P U
-template <class T>
+template <class T, int N>
 __global__ void k_prolong_fine(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                                const T* __restrict__ val, const T* __restrict__ U, T* __restrict__ u) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool act = i < n;
-  Row<T> row;
+  Row<T, N> row;
   if (act) row_load(row, i, off, col, val);
   pdl_wait();
   if (act) u[i] += row_dot(row, col, val, U);
@@ -167,13 +167,13 @@ __global__ void k_cast_fine(int64_t n, const double* __restrict__ r, T* __restri
 // ------------------------------------------------------ auxiliary levels
 // one colour of an up (post-smoothing) sweep on the smoothing rows of a
 // level: U[i] += (fs_k - (A_l U)_i) / a_ii with the F saved on the way down
-template <class T, class V>
+template <class T, class V, int N>
 __global__ void k_gs_aux(int64_t k0, int64_t nk, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                          const V* __restrict__ val, const T* __restrict__ dinv, const int32_t* __restrict__ rows,
                          const T* __restrict__ fs, T* U) {
   const int64_t k = k0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int32_t i = -1;
-  Row<T> row;
+  Row<T, N> row;
   T di = 0;
   if (k < k0 + nk) {
     i = rows[k];
@@ -196,13 +196,13 @@ __global__ void k_gs_aux(int64_t k0, int64_t nk, const int64_t* __restrict__ off
 // later ones: only columns of earlier classes (below k0) are read, and the
 // class's rows are set rather than updated.  The first sweep takes F and
 // saves it in fs.
-template <class T, class V>
+template <class T, class V, int N>
 __global__ void k_gs_aux_down(int64_t k0, int64_t nk, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                               const V* __restrict__ val, const T* __restrict__ dinv, const int32_t* __restrict__ rows,
                               const T* __restrict__ F, int first, T* __restrict__ fs, T* us) {
   const int64_t k = k0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int32_t i = -1;
-  Row<T> row;
+  Row<T, N> row;
   T di = 0;
   if (k < k0 + nk) {
     i = rows[k];
@@ -218,9 +218,9 @@ __global__ void k_gs_aux_down(int64_t k0, int64_t nk, const int64_t* __restrict_
       f = F[i];
       fs[k] = f;
 #pragma unroll
-      for (int q = 0; q < MAXW; ++q)
+      for (int q = 0; q < N; ++q)
         if (q < row.w && row.c[q] < k0) acc += row.v[q] * us[row.c[q]];
-      for (int q = MAXW; q < row.w; ++q) {
+      for (int q = N; q < row.w; ++q) {
         const int64_t e = row.b + ((int64_t)q << 5) + row.lane;
         const int32_t c = __ldg(col + e);
         if (c < k0) acc += (T)ldg_val(val + e) * us[c];
@@ -235,13 +235,13 @@ __global__ void k_gs_aux_down(int64_t k0, int64_t nk, const int64_t* __restrict_
 }
 
 // F_i -= sum_{j in N~_l} a_ij U_j on the rows E_l
-template <class T, class V>
+template <class T, class V, int N>
 __global__ void k_resid_aux(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                             const V* __restrict__ val, const int32_t* __restrict__ rows, const T* __restrict__ U,
                             T* __restrict__ F) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int32_t i = -1;
-  Row<T> row;
+  Row<T, N> row;
   if (k < n) {
     i = rows[k];
     if (i >= 0) row_load(row, k, off, col, val);
@@ -539,10 +539,11 @@ __global__ void k_pupd(int64_t n, const T* __restrict__ z, double* __restrict__ 
 // q = A p, <p, q>  ->  alpha.  Each row's entries are loaded into registers
 // at once (row_load), the thread's first row before the wait on the previous
 // kernel (graded 2049^2: 3.1 -> 4.3 TB/s against a plain loop over the row).
+template <int N>
 __global__ void k_spmv_dot(int64_t n, SellView<double> A, const double* __restrict__ p, double* __restrict__ q,
                            double* partial, unsigned int* ticket, PcgScalars* sc) {
   const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
-  Row<double> row;
+  Row<double, N> row;
   if (i0 < n) row_load(row, i0, A.off, A.col, A.val);
   pdl_wait();
   double v[1] = {0};
@@ -793,16 +794,20 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
         if (!nk) continue;
         const int64_t by = L.cnnz_d[c] * (sv + 4) + L.crows[c] * (4 + (sweep == 0 ? 4 + 4 * sz : 4 * sz));
         LAUNCH(ASMG_PROF_AUX_GS, by,
-               launch(h.prm.use_pdl, k_gs_aux_down<T, V>, nblk(nk, rows_tpb(nk)), rows_tpb(nk), s, k0, nk, SMd.off,
+               (by_rows(nk, [&](auto w) {
+               launch(h.prm.use_pdl, k_gs_aux_down<T, V, decltype(w)::value>, nblk(nk, rows_tpb(nk)), rows_tpb(nk), s, k0, nk, SMd.off,
                       SMd.col, sell_vals(L.SMd, (const V*)nullptr), L.sm_dinv.p, L.sm_rows.p, (const T*)SP.F.p, sweep == 0 ? 1 : 0, SP.fs[li].p,
-                      SP.us[li].p));
+                      SP.us[li].p);
+             })));
         ++launches;
       }
     }
     auto RS = view(L.RS);
     LAUNCH(ASMG_PROF_AUX_RESID, L.RS.nnz_real * (sv + 4) + L.nrs_real * (4 + 2 * sz) + L.nsm_real * sz,
-           launch(h.prm.use_pdl, k_resid_aux<T, V>, nblk(L.nrs, rows_tpb(L.nrs)), rows_tpb(L.nrs), s, L.nrs, RS.off, RS.col, sell_vals(L.RS, (const V*)nullptr), L.rs_rows.p,
-                  (const T*)SP.us[li].p, SP.F.p));
+           (by_rows(L.nrs, [&](auto w) {
+               launch(h.prm.use_pdl, k_resid_aux<T, V, decltype(w)::value>, nblk(L.nrs, rows_tpb(L.nrs)), rows_tpb(L.nrs), s, L.nrs, RS.off, RS.col, sell_vals(L.RS, (const V*)nullptr), L.rs_rows.p,
+                  (const T*)SP.us[li].p, SP.F.p);
+             })));
     LAUNCH(ASMG_PROF_AUX_TRANSFER, L.nchild * (4 + sz) + L.npar * (8 + 2 * sz),
            launch(h.prm.use_pdl, k_restrict_aux<T>, nblk(L.npar, rows_tpb(L.npar)), rows_tpb(L.npar), s, L.npar, L.rp_id.p,
                   L.rp_ptr.p, L.rp_child.p, SP.F.p));
@@ -869,8 +874,10 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
         int64_t k0 = L.cstart[c], nk = L.cstart[c + 1] - L.cstart[c];
         if (!nk) continue;
         LAUNCH(ASMG_PROF_AUX_GS, L.cnnz[c] * (sv + 4) + L.crows[c] * (4 + 5 * sz),
-               launch(h.prm.use_pdl, k_gs_aux<T, V>, nblk(nk, rows_tpb(nk)), rows_tpb(nk), s, k0, nk, SM.off, SM.col, sell_vals(L.SM, (const V*)nullptr), L.sm_dinv.p,
-                      L.sm_rows.p, (const T*)SP.fs[li].p, SP.U.p));
+               (by_rows(nk, [&](auto w) {
+               launch(h.prm.use_pdl, k_gs_aux<T, V, decltype(w)::value>, nblk(nk, rows_tpb(nk)), rows_tpb(nk), s, k0, nk, SM.off, SM.col, sell_vals(L.SM, (const V*)nullptr), L.sm_dinv.p,
+                      L.sm_rows.p, (const T*)SP.fs[li].p, SP.U.p);
+             })));
         ++launches;
       }
   }
@@ -922,8 +929,10 @@ int enqueue_precond(asmg_s& h, Slot& S, const double* r, cudaStream_t s, bool fi
           int64_t r0 = h.fine_cstart[c], nr = h.fine_cstart[c + 1] - r0;
           if (!nr || (!forward && last_later && c == 0 && m == h.prm.fine_sweeps - 1)) continue;
           LAUNCH(ASMG_PROF_FINE_GS, h.fine_cnnz[c] * (sz + 4) + h.fine_crows[c] * (8 + 4 * sz),
-                 launch(h.prm.use_pdl, k_gs_fine<T, double>, nblk(nr, rows_tpb(nr)), rows_tpb(nr), s, r0, nr, A.off,
-                        A.col, A.val, dinv, r, SP.uf.p));
+                 (by_rows(nr, [&](auto w) {
+               launch(h.prm.use_pdl, k_gs_fine<T, double, decltype(w)::value>, nblk(nr, rows_tpb(nr)), rows_tpb(nr), s, r0, nr, A.off,
+                        A.col, A.val, dinv, r, SP.uf.p);
+             })));
           ++launches;
         }
       } else if (zero) {
@@ -948,8 +957,10 @@ int enqueue_precond(asmg_s& h, Slot& S, const double* r, cudaStream_t s, bool fi
       const int64_t r0 = h.fine_cstart[c], nr = h.fine_cstart[c + 1] - r0;
       if (!nr) continue;
       LAUNCH(ASMG_PROF_FINE_GS, h.fine_lnnz[c] * (sz + 4) + h.fine_crows[c] * (8 + 3 * sz),
-             launch(h.prm.use_pdl, k_gs_first<T>, nblk(nr, rows_tpb(nr)), rows_tpb(nr), s, r0, nr, Lo.off, Lo.col,
-                    Lo.val, dinv, r, SP.uf.p));
+             (by_rows(nr, [&](auto w) {
+               launch(h.prm.use_pdl, k_gs_first<T, decltype(w)::value>, nblk(nr, rows_tpb(nr)), rows_tpb(nr), s, r0, nr, Lo.off, Lo.col,
+                    Lo.val, dinv, r, SP.uf.p);
+             })));
       ++launches;
     }
   } else {
@@ -964,8 +975,10 @@ int enqueue_precond(asmg_s& h, Slot& S, const double* r, cudaStream_t s, bool fi
     } else if (split) {
       auto Up = view(P.Up);
       LAUNCH(ASMG_PROF_FINE_RESID, P.Up.nnz_real * (sz + 4) + n * 2 * sz,
-             launch(h.prm.use_pdl, k_resid_upper<T>, nblk(h.npad), TPB, s, h.npad, Up.off, Up.col, Up.val,
-                    (const T*)SP.uf.p, SP.rho.p));
+             (by_rows(h.npad, [&](auto w) {
+               launch(h.prm.use_pdl, k_resid_upper<T, decltype(w)::value>, nblk(h.npad), TPB, s, h.npad, Up.off, Up.col, Up.val,
+                    (const T*)SP.uf.p, SP.rho.p);
+             })));
     } else {
       LAUNCH(ASMG_PROF_FINE_RESID, h.A64.nnz_real * (sz + 4) + n * (8 + 2 * sz),
              launch(h.prm.use_pdl, k_resid_fine<T>, nblk(h.npad), TPB, s, h.npad, A.off, A.col, A.val, r, SP.uf.p,
@@ -973,12 +986,16 @@ int enqueue_precond(asmg_s& h, Slot& S, const double* r, cudaStream_t s, bool fi
     }
     auto PT = view(P.PT);
     LAUNCH(ASMG_PROF_RESTRICT, P.PT.nnz_real * (sz + 4) + n * sz + 2 * nJ * sz,
-           launch(h.prm.use_pdl, k_restrict_fine<T>, nblk(h.nJpad), TPB, s, h.nJpad, PT.off, PT.col, PT.val, SP.rho.p, SP.F.p, SP.U.p));
+           (by_rows<TRANSFER_W>(h.nJpad, [&](auto w) {
+               launch(h.prm.use_pdl, k_restrict_fine<T, decltype(w)::value>, nblk(h.nJpad), TPB, s, h.nJpad, PT.off, PT.col, PT.val, SP.rho.p, SP.F.p, SP.U.p);
+             })));
     launches += 2;
     launches += enqueue_vcycle_vals<T>(h, S, s);
     auto PP = view(P.P);
     LAUNCH(ASMG_PROF_PROLONG, P.P.nnz_real * (sz + 4) + nJ * sz + 2 * n * sz,
-           launch(h.prm.use_pdl, k_prolong_fine<T>, nblk(h.npad), TPB, s, h.npad, PP.off, PP.col, PP.val, SP.U.p, SP.uf.p));
+           (by_rows<TRANSFER_W>(h.npad, [&](auto w) {
+               launch(h.prm.use_pdl, k_prolong_fine<T, decltype(w)::value>, nblk(h.npad), TPB, s, h.npad, PP.off, PP.col, PP.val, SP.U.p, SP.uf.p);
+             })));
     ++launches;
   }
   // (3) multiplicative only: u3 = u2 + S^T (r - A u2)
@@ -1000,7 +1017,9 @@ int enqueue_body(asmg_s& h, Slot& S, cudaStream_t s, cudaGraphConditionalHandle 
                 S.partial.p, S.ticket.p, S.scal.p));
   LAUNCH(ASMG_PROF_CG_VECTOR, n * (sz + 16), launch(h.prm.use_pdl, k_pupd<T>, GV, TPB, s, h.npad, z, S.p.p, S.scal.p));
   LAUNCH(ASMG_PROF_CG_SPMV, h.A64.nnz_real * 12 + n * 16,
-         launch(h.prm.use_pdl, k_spmv_dot, G, TPB, s, h.npad, view(h.A64), S.p.p, S.q.p, S.partial.p, S.ticket.p, S.scal.p));
+         (by_rows(h.npad, [&](auto w) {
+               launch(h.prm.use_pdl, k_spmv_dot<decltype(w)::value>, G, TPB, s, h.npad, view(h.A64), S.p.p, S.q.p, S.partial.p, S.ticket.p, S.scal.p);
+             })));
   LAUNCH(ASMG_PROF_CG_VECTOR, n * 48 + n0 * 2 * sz,
          launch(h.prm.use_pdl, k_axpy_norm<T>, GV, TPB, s, h.npad, S.p.p, S.q.p, S.x.p, S.r.p, n0, dinv, z, S.partial.p,
                 S.ticket.p, S.scal.p, S.hist.p, hnd, use_hnd));

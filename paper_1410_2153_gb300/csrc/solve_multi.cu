@@ -75,19 +75,19 @@ __device__ __forceinline__ void stk(T* p, const VK<T>& r) {
 }
 
 // acc[j] += sum_e a_e x[c_e][j] over a SELL row held in registers (the order of row_dot)
-template <class T, class X, class V>
-__device__ __forceinline__ void row_dot_k(const Row<T>& R, const int32_t* __restrict__ col, const V* __restrict__ val,
+template <class T, class X, int N, class V>
+__device__ __forceinline__ void row_dot_k(const Row<T, N>& R, const int32_t* __restrict__ col, const V* __restrict__ val,
                                           const X* x, T (&acc)[K]) {
 #pragma unroll
   for (int j = 0; j < K; ++j) acc[j] = 0;
 #pragma unroll
-  for (int q = 0; q < MAXW; ++q)
+  for (int q = 0; q < N; ++q)
     if (q < R.w) {
       const VK<X> xv = ldk<X>(x + (int64_t)R.c[q] * K);
 #pragma unroll
       for (int j = 0; j < K; ++j) acc[j] += R.v[q] * (T)xv.v[j];
     }
-  for (int q = MAXW; q < R.w; ++q) {
+  for (int q = N; q < R.w; ++q) {
     const int64_t e = R.b + ((int64_t)q << 5) + R.lane;
     const T a = (T)ldg_val(val + e);
     const VK<X> xv = ldk<X>(x + (int64_t)__ldg(col + e) * K);
