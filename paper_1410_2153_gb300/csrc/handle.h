@@ -44,7 +44,8 @@ constexpr int READBACK_HIST = 512;
 
 // Scalars of the PCG recurrences, device resident.
 struct PcgScalars {
-  double rz;      // <r_k, z_k>
+  double rz;      // <r_k, z_k> of the step before
+  double rz_next; // of this step
   double alpha, beta, pq, rr, bnorm, tol;
   int k, maxit, status, cond;
   int timeout;    // set by a kernel whose bounded wait expired (the solve then stops)

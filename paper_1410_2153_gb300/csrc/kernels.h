@@ -171,42 +171,62 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return v;  // valid in thread 0
 }
 
-// Deterministic grid reduction of NV values: partials per block, the last
-// block to finish sums them in block order.  Returns true in that block.
+// v[j] of a block's threads -> its partials (value j of block b at j * grid + b)
 template <int NV>
-__device__ bool grid_reduce(double (&v)[NV], double* partial, unsigned int* ticket) {
+__device__ __forceinline__ void block_partials(const double (&v)[NV], double* partial) {
   __shared__ double sh[32];
-  __shared__ bool last;
   for (int j = 0; j < NV; ++j) {
-    double t = block_sum(v[j], sh);
+    const double t = block_sum(v[j], sh);
     if (threadIdx.x == 0) partial[j * gridDim.x + blockIdx.x] = t;
   }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
+}
+
+// The sums of nb blocks' partials, in block order; valid in thread 0.
+template <int NV>
+__device__ __forceinline__ void sum_partials(double (&v)[NV], const double* partial, unsigned nb) {
+  __shared__ double sh[32];
   for (int j = 0; j < NV; ++j) {
     // the partials of this thread (blocks t, t + blockDim, ...) summed in
     // ascending order, eight loads in flight
-    const double* pj = partial + (int64_t)j * gridDim.x;
+    const double* pj = partial + (int64_t)j * nb;
     double s = 0;
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += 8 * blockDim.x) {
+    for (unsigned b = threadIdx.x; b < nb; b += 8 * blockDim.x) {
       double x[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const unsigned bb = b + u * blockDim.x;
-        x[u] = bb < gridDim.x ? __ldcg(pj + bb) : 0.0;
+        x[u] = bb < nb ? __ldcg(pj + bb) : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) s += x[u];
     }
     v[j] = block_sum(s, sh);
   }
+}
+
+// Deterministic grid reduction of NV values: partials per block, the last
+// block to finish sums them in block order.  Returns true in that block.
+template <int NV>
+__device__ bool grid_reduce(double (&v)[NV], double* partial, unsigned int* ticket) {
+  __shared__ bool last;
+  block_partials(v, partial);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  sum_partials(v, partial, gridDim.x);
   if (threadIdx.x == 0) *ticket = 0;
   return true;
 }
+
+// Up to this many blocks a reduction's result is summed by every block of the
+// kernel that uses it, from the partials, instead of by the reduction's last
+// block: the ticket, that block's second pass and the read of its result drop
+// out of the chain of a small solve (65^2 FP64 725 -> 695 us).  With more
+// blocks the repeated sums cost more than they save.
+constexpr int DIRECT_BLOCKS = 2 * NSM;
 
 }  // namespace kern
 }  // namespace asmg

@@ -297,18 +297,38 @@ __global__ void k_addsaved_aux(int64_t nsm, const int32_t* __restrict__ rows, co
   if (i >= 0) U[i] += us[t];
 }
 
-// coarsest level: U[cid] = A_c^{-1} F[cid] in FP64, one warp per row
+// coarsest level: U[cid] = A_c^{-1} F[cid] in FP64, one warp per row.  A lane's
+// part of the row and its node IDs (setup data; the default cap of 512 nodes
+// is 16 entries) are in registers before the wait on the previous kernel.
+constexpr int COARSE_W = 16;
 template <class T>
 __global__ void k_coarse(int64_t nc, const int32_t* __restrict__ cid, const double* __restrict__ inv,
                          const T* __restrict__ F, T* __restrict__ U) {
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  double a[COARSE_W];
+  int32_t id[COARSE_W];
+  int32_t out = 0;
+  if (row < nc) {
+#pragma unroll
+    for (int q = 0; q < COARSE_W; ++q) {
+      const int64_t j = lane + 32 * q;
+      if (j < nc) {
+        a[q] = inv[row * nc + j];
+        id[q] = cid[j];
+      }
+    }
+    out = cid[row];
+  }
   pdl_wait();
   if (row < nc) {
     double s = 0;
-    for (int64_t j = lane; j < nc; j += 32) s += inv[row * nc + j] * (double)F[cid[j]];
+#pragma unroll
+    for (int q = 0; q < COARSE_W; ++q)
+      if (lane + 32 * q < nc) s += a[q] * (double)F[id[q]];
+    for (int64_t j = lane + 32 * COARSE_W; j < nc; j += 32) s += inv[row * nc + j] * (double)F[cid[j]];
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) U[cid[row]] = (T)s;
+    if (lane == 0) U[out] = (T)s;
   }
 }
 
@@ -476,6 +496,7 @@ __global__ void k_pcg_init(int64_t n, SellView<double> A, const double* __restri
     sc->maxit = maxit;
     sc->status = 1;
     sc->rz = 0;
+    sc->rz_next = 0;
     sc->alpha = 0;
     sc->beta = 0;
     sc->timeout = 0;
@@ -486,6 +507,15 @@ __global__ void k_pcg_init(int64_t n, SellView<double> A, const double* __restri
   }
 }
 
+// beta of this step from <z, q_prev> and the scalars of the step before
+__device__ __forceinline__ double step_beta(const PcgScalars& sc, double zq) {
+  return sc.k == 0 ? 0.0 : -sc.alpha * zq / sc.rz;
+}
+// alpha of this step from <p, q>; 0 on breakdown
+__device__ __forceinline__ double step_alpha(const PcgScalars& sc, double pq) {
+  return !(pq > 0) || sc.status == ASMG_ERR_BREAKDOWN ? 0.0 : sc.rz_next / pq;
+}
+
 // <z, r>, <z, q_prev>  ->  beta (flexible: -alpha <z_{k+1}, q_k> / <z_k, r_k>), rz.
 // The first n0 rows (colour class 0, the last of the backward sweep) take their
 // Gauss-Seidel step here: every other class is done, and no row reads theirs
@@ -493,7 +523,7 @@ __global__ void k_pcg_init(int64_t n, SellView<double> A, const double* __restri
 template <class T>
 __global__ void k_dots(int64_t n, int64_t n0, SellView<T> A, const T* __restrict__ dinv, T* z,
                        const double* __restrict__ r, const double* __restrict__ q, double* partial,
-                       unsigned int* ticket, PcgScalars* sc) {
+                       unsigned int* ticket, PcgScalars* sc, int direct) {
   const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
   Row<T> row;
   if (i0 < n0) row_load(row, i0, A.off, A.col, A.val);
@@ -515,22 +545,38 @@ __global__ void k_dots(int64_t n, int64_t n0, SellView<T> A, const T* __restrict
     v[0] += zi * r[i];
     v[1] += zi * q[i];
   }
-  if (grid_reduce<2>(v, partial, ticket) && threadIdx.x == 0) {
-    if (sc->k == 0) {
-      sc->beta = 0;
-    } else {
-      sc->beta = -sc->alpha * v[1] / sc->rz;
-    }
-    sc->rz = v[0];
+  if (direct) {
+    block_partials(v, partial);  // k_pupd sums them
+  } else if (grid_reduce<2>(v, partial, ticket) && threadIdx.x == 0) {
+    sc->beta = step_beta(*sc, v[1]);
+    sc->rz_next = v[0];
     if (!(v[0] > 0)) sc->status = ASMG_ERR_BREAKDOWN;
   }
 }
 
-// p = z + beta p
+// p = z + beta p; nb > 0: beta from the nb partials of k_dots
 template <class T>
-__global__ void k_pupd(int64_t n, const T* __restrict__ z, double* __restrict__ p, const PcgScalars* __restrict__ sc) {
+__global__ void k_pupd(int64_t n, const T* __restrict__ z, double* __restrict__ p, const double* partial, int nb,
+                       PcgScalars* sc) {
+  __shared__ double sh_beta;
   pdl_wait();
-  const double beta = sc->beta;
+  double beta;
+  if (nb) {
+    double v[2];
+    sum_partials(v, partial, (unsigned)nb);
+    if (threadIdx.x == 0) {
+      sh_beta = step_beta(*sc, v[1]);  // reads k, alpha and rz, which this kernel does not write
+      if (blockIdx.x == 0) {
+        sc->beta = sh_beta;
+        sc->rz_next = v[0];
+        if (!(v[0] > 0)) sc->status = ASMG_ERR_BREAKDOWN;
+      }
+    }
+    __syncthreads();
+    beta = sh_beta;
+  } else {
+    beta = sc->beta;
+  }
 #pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     p[i] = (double)z[i] + beta * p[i];
@@ -541,7 +587,7 @@ __global__ void k_pupd(int64_t n, const T* __restrict__ z, double* __restrict__ 
 // kernel (graded 2049^2: 3.1 -> 4.3 TB/s against a plain loop over the row).
 template <int N>
 __global__ void k_spmv_dot(int64_t n, SellView<double> A, const double* __restrict__ p, double* __restrict__ q,
-                           double* partial, unsigned int* ticket, PcgScalars* sc) {
+                           double* partial, unsigned int* ticket, PcgScalars* sc, int direct) {
   const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
   Row<double, N> row;
   if (i0 < n) row_load(row, i0, A.off, A.col, A.val);
@@ -553,14 +599,12 @@ __global__ void k_spmv_dot(int64_t n, SellView<double> A, const double* __restri
     q[i] = qi;
     v[0] += p[i] * qi;
   }
-  if (grid_reduce<1>(v, partial, ticket) && threadIdx.x == 0) {
+  if (direct) {
+    block_partials(v, partial);  // k_axpy_norm sums them
+  } else if (grid_reduce<1>(v, partial, ticket) && threadIdx.x == 0) {
     sc->pq = v[0];
-    if (!(v[0] > 0) || sc->status == ASMG_ERR_BREAKDOWN) {
-      sc->status = ASMG_ERR_BREAKDOWN;
-      sc->alpha = 0;
-    } else {
-      sc->alpha = sc->rz / v[0];
-    }
+    sc->alpha = step_alpha(*sc, v[0]);
+    if (!(v[0] > 0)) sc->status = ASMG_ERR_BREAKDOWN;
   }
 }
 
@@ -569,10 +613,28 @@ __global__ void k_spmv_dot(int64_t n, SellView<double> A, const double* __restri
 template <class T>
 __global__ void k_axpy_norm(int64_t n, const double* __restrict__ p, const double* __restrict__ q,
                             double* __restrict__ x, double* __restrict__ r, int64_t n0, const T* __restrict__ dinv,
-                            T* __restrict__ u, double* partial, unsigned int* ticket,
-                            PcgScalars* sc, double* hist, cudaGraphConditionalHandle hnd, int use_hnd) {
+                            T* __restrict__ u, const double* pq_partial, int nb, double* partial,
+                            unsigned int* ticket, PcgScalars* sc, double* hist, cudaGraphConditionalHandle hnd,
+                            int use_hnd) {
+  __shared__ double sh_alpha;
   pdl_wait();
-  const double a = sc->alpha;
+  double a;
+  if (nb) {  // alpha from the nb partials of k_spmv_dot
+    double pq[1];
+    sum_partials(pq, pq_partial, (unsigned)nb);
+    if (threadIdx.x == 0) {
+      sh_alpha = step_alpha(*sc, pq[0]);  // a breakdown written below leaves this 0 in every block
+      if (blockIdx.x == 0) {
+        sc->pq = pq[0];
+        sc->alpha = sh_alpha;
+        if (!(pq[0] > 0)) sc->status = ASMG_ERR_BREAKDOWN;
+      }
+    }
+    __syncthreads();
+    a = sh_alpha;
+  } else {
+    a = sc->alpha;
+  }
   double v[1] = {0};
 #pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -593,6 +655,7 @@ __global__ void k_axpy_norm(int64_t n, const double* __restrict__ p, const doubl
       return;
     }
     sc->k += 1;
+    sc->rz = sc->rz_next;
     sc->rr = v[0];
     const double nr = sqrt(v[0]);
     hist[sc->k] = nr;
@@ -1011,18 +1074,22 @@ int enqueue_body(asmg_s& h, Slot& S, cudaStream_t s, cudaGraphConditionalHandle 
   T* z = slotprec<T>(S).uf.p;
   const T* dinv = fine_dinv<T>(h);
   const int G = red_grid(h.npad, RED_BLOCKS), GV = red_grid(h.npad, VEC_BLOCKS);
+  const int nb = GV <= DIRECT_BLOCKS ? GV : 0;  // then G == GV
+  double* pq = S.partial.p + 2 * VEC_BLOCKS;     // partials of <p, q>, which k_axpy_norm reads beside its own
   const int64_t n = h.n, sz = sizeof(T);
   LAUNCH(ASMG_PROF_CG_VECTOR, n * (sz + 16) + (n0 ? h.fine_cnnz[0] * (sz + 4) + h.fine_crows[0] * (8 + 2 * sz) : 0),
          launch(h.prm.use_pdl, k_dots<T>, GV, TPB, s, h.npad, n0, fine_smoother<T>(h), dinv, z, S.r.p, S.q.p,
-                S.partial.p, S.ticket.p, S.scal.p));
-  LAUNCH(ASMG_PROF_CG_VECTOR, n * (sz + 16), launch(h.prm.use_pdl, k_pupd<T>, GV, TPB, s, h.npad, z, S.p.p, S.scal.p));
+                S.partial.p, S.ticket.p, S.scal.p, nb));
+  LAUNCH(ASMG_PROF_CG_VECTOR, n * (sz + 16),
+         launch(h.prm.use_pdl, k_pupd<T>, GV, TPB, s, h.npad, (const T*)z, S.p.p, (const double*)S.partial.p, nb,
+                S.scal.p));
   LAUNCH(ASMG_PROF_CG_SPMV, h.A64.nnz_real * 12 + n * 16,
          (by_rows(h.npad, [&](auto w) {
-               launch(h.prm.use_pdl, k_spmv_dot<decltype(w)::value>, G, TPB, s, h.npad, view(h.A64), S.p.p, S.q.p, S.partial.p, S.ticket.p, S.scal.p);
+               launch(h.prm.use_pdl, k_spmv_dot<decltype(w)::value>, G, TPB, s, h.npad, view(h.A64), S.p.p, S.q.p, pq, S.ticket.p, S.scal.p, nb);
              })));
   LAUNCH(ASMG_PROF_CG_VECTOR, n * 48 + n0 * 2 * sz,
-         launch(h.prm.use_pdl, k_axpy_norm<T>, GV, TPB, s, h.npad, S.p.p, S.q.p, S.x.p, S.r.p, n0, dinv, z, S.partial.p,
-                S.ticket.p, S.scal.p, S.hist.p, hnd, use_hnd));
+         launch(h.prm.use_pdl, k_axpy_norm<T>, GV, TPB, s, h.npad, S.p.p, S.q.p, S.x.p, S.r.p, n0, dinv, z, (const double*)pq, nb,
+                S.partial.p, S.ticket.p, S.scal.p, S.hist.p, hnd, use_hnd));
   ASMG_CUDA(cudaGetLastError());
   return launches + 4;
 }
@@ -1443,7 +1510,7 @@ Slot& add_slot(asmg_s& h, cudaStream_t s) {
   S.q.zero(s);
   S.vb.alloc(h.mesh.nv);
   S.vu.alloc(h.mesh.nv);
-  S.partial.alloc(std::max(4 * RED_BLOCKS, 2 * VEC_BLOCKS));
+  S.partial.alloc(std::max(4 * RED_BLOCKS, 2 * VEC_BLOCKS + RED_BLOCKS));
   S.ticket.alloc(1);
   S.ticket.zero(s);
   S.scal.alloc(1);

@@ -412,22 +412,40 @@ __global__ void k_addsaved_aux_k(int64_t nsm, const int32_t* __restrict__ rows, 
 }
 
 // coarsest level, FP64, one warp per row (the lanes' order of k_coarse per column)
+constexpr int COARSE_WK = 16;
 template <class T>
 __global__ void k_coarse_k(int64_t nc, const int32_t* __restrict__ cid, const double* __restrict__ inv,
                            const T* __restrict__ F, T* __restrict__ U) {
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  double a[COARSE_WK];
+  int32_t id[COARSE_WK];
+  int32_t out = 0;
+  if (row < nc) {
+#pragma unroll
+    for (int q = 0; q < COARSE_WK; ++q) {
+      const int64_t c = lane + 32 * q;
+      if (c < nc) {
+        a[q] = inv[row * nc + c];
+        id[q] = cid[c];
+      }
+    }
+    out = cid[row];
+  }
   pdl_wait();
   if (row < nc) {
     double s[K];
 #pragma unroll
     for (int j = 0; j < K; ++j) s[j] = 0;
-    for (int64_t c = lane; c < nc; c += 32) {
-      const double a = inv[row * nc + c];
-      const VK<T> f = ldk<T>(F + (int64_t)cid[c] * K);
+    auto add = [&](double x, int32_t i) {
+      const VK<T> f = ldk<T>(F + (int64_t)i * K);
 #pragma unroll
-      for (int j = 0; j < K; ++j) s[j] += a * (double)f.v[j];
-    }
+      for (int j = 0; j < K; ++j) s[j] += x * (double)f.v[j];
+    };
+#pragma unroll
+    for (int q = 0; q < COARSE_WK; ++q)
+      if (lane + 32 * q < nc) add(a[q], id[q]);
+    for (int64_t c = lane + 32 * COARSE_WK; c < nc; c += 32) add(inv[row * nc + c], cid[c]);
 #pragma unroll
     for (int j = 0; j < K; ++j)
       for (int o = 16; o; o >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
@@ -435,7 +453,7 @@ __global__ void k_coarse_k(int64_t nc, const int32_t* __restrict__ cid, const do
       VK<T> o;
 #pragma unroll
       for (int j = 0; j < K; ++j) o.v[j] = (T)s[j];
-      stk<T>(U + (int64_t)cid[row] * K, o);
+      stk<T>(U + (int64_t)out * K, o);
     }
   }
 }
