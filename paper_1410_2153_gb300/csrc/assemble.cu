@@ -236,23 +236,37 @@ __global__ void k_mass_gather(int64_t nv, const int64_t* __restrict__ v2e_ptr, c
   if (rowv[v] >= 0) {
     const double fv = f[v];
     const int64_t p1 = v2e_ptr[v + 1];
-    for (int64_t p = v2e_ptr[v]; p < p1; ++p) {
-      const int64_t t = v2e[p];
-      int32_t q[NV];
-      if constexpr (NV == 4) {
-        const int4 e = *reinterpret_cast<const int4*>(E + 4 * t);
-        q[0] = e.x;
-        q[1] = e.y;
-        q[2] = e.z;
-        q[3] = e.w;
-      } else {
+    // four elements at a time: each step of the chain (element, its vertices,
+    // their values) has its loads in flight together; added in ascending order
+    for (int64_t p = v2e_ptr[v]; p < p1; p += 4) {
+      int64_t t[4];
+      int32_t q[4][NV];
+      double sum[4], wt[4];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) q[k] = E[NV * t + k];
+      for (int u = 0; u < 4; ++u) t[u] = v2e[p + u < p1 ? p + u : p];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        wt[u] = w[t[u]];
+        if constexpr (NV == 4) {
+          const int4 e = *reinterpret_cast<const int4*>(E + 4 * t[u]);
+          q[u][0] = e.x;
+          q[u][1] = e.y;
+          q[u][2] = e.z;
+          q[u][3] = e.w;
+        } else {
+#pragma unroll
+          for (int k = 0; k < NV; ++k) q[u][k] = E[NV * t[u] + k];
+        }
       }
-      double sum = f[q[0]];
 #pragma unroll
-      for (int k = 1; k < NV; ++k) sum += f[q[k]];
-      acc += w[t] * (sum + fv);
+      for (int u = 0; u < 4; ++u) {
+        sum[u] = f[q[u][0]];
+#pragma unroll
+        for (int k = 1; k < NV; ++k) sum[u] += f[q[u][k]];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (p + u < p1) acc += wt[u] * (sum[u] + fv);
     }
   }
   b[v] = acc;

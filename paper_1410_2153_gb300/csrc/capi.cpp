@@ -1697,7 +1697,7 @@ int amg_precond_apply(asmg_handle h, const double* r, double* z, void* stream) {
   gather_rows(*h, input(r, S0.vb.p, nv, s), S0.r.p, s);
   int* tflag = reinterpret_cast<int*>(reinterpret_cast<char*>(S0.scal.p) + offsetof(PcgScalars, timeout));
   ASMG_CUDA(cudaMemsetAsync(tflag, 0, sizeof(int), s));
-  precond_apply(*h, S0.r.p, s);
+  precond_apply(*h, s);
   const bool direct = in_place(z);
   double* out = direct ? z : S0.vu.p;
   if (h->prm.precision == ASMG_MIXED)

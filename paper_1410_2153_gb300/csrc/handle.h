@@ -86,7 +86,9 @@ struct Slot {
   cudaGraph_t graph = nullptr;       // single-solve graph
   cudaGraphExec_t gexec = nullptr;
   double graph_rtol = -1;
+  cudaGraphExec_t pexec = nullptr;   // one preconditioner application (r -> uf)
   ~Slot() {
+    if (pexec) cudaGraphExecDestroy(pexec);
     if (gexec) cudaGraphExecDestroy(gexec);
     if (graph) cudaGraphDestroy(graph);
   }
@@ -193,7 +195,7 @@ int run_solve(asmg_s& h, Slot& S, double rtol, cudaStream_t s);
 Slot& add_slot(asmg_s& h, cudaStream_t s);
 cudaGraphNode_t capture_solve(asmg_s& h, Slot& S, double rtol, cudaGraph_t g, const cudaGraphNode_t* deps,
                               size_t ndeps);
-void precond_apply(asmg_s& h, const double* r_perm, cudaStream_t s);  // result in h.p*.uf
+void precond_apply(asmg_s& h, cudaStream_t s);  // slot 0's r -> its uf
 void spmv64(asmg_s& h, const double* x_perm, double* y_perm, cudaStream_t s);
 void gather_rows(asmg_s& h, const double* vsrc, double* dst, cudaStream_t s);
 void scatter_rows(asmg_s& h, const void* src, bool src_float, double* vdst, cudaStream_t s);

@@ -1172,12 +1172,33 @@ void mask_pair(asmg_s& h, const double* u, const double* lambda, double* pair, c
   ASMG_CUDA(cudaGetLastError());
 }
 
-void precond_apply(asmg_s& h, const double* r_perm, cudaStream_t s) {
-  Slot& S = *h.slots[0];
+static void enqueue_precond_any(asmg_s& h, Slot& S, cudaStream_t s) {
   if (h.prm.precision == ASMG_MIXED)
-    enqueue_precond<float>(h, S, r_perm, s);
+    enqueue_precond<float>(h, S, S.r.p, s);
   else
-    enqueue_precond<double>(h, S, r_perm, s);
+    enqueue_precond<double>(h, S, S.r.p, s);
+}
+
+// One application as a graph (use_graph): some 50 launches, which the host
+// issues more slowly than the device runs them (kuhn65 FP64 306 -> 285 us).
+void precond_apply(asmg_s& h, cudaStream_t s) {
+  Slot& S = *h.slots[0];
+  if (!h.prm.use_graph) {
+    enqueue_precond_any(h, S, s);
+    return;
+  }
+  if (!S.pexec) {
+    cudaStream_t cs;
+    cudaGraph_t g;
+    ASMG_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    ASMG_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    enqueue_precond_any(h, S, cs);
+    ASMG_CUDA(cudaStreamEndCapture(cs, &g));
+    ASMG_CUDA(cudaStreamDestroy(cs));
+    ASMG_CUDA(cudaGraphInstantiate(&S.pexec, g, 0));
+    ASMG_CUDA(cudaGraphDestroy(g));
+  }
+  ASMG_CUDA(cudaGraphLaunch(S.pexec, s));
 }
 
 // y = A x, a row's entries loaded into registers at once
