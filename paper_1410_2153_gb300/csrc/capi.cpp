@@ -83,13 +83,13 @@ int64_t pad32(int64_t n) { return (n + 31) / 32 * 32; }
 // Temporally blocked sweeps (asmg_params::tile_rows = 0): own rows per tile on
 // levels of two colour classes, and on levels of more (whose longer dependency
 // chains make deeper halos, which larger tiles amortise) as a share of the rows
-// a block holds (1,024).  A larger share overflows and its tiles are halved
-// (graded 2049^2 with BF16 levels, post-sweeps at a share of 0.5: 4,104 tiles
-// where 3,758 of 0.375 do, 232.3 against 231.6 ms); a smaller one carries more
-// halo (0.38 down and 0.3 up: 235.1 ms).  TILE_MAX_HALO: the largest halo
-// accepted, as a multiple of the own rows.
+// a block holds (1,024).  A larger share overflows and its tiles are halved, a
+// smaller one carries more halo: pre-sweeps at a share of 0.5 / 0.44 / 0.375
+// take graded 2049^2 BF16 209.4 / 205.2 / 205.1 ms, graded 513^2 FP64 29.6 /
+// 28.8 / 28.6 ms.  TILE_MAX_HALO: the largest halo accepted, as a multiple of
+// the own rows.
 constexpr int TILE_ROWS_2COL = 256;
-constexpr double TILE_OWN_DOWN = 0.5, TILE_OWN_UP = 0.375;
+constexpr double TILE_OWN = 0.375;
 constexpr double TILE_MAX_HALO = 1.5;
 constexpr int64_t TILE_MIN_ROWS = 64;  // smoothing rows of a tiled level (below, the fused runs hold every level)
 
@@ -259,7 +259,8 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
 // zero on the way down (such reads need no row), read from us on the way up
 // (the row is kept, with its start value).  Every entry of a kept row that
 // points to a row of N~_l outside the tile is left out: no pair of the
-// closure reads it.  Entries of the post-sweeps' rows whose column lies
+// closure reads it.  On the way down the own rows' residual reads the last
+// value of every coupled row.  Entries of the post-sweeps' rows whose column lies
 // outside N~_l become the tile's outside values.  SMd: SM-order rows with
 // their N~_l columns as SM rows; SM: the same rows with all columns as aux
 // IDs; pos: aux ID -> SM row.  Returns false (and builds nothing) when a row
@@ -333,6 +334,9 @@ bool build_tiles(bool up, int nu, int tile_rows, const std::vector<int64_t>& sel
           for (int64_t q = o0; q < o1; ++q) {
             ownm[own[q]] = tag;
             need(own[q], nu - 1);
+            // the residual of the own rows reads every coupled row's last value
+            if (!up)
+              for (int64_t p = SMd.ptr[own[q]]; p < SMd.ptr[own[q] + 1]; ++p) need(SMd.col[p], nu - 1);
           }
           while (!stack.empty()) {
             const auto [k, sw] = stack.back();
@@ -690,8 +694,7 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
       if (pos[id] < 0) ok = false;
     const double max_halo = prm.tile_rows > 0 ? 1e30 : TILE_MAX_HALO;
     const int cap = TILE_SLOTS_MAX * TILE_THREADS;
-    const int rd = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN_DOWN);
-    const int ru = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN_UP);
+    const int trows = prm.tile_rows > 0 ? prm.tile_rows : ncol <= 2 ? TILE_ROWS_2COL : (int)(cap * TILE_OWN);
     if (ok && D.nsm_real >= TILE_MIN_ROWS) {
       // the two directions are built at the same time, each on half the host threads
       TileSweeps<T> td, tu;
@@ -700,13 +703,13 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
       std::exception_ptr eu, ed;
       std::thread up_th([&] {
         try {
-          oku = build_tiles<T>(true, prm.nu_post, ru, sel, D.cstart, dinv, SMd, SM, pos, max_halo, half, bf16, tu, s);
+          oku = build_tiles<T>(true, prm.nu_post, trows, sel, D.cstart, dinv, SMd, SM, pos, max_halo, half, bf16, tu, s);
         } catch (...) {
           eu = std::current_exception();
         }
       });
       try {
-        okd = build_tiles<T>(false, prm.nu_pre, rd, sel, D.cstart, dinv, SMd, SM, pos, max_halo, half, bf16, td, s);
+        okd = build_tiles<T>(false, prm.nu_pre, trows, sel, D.cstart, dinv, SMd, SM, pos, max_halo, half, bf16, td, s);
       } catch (...) {
         ed = std::current_exception();
       }
@@ -724,7 +727,7 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
         D.tdown = std::move(td);
         D.tup = std::move(tu);
         D.tiled = D.tiled_down = D.tiled_up = true;
-        D.tile_rows = rd;
+        D.tile_rows = trows;
       }
     }
   }
@@ -775,6 +778,46 @@ void build_level_dev(const AuxLevelHost& L, const HostCSR& Arows, const std::vec
   D.rp_id.upload(pid, s);
   D.rp_ptr.upload(pptr, s);
   D.rp_child.upload(child, s);
+  if (D.tiled) {
+    // residual and restriction after tiled pre-sweeps
+    std::vector<uint8_t> isnew(Arows.nr, 0);
+    for (int32_t id : L.new_id) isnew[id] = 1;
+    std::vector<int32_t> par(Arows.nr, -1);
+    for (size_t t = 0; t < pid.size(); ++t) par[pid[t]] = (int32_t)t;
+    std::vector<int64_t> other;
+    std::vector<int32_t> id, src, cptr(1, 0), cch;
+    auto add = [&](int32_t v) {
+      id.push_back(v);
+      if (v >= 0 && par[v] >= 0)
+        for (int32_t p = pptr[par[v]]; p < pptr[par[v] + 1]; ++p) cch.push_back(pos[child[p]]);
+      cptr.push_back((int32_t)cch.size());
+    };
+    for (int64_t v = 0; v < Arows.nr; ++v) {
+      if (isnew[v]) continue;
+      if (pos[v] >= 0) {
+        add((int32_t)v);
+        src.push_back(pos[v]);
+      } else if (touched[v] || par[v] >= 0) {
+        other.push_back(v);
+      }
+    }
+    while (id.size() % 32) add(-1);
+    src.resize(id.size(), 0);
+    D.trest.n1 = (int64_t)id.size();
+    for (int64_t v : other) add((int32_t)v);
+    while (id.size() % 32) add(-1);
+    while (other.size() % 32) other.push_back(-1);
+    D.trest.n2 = (int64_t)id.size() - D.trest.n1;
+    D.trest.nchild = (int64_t)cch.size();
+    sell_build<T>(D.trest.X, select_rows(Arows, other, &pos, &inset), 0, s);
+    if constexpr (std::is_same<T, float>::value)
+      if (bf16) sell_bf16(D.trest.X, s);
+    D.trest.id.upload(id, s);
+    D.trest.src.upload(src, s);
+    D.trest.ptr.upload(cptr, s);
+    D.trest.child.upload(cch, s);
+    ASMG_CUDA(cudaStreamSynchronize(s));
+  }
   build_nb_dev<T>(L, Arows, pos, D, s);
   // a level with a near-boundary solve keeps its own launches (the solve sits
   // between the coarse correction and the post-smoothing)

@@ -68,6 +68,7 @@ template <class T>
 struct SlotPrec {
   DBuf<T> uf, rho, F, U;            // fine work vector, fine residual, aux rhs / correction
   std::vector<DBuf<T>> fs, us;      // per level: saved rhs / pre-smoothed values on N~_l
+  std::vector<DBuf<T>> fr;          // per level with tiled pre-sweeps: residual on N~_l
   std::vector<DBuf<double>> nbr, nbs;  // per level: near-boundary rhs / solution pools (mixed boundaries)
   std::vector<DBuf<T>> ust, fsl;    // per level with tiled post-sweeps: start values and saved rhs in tile order
   DBuf<T> deep_fs, deep_us, bot_fs, bot_us;  // the same for the levels of the fused runs
@@ -109,7 +110,7 @@ struct MultiScalars {
 template <class T>
 struct MultiPrec {
   DBuf<T> uf, rho, F, U;                  // [rows][KRHS]
-  std::vector<DBuf<T>> fs, us;            // per level [nsm][KRHS]
+  std::vector<DBuf<T>> fs, us, fr;        // per level [nsm][KRHS] (fr: with tiled pre-sweeps)
   std::vector<DBuf<T>> ust, fsl;          // per level with tiled post-sweeps [nloc][KRHS]
   DBuf<T> deep_fs, deep_us, bot_fs, bot_us;  // the same for the levels of the fused runs
 };

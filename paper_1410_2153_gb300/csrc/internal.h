@@ -397,6 +397,21 @@ struct TileSweeps {
   int64_t smem() const { return ((int64_t)(slots * TILE_THREADS + maxext) * (int64_t)sizeof(T) + 127) / 128 * 128 + maxblob; }
 };
 
+// What follows the tiled pre-sweeps of a level (k_restrict_tile): the tiles
+// leave the residual of the smoothing rows in fr (SM order); every other node
+// that the coarser levels read takes its own, and half the sum of its new
+// children's.  Rows [0, n1) are smoothing rows carried from the coarser level
+// (src: their SM row), rows [n1, n1 + n2) the other nodes of E_l and the
+// parents outside it, with the level's matrix rows in X (columns SM rows).
+template <class T>
+struct TileRestrict {
+  int64_t n1 = 0, n2 = 0;        // multiples of 32
+  int64_t nchild = 0;
+  DBuf<int32_t> id, src;         // [n1 + n2], [n1] aux ID (-1 padding), SM row
+  DBuf<int32_t> ptr, child;      // children as SM rows (CSR over the n1 + n2 rows)
+  Sell<T> X;                     // [n2]
+};
+
 // The exact near-boundary solve of Algorithm 3 on the device: the block
 // cyclic reduction of nb::Factor flattened into arrays.  Ordered positions q
 // (0..m-1) follow the factor's breadth-first order.  Round r has nblk[r]
@@ -447,6 +462,7 @@ struct AuxLevelDev {
   bool tiled_down = false, tiled_up = false;  // the directions that run on them (the autotuner's choice)
   int tile_rows = 0;                 // own rows per tile
   TileSweeps<T> tdown, tup;
+  TileRestrict<T> trest;             // with tiled pre-sweeps: residual and restriction after them
   DBuf<int32_t> sm_par0, sm_par1;    // per SM row: parents of a new node (-1 Dirichlet), -3 not new
   // mixed boundaries: the near-boundary correction of Algorithm 3 (nb.m > 0):
   // rows of A_l on J_{l,j} in ordered positions (all columns, aux IDs) and the

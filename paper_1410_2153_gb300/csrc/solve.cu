@@ -843,15 +843,19 @@ int enqueue_vcycle(asmg_s& h, Slot& S, cudaStream_t s) {
       // all pre-sweeps of the level in one launch (compulsory bytes: the
       // tiles' blocks once, F gathered and saved, us written)
       const TileSweeps<T>& Tl = L.tdown;
-      const int64_t by = Tl.nnz_real * (sv + 2) + (Tl.interior + Tl.halo) * (8 + 2 * sz) + Tl.interior * (4 + sz);
+      const int64_t by = Tl.nnz_real * (sv + 2) + (Tl.interior + Tl.halo) * (8 + 2 * sz) + Tl.interior * (4 + 2 * sz);
       LAUNCH(ASMG_PROF_AUX_GS, by,
-             (tiles::launch_down<T, V, 1>(h.prm.use_pdl, Tl, L.ncolours, SP.F.p, SP.fs[li].p, SP.us[li].p, npre,
+             (tiles::launch_down<T, V, 1>(h.prm.use_pdl, Tl, L.ncolours, SP.F.p, SP.fs[li].p, SP.us[li].p, SP.fr[li].p, npre,
                                           timeout_flag(S), h.prm.inject_timeout, s)));
-      ++launches;
+      const TileRestrict<T>& R = L.trest;
+      LAUNCH(ASMG_PROF_AUX_TRANSFER, R.X.nnz_real * (sv + 4) + R.n1 * (12 + 2 * sz) + R.n2 * (8 + 2 * sz) + R.nchild * (4 + sz),
+             (tiles::launch_restrict<T, V, 1>(h.prm.use_pdl, R, SP.fr[li].p, SP.us[li].p, SP.F.p, s)));
+      launches += 2;
+      continue;
     }
     // pre-sweeps on us (SM order); the first also saves F on N~_l for the
     // post-sweeps (nu_pre >= 1)
-    for (int sweep = 0; sweep < (L.tiled_down ? 0 : npre); ++sweep) {
+    for (int sweep = 0; sweep < npre; ++sweep) {
       for (int c = 0; c < L.ncolours; ++c) {
         int64_t k0 = L.cstart[c], nk = L.cstart[c + 1] - L.cstart[c];
         if (!nk) continue;
@@ -1376,11 +1380,17 @@ void alloc_slot_prec(asmg_s& h, Prec<T>& P, SlotPrec<T>& SP, cudaStream_t s) {
   SP.fsl.clear();
   SP.ust.resize(nlev);
   SP.fsl.resize(nlev);
+  SP.fr.clear();
+  SP.fr.resize(nlev);
   for (int li = 0; li < nlev; ++li) {
     SP.fs[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1));
     SP.us[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1));
     SP.fs[li].zero(s);
     SP.us[li].zero(s);
+    if (P.lev[li].tiled_down) {
+      SP.fr[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1));
+      SP.fr[li].zero(s);
+    }
     if (P.lev[li].tiled_up) {
       // post-sweep start values and saved rhs in tile order (padding rows stay 0)
       SP.ust[li].alloc(std::max<int64_t>(P.lev[li].tup.nloc, 1));
@@ -1485,7 +1495,11 @@ void drop_untiled(asmg_s& h) {
   for (size_t li = 0; li < P.lev.size(); ++li) {
     AuxLevelDev<T>& L = P.lev[li];
     if (!L.tiled) continue;
-    if (!L.tiled_down) L.tdown = TileSweeps<T>();
+    if (!L.tiled_down) {
+      L.tdown = TileSweeps<T>();
+      L.trest = TileRestrict<T>();
+      SP.fr[li] = DBuf<T>();
+    }
     if (!L.tiled_up) {
       L.tup = TileSweeps<T>();
       SP.ust[li] = DBuf<T>();
@@ -1554,6 +1568,7 @@ void drop_unused_tiles(Prec<T>& P) {
       P.lev[li].tiled = P.lev[li].tiled_down = P.lev[li].tiled_up = false;
       P.lev[li].tdown = TileSweeps<T>();
       P.lev[li].tup = TileSweeps<T>();
+      P.lev[li].trest = TileRestrict<T>();
     }
 }
 

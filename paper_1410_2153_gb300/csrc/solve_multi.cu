@@ -769,10 +769,13 @@ void enqueue_vcycle_k(asmg_s& h, MultiSlot& S, cudaStream_t s) {
     AuxLevelDev<T>& L = P.lev[li];
     auto SMd = view(L.SMd);
     const bool tiled = L.tiled_down && tiles_fit(L.tdown);
-    if (tiled)
-      tiles::launch_down<T, V, K>(pdl, L.tdown, L.ncolours, M.F.p, M.fs[li].p, M.us[li].p, npre, timeout_flag_k(S),
-                                  h.prm.inject_timeout, s);
-    for (int sweep = 0; sweep < (tiled ? 0 : npre); ++sweep)
+    if (tiled) {
+      tiles::launch_down<T, V, K>(pdl, L.tdown, L.ncolours, M.F.p, M.fs[li].p, M.us[li].p, M.fr[li].p, npre,
+                                  timeout_flag_k(S), h.prm.inject_timeout, s);
+      tiles::launch_restrict<T, V, K>(pdl, L.trest, M.fr[li].p, M.us[li].p, M.F.p, s);
+      continue;
+    }
+    for (int sweep = 0; sweep < npre; ++sweep)
       for (int c = 0; c < L.ncolours; ++c) {
         const int64_t k0 = L.cstart[c], nk = L.cstart[c + 1] - L.cstart[c];
         if (!nk) continue;
@@ -925,11 +928,17 @@ void alloc_multi_prec(asmg_s& h, MultiPrec<T>& M, cudaStream_t s) {
   M.fsl.clear();
   M.ust.resize(nlev);
   M.fsl.resize(nlev);
+  M.fr.clear();
+  M.fr.resize(nlev);
   for (int li = 0; li < nlev; ++li) {
     M.fs[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1) * K);
     M.us[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1) * K);
     M.fs[li].zero(s);
     M.us[li].zero(s);
+    if (P.lev[li].tiled_down && tiles_fit(P.lev[li].tdown)) {
+      M.fr[li].alloc(std::max<int64_t>(P.lev[li].nsm, 1) * K);
+      M.fr[li].zero(s);
+    }
     if (P.lev[li].tiled_up && tiles_fit(P.lev[li].tup)) {
       M.ust[li].alloc(std::max<int64_t>(P.lev[li].tup.nloc, 1) * K);
       M.fsl[li].alloc(std::max<int64_t>(P.lev[li].tup.nloc, 1) * K);

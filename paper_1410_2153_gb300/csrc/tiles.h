@@ -205,11 +205,14 @@ constexpr int tile_min_blocks() {
 }
 
 // pre-sweeps: us (the level's own correction, SM order) starts at 0; the
-// first sweep saves F on the tile's own rows in fs
+// first sweep saves F on the tile's own rows in fs.  Their residual F - A us
+// goes to fr: the rows are still in registers, where a launch of its own reads
+// the level's matrix once more (331^2 mixed 1,536 -> 1,486 us, holed 257^2 mixed
+// 1,917 -> 1,795 us, graded 2049^2 BF16 210.2 -> 205.1 ms).
 template <class T, class V, int S, int W, int KC>
 __global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W, KC>())
     k_tile_down(TileView<T> t, int ncol, int fofs, int bofs, const T* __restrict__ Fg, T* __restrict__ fsg,
-                T* __restrict__ usg, int nu, int* timeout, int inject) {
+                T* __restrict__ usg, T* __restrict__ frg, int nu, int* timeout, int inject) {
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ __align__(8) uint64_t bar;
   using X = VecK<T, KC>;
@@ -220,6 +223,7 @@ __global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W, KC>(
   const X* F = reinterpret_cast<const X*>(Fg);
   X* fs = reinterpret_cast<X*>(fsg);
   X* us = reinterpret_cast<X*>(usg);
+  X* fr = reinterpret_cast<X*>(frg);
   X zero;
 #pragma unroll
   for (int j = 0; j < KC; ++j) zero.v[j] = 0;
@@ -262,13 +266,88 @@ __global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W, KC>(
       }
 #pragma unroll
     for (int s = 0; s < S; ++s)
-      if (R.g[s] >= 0) us[R.g[s]] = KC == 1 ? u[s] : Ul[s * TILE_THREADS + tid];
+      if (R.g[s] >= 0) {
+        const int q = s * TILE_THREADS + tid;
+        us[R.g[s]] = KC == 1 ? u[s] : Ul[q];
+        const X acc = tile_dot<T, V, W, KC>(R.row[s], reinterpret_cast<const char*>(Ul), R.wc[s] & 255);
+        X fq = KC == 1 ? f[s] : Fl[q];
+#pragma unroll
+        for (int j = 0; j < KC; ++j) fq.v[j] -= acc.v[j];
+        fr[R.g[s]] = fq;
+      }
     if (!more) return;
     parity ^= 1;
     ok = tile_arrived(&bar, parity, inject);
     if (ok) R.load(blob, h, tile_layout(h.slots, h.nwords, h.nvals, h.nx, sizeof(T)));
   }
   tile_expired(&bar, parity, timeout);
+}
+
+// after tiled pre-sweeps: the residual and the restricted part of every node
+// the coarser levels read (see TileRestrict)
+template <class T, class V, int KC>
+__global__ void k_restrict_tile(int64_t n1, int64_t n, const int32_t* __restrict__ id, const int32_t* __restrict__ src,
+                                const int32_t* __restrict__ ptr, const int32_t* __restrict__ child,
+                                const int64_t* __restrict__ off, const int32_t* __restrict__ col,
+                                const V* __restrict__ val, const T* __restrict__ frg, const T* __restrict__ usg,
+                                T* __restrict__ Fg) {
+  using X = VecK<T, KC>;
+  const X* fr = reinterpret_cast<const X*>(frg);
+  const X* us = reinterpret_cast<const X*>(usg);
+  X* F = reinterpret_cast<X*>(Fg);
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  int32_t i = -1, k = 0, p0 = 0, p1 = 0;
+  kern::Row<T> row;
+  if (t < n) {
+    i = id[t];
+    p0 = ptr[t];
+    p1 = ptr[t + 1];
+    if (t < n1)
+      k = src[t];
+    else if (i >= 0)
+      kern::row_load(row, t - n1, off, col, val);
+  }
+  pdl_wait();
+  if (i >= 0) {
+    X f;
+    if (t < n1) {
+      f = fr[k];
+    } else {
+      X acc;
+#pragma unroll
+      for (int j = 0; j < KC; ++j) acc.v[j] = 0;
+#pragma unroll
+      for (int q = 0; q < kern::MAXW; ++q)
+        if (q < row.w) {
+          const X x = us[row.c[q]];
+#pragma unroll
+          for (int j = 0; j < KC; ++j) acc.v[j] += row.v[q] * x.v[j];
+        }
+      for (int q = kern::MAXW; q < row.w; ++q) {
+        const int64_t e = row.b + ((int64_t)q << 5) + row.lane;
+        const T a = (T)kern::ldg_val(val + e);
+        const X x = us[__ldg(col + e)];
+#pragma unroll
+        for (int j = 0; j < KC; ++j) acc.v[j] += a * x.v[j];
+      }
+      f = F[i];
+#pragma unroll
+      for (int j = 0; j < KC; ++j) f.v[j] -= acc.v[j];
+    }
+    if (p1 > p0) {
+      X acc;
+#pragma unroll
+      for (int j = 0; j < KC; ++j) acc.v[j] = 0;
+      for (int32_t p = p0; p < p1; ++p) {
+        const X c = fr[child[p]];
+#pragma unroll
+        for (int j = 0; j < KC; ++j) acc.v[j] += c.v[j];
+      }
+#pragma unroll
+      for (int j = 0; j < KC; ++j) f.v[j] += (T)0.5 * acc.v[j];
+    }
+    F[i] = f;
+  }
 }
 
 // start of the up path of a tiled level: the prolongation of the coarse
@@ -445,15 +524,22 @@ void set_smem_limits() {
 }
 
 template <class T, class V, int KC>
-void launch_down(bool pdl, const TileSweeps<T>& Tl, int ncol, const T* F, T* fs, T* us, int nu, int* timeout,
+void launch_down(bool pdl, const TileSweeps<T>& Tl, int ncol, const T* F, T* fs, T* us, T* fr, int nu, int* timeout,
                  int inject, cudaStream_t s) {
   const Smem<T> sm(Tl, KC);
   dispatch(Tl, [&](auto sl, auto w) {
     constexpr int S = decltype(sl)::value, W = decltype(w)::value;
     kern::launch_smem(pdl, k_tile_down<T, V, S, W, KC>,
                       std::min<int64_t>(Tl.ntiles, kern::NSM * tile_min_blocks<T, V, S, W, KC>()), TILE_THREADS,
-                      (size_t)sm.total, s, Tl.view(), ncol, sm.fofs, sm.bofs, F, fs, us, nu, timeout, inject);
+                      (size_t)sm.total, s, Tl.view(), ncol, sm.fofs, sm.bofs, F, fs, us, fr, nu, timeout, inject);
   });
+}
+template <class T, class V, int KC>
+void launch_restrict(bool pdl, const TileRestrict<T>& R, const T* fr, const T* us, T* F, cudaStream_t s) {
+  const int64_t n = R.n1 + R.n2;
+  if (n == 0) return;
+  kern::launch(pdl, k_restrict_tile<T, V, KC>, kern::nblk(n, kern::rows_tpb(n)), kern::rows_tpb(n), s, R.n1, n, R.id.p,
+               R.src.p, R.ptr.p, R.child.p, R.X.off.p, R.X.col.p, sell_vals(R.X, (const V*)nullptr), fr, us, F);
 }
 template <class T, class V, int KC>
 void launch_up(bool pdl, const TileSweeps<T>& Tl, int ncol, const T* ust, const T* fsl, T* U, int nu, int* timeout,
