@@ -1405,6 +1405,7 @@ struct asmg_batch_s {
   // `per` solutions (NULL: an unused column, right-hand side 0); and the
   // branches' scalars read back
   int per = 1;
+  std::vector<int64_t> generation;  // of each handle when the graph was captured
   DBuf<double*> tab;
   PinnedBuf tab_host, back;
   ~asmg_batch_s() {
@@ -1442,6 +1443,7 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
     }
   }
   B->per = B->multi ? KRHS : 1;
+  for (auto h : B->H) B->generation.push_back(h->generation);
   const int nbranch = nprob * (B->multi ? ngroups : nrhs);
   B->tab.alloc(2 * (int64_t)B->per * nbranch);
   B->tab_host.alloc(sizeof(double*) * (size_t)B->tab.n);
@@ -1509,6 +1511,9 @@ int amg_batch_solve(asmg_batch B, const double* const* bs, double* const* us, in
   const int np = (int)B->H.size(), nr = B->nrhs;
   for (int k = 0; k < np * nr; ++k)
     if (!bs[k] || !us[k]) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null array in batch");
+  for (int p = 0; p < np; ++p)
+    if (B->H[p]->generation != B->generation[p])
+      ASMG_FAIL(ASMG_ERR_INVALID_ARG, "problem %d's coefficients changed after the batch was created", p);
   // the branches read and write the caller's device arrays through the table;
   // other arrays are staged
   const int ngroups = B->multi ? (nr + KRHS - 1) / KRHS : nr;

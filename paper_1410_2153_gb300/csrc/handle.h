@@ -177,6 +177,7 @@ struct asmg_s {
   std::vector<std::unique_ptr<asmg::Slot>> slots;
   // multiple-right-hand-side solves (slot 0 serves amg_solve_multi)
   std::vector<std::unique_ptr<asmg::MultiSlot>> mslots;
+  int64_t generation = 0;           // counts the setups of the operators (a coefficient update is one)
   int64_t bytes_iter = 0;
   asmg::Stats stats;
   int gpu_launches_per_iter = 0;
