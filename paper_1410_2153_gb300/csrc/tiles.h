@@ -283,6 +283,11 @@ __global__ void __launch_bounds__(TILE_THREADS, tile_min_blocks<T, V, S, W, KC>(
   tile_expired(&bar, parity, timeout);
 }
 
+// index lists of a row (children, places in the tiles) read before the wait on
+// the previous kernel; longer ones read the rest after it (331^2 mixed 1,487 ->
+// 1,465 us, graded 513^2 FP64 28.6 -> 28.1 ms, graded 2049^2 BF16 205.2 -> 202.7 ms)
+constexpr int AHEAD = 4;
+
 // after tiled pre-sweeps: the residual and the restricted part of every node
 // the coarser levels read (see TileRestrict)
 template <class T, class V, int KC>
@@ -297,11 +302,15 @@ __global__ void k_restrict_tile(int64_t n1, int64_t n, const int32_t* __restrict
   X* F = reinterpret_cast<X*>(Fg);
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int32_t i = -1, k = 0, p0 = 0, p1 = 0;
+  int32_t ch[AHEAD];
   kern::Row<T> row;
   if (t < n) {
     i = id[t];
     p0 = ptr[t];
     p1 = ptr[t + 1];
+#pragma unroll
+    for (int q = 0; q < AHEAD; ++q)
+      if (p0 + q < p1) ch[q] = child[p0 + q];
     if (t < n1)
       k = src[t];
     else if (i >= 0)
@@ -338,11 +347,15 @@ __global__ void k_restrict_tile(int64_t n1, int64_t n, const int32_t* __restrict
       X acc;
 #pragma unroll
       for (int j = 0; j < KC; ++j) acc.v[j] = 0;
-      for (int32_t p = p0; p < p1; ++p) {
-        const X c = fr[child[p]];
+      auto add = [&](int32_t c) {
+        const X x = fr[c];
 #pragma unroll
-        for (int j = 0; j < KC; ++j) acc.v[j] += c.v[j];
-      }
+        for (int j = 0; j < KC; ++j) acc.v[j] += x.v[j];
+      };
+#pragma unroll
+      for (int q = 0; q < AHEAD; ++q)
+        if (p0 + q < p1) add(ch[q]);
+      for (int32_t p = p0 + AHEAD; p < p1; ++p) add(child[p]);
 #pragma unroll
       for (int j = 0; j < KC; ++j) f.v[j] += (T)0.5 * acc.v[j];
     }
@@ -366,12 +379,16 @@ __global__ void k_up_init(int64_t nsm, const int32_t* __restrict__ rows, const i
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int32_t i = -1, a = -3, b = -3;
   int64_t p0 = 0, p1 = 0;
+  int32_t at[AHEAD];
   if (k < nsm) {
     i = rows[k];
     a = par0[k];
     b = par1[k];
     p0 = pos_ptr[k];
     p1 = pos_ptr[k + 1];
+#pragma unroll
+    for (int q = 0; q < AHEAD; ++q)
+      if (p0 + q < p1) at[q] = pos[p0 + q];
   }
   pdl_wait();
   if (i >= 0) {
@@ -397,11 +414,14 @@ __global__ void k_up_init(int64_t nsm, const int32_t* __restrict__ rows, const i
     const X s = reinterpret_cast<const X*>(usg)[k], f = reinterpret_cast<const X*>(fsg)[k];
 #pragma unroll
     for (int j = 0; j < KC; ++j) v.v[j] = v.v[j] + s.v[j];
-    for (int64_t q = p0; q < p1; ++q) {
-      const int32_t o = pos[q];
+    auto put = [&](int32_t o) {
       reinterpret_cast<X*>(ustg)[o] = v;
       reinterpret_cast<X*>(fslg)[o] = f;
-    }
+    };
+#pragma unroll
+    for (int q = 0; q < AHEAD; ++q)
+      if (p0 + q < p1) put(at[q]);
+    for (int64_t q = p0 + AHEAD; q < p1; ++q) put(pos[q]);
   }
 }
 
