@@ -336,7 +336,10 @@ int amg_profile_levels(asmg_handle h, const double* b, double rtol, double* out,
  *                     and may not be destroyed before it.
  *   amg_batch_solve   bs[p * nrhs + j]: float64 [nv_p] right-hand side j of
  *                     problem p; us[...]: initial guess in, solution out (host
- *                     or device arrays).  iterations, status: host int
+ *                     or device arrays).  Arrays may overlap: every input is
+ *                     read before any solution is written, and solutions are
+ *                     written in order (arrays that overlap across branches
+ *                     are staged, others used in place).  iterations, status: host int
  *                     [nprob * nrhs], the PCG steps and the per-solve status
  *                     (ASMG_OK, ASMG_NOT_CONVERGED, ASMG_ERR_BREAKDOWN).
  *                     Returns the worst status.

@@ -1416,6 +1416,44 @@ struct asmg_batch_s {
   MultiSlot& mslot(int p, int g) { return *H[p]->mslots.at(1 + g); }
 };
 
+namespace {
+// Whether the branches of a batch, which run in any order, may read and write
+// the caller's arrays where they lie: no solution meets another solution, nor a
+// right-hand side of another branch (of its own branch it may: a branch gathers
+// all its inputs before its solve).  One pass over the arrays by address, with
+// the furthest end so far of the solutions and of the right-hand sides; for the
+// latter, and for solutions met by a right-hand side, of two different branches.
+struct ArrayRange {
+  uintptr_t begin, end;
+  int branch;
+  bool out;
+};
+bool branches_apart(std::vector<ArrayRange>& R) {
+  std::sort(R.begin(), R.end(), [](const ArrayRange& a, const ArrayRange& b) { return a.begin < b.begin; });
+  struct Furthest {
+    uintptr_t end[2] = {0, 0};  // of `branch`, and of any other branch
+    int branch = -1;
+    void add(const ArrayRange& r) {
+      if (r.branch == branch) {
+        end[0] = std::max(end[0], r.end);
+      } else if (r.end > end[0]) {
+        end[1] = end[0];
+        end[0] = r.end;
+        branch = r.branch;
+      } else {
+        end[1] = std::max(end[1], r.end);
+      }
+    }
+    uintptr_t other(int b) const { return b == branch ? end[1] : end[0]; }
+  } in, out;
+  for (const ArrayRange& r : R) {
+    if (r.begin < (r.out ? std::max(out.end[0], in.other(r.branch)) : out.other(r.branch))) return false;
+    (r.out ? out : in).add(r);
+  }
+  return true;
+}
+}  // namespace
+
 extern "C" {
 
 int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rtol, void* stream, asmg_batch* out) {
@@ -1515,8 +1553,23 @@ int amg_batch_solve(asmg_batch B, const double* const* bs, double* const* us, in
     if (B->H[p]->generation != B->generation[p])
       ASMG_FAIL(ASMG_ERR_INVALID_ARG, "problem %d's coefficients changed after the batch was created", p);
   // the branches read and write the caller's device arrays through the table;
-  // other arrays are staged
+  // other arrays are staged, and every array of a call whose arrays overlap
+  // across branches: all inputs are then copied before the branches start, and
+  // the solutions after they end, in order
   const int ngroups = B->multi ? (nr + KRHS - 1) / KRHS : nr;
+  std::vector<ArrayRange> ranges;
+  ranges.reserve(2 * (size_t)np * nr);
+  for (int k = 0; k < np * nr; ++k)
+    for (bool out : {false, true}) {
+      const uintptr_t a = out ? (uintptr_t)us[k] : (uintptr_t)bs[k];
+      ranges.push_back({a, a + 8 * (uintptr_t)B->H[k / nr]->mesh.nv, k / nr * ngroups + k % nr / B->per, out});
+    }
+  const bool apart = branches_apart(ranges);
+  auto array = [&](const double* user, double* stage, int64_t n) {
+    if (apart) return const_cast<double*>(input(user, stage, n, s));
+    copy_in(stage, user, n, s);
+    return stage;
+  };
   double** tab = static_cast<double**>(B->tab_host.p);
   struct Out {
     double *user, *stage;
@@ -1535,8 +1588,8 @@ int amg_batch_solve(asmg_batch B, const double* const* bs, double* const* us, in
         if (j >= nr) continue;
         const double* b = bs[p * nr + j];
         double* u = us[p * nr + j];
-        t[c] = const_cast<double*>(input(b, vb + c * nv, nv, s));
-        t[B->per + c] = const_cast<double*>(input(u, vu + c * nv, nv, s));
+        t[c] = array(b, vb + c * nv, nv);
+        t[B->per + c] = array(u, vu + c * nv, nv);
         if (t[B->per + c] != u) staged.push_back({u, vu + c * nv, nv});
       }
     }

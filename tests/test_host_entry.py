@@ -1,0 +1,117 @@
+"""What the entry points do around the kernels, on the CPU.
+
+capi.cpp is built with g++ around `tests/host_entry_shim.cpp`: its device
+memory is host memory of a settable capacity, its graphs run their branches one
+after another, and a solve returns its right-hand side.  So calls that would
+race or read memory the library does not hold can be looked at without a GPU.
+"""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1410_2153_gb300", "csrc")
+INVALID_ARG, CUDA, OOM = -1, -5, -6
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    if not shutil.which("g++") or not os.path.exists(os.path.join(inc, "cuda_runtime.h")):
+        pytest.skip("g++ or the CUDA headers are missing")
+    out = str(tmp_path_factory.mktemp("entry") / "libentry.so")
+    # -Bsymbolic: the library's runtime calls reach the stand-in, whatever else the process has loaded
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-pthread", "-Wl,-Bsymbolic", "-I", inc,
+                           os.path.join(ROOT, "tests", "host_entry_shim.cpp"), os.path.join(CSRC, "capi.cpp"),
+                           "-o", out])
+    L = ctypes.CDLL(out)
+    L.shim_device.restype = ctypes.c_void_p
+    L.shim_device.argtypes = [ctypes.c_int64]
+    L.shim_device_free.argtypes = [ctypes.c_void_p]
+    L.shim_capacity.argtypes = [ctypes.c_int64]
+    L.shim_used.restype = ctypes.c_int64
+    L.amg_last_error.restype = ctypes.c_char_p
+    L.amg_destroy.argtypes = L.amg_batch_destroy.argtypes = [ctypes.c_void_p]
+    L.amg_destroy.restype = L.amg_batch_destroy.restype = None
+    yield L
+    L.shim_capacity(-1)
+
+
+class Device:
+    """A device array of the stand-in runtime; `.a` views it."""
+
+    def __init__(self, lib, values):
+        values = np.asarray(values, np.float64)
+        self.lib, self.p = lib, lib.shim_device(values.size)
+        assert self.p
+        self.a = np.ctypeslib.as_array(ctypes.cast(self.p, ctypes.POINTER(ctypes.c_double)), (values.size,))
+        self.a[:] = values
+
+    def __del__(self):
+        self.lib.shim_device_free(self.p)
+
+
+def vp(a, offset=0):
+    return ctypes.c_void_p((a.p if isinstance(a, Device) else a.ctypes.data) + 8 * offset)
+
+
+def setup(lib, m, coeff=None):
+    h = ctypes.c_void_p()
+    rc = lib.amg_setup(2, ctypes.c_int64(m.nv), vp(m.verts), ctypes.c_int64(m.ne), vp(m.elems), vp(m.bflag),
+                       None if coeff is None else vp(coeff), None, None, ctypes.byref(h))
+    assert rc == 0, lib.amg_last_error()
+    return h
+
+
+def batch_create(lib, handles, nrhs):
+    b = ctypes.c_void_p()
+    rc = lib.amg_batch_create(len(handles), (ctypes.c_void_p * len(handles))(*[h.value for h in handles]), nrhs,
+                              ctypes.c_double(1e-8), None, ctypes.byref(b))
+    assert rc == 0, lib.amg_last_error()
+    return b
+
+
+def batch_solve(lib, batch, bs, us):
+    n = len(bs)
+    its = (ctypes.c_int * n)()
+    return lib.amg_batch_solve(batch, (ctypes.c_void_p * n)(*[p.value for p in bs]),
+                               (ctypes.c_void_p * n)(*[p.value for p in us]), its, None, None)
+
+
+# Arrays of a batched call, in units of nv: (bs, us) offsets into one device
+# allocation.  Every right-hand side and guess is taken before any solution is
+# written, and of two solutions written to one place the later one stays.
+OVERLAPS = {
+    "u0 on b1": (lambda k: ([0] + [10 + j for j in range(1, k)], [11] + [20 + j for j in range(1, k)])),
+    "u0 on half of b1": (lambda k: ([0] + [10 + 2 * j for j in range(1, k)], [12.5] + [30 + j for j in range(1, k)])),
+    "last u on b0": (lambda k: ([5 + j for j in range(k)], [20 + j for j in range(k - 1)] + [5])),
+    "one u for all": (lambda k: ([j for j in range(k)], [15] * k)),
+    "shifted us": (lambda k: ([j for j in range(k)], [15 + 0.5 * j for j in range(k)])),
+    "u on its own b": (lambda k: ([j for j in range(k)], [j for j in range(k)])),
+    "one b for all": (lambda k: ([3] * k, [10 + j for j in range(k)])),
+    "apart": (lambda k: ([j for j in range(k)], [20 + j for j in range(k)])),
+}
+
+
+@pytest.mark.parametrize("name", OVERLAPS)
+@pytest.mark.parametrize("nprob,nrhs", [(2, 1), (1, 3), (2, 3), (1, 6)])
+def test_batched_arrays_may_overlap(lib, gen, nprob, nrhs, name):
+    k = nprob * nrhs
+    m = gen.grid2d(5, 1)
+    handles = [setup(lib, m) for _ in range(nprob)]
+    batch = batch_create(lib, handles, nrhs)
+    ob, ou = ([int(o * m.nv) for o in off] for off in OVERLAPS[name](k))
+    mem = Device(lib, np.random.default_rng(5).uniform(1, 2, 45 * m.nv))
+    want = mem.a.copy()
+    sols = [np.where(m.bflag == 0, want[o:o + m.nv], 0) for o in ob]
+    for o, u in zip(ou, sols):
+        want[o:o + m.nv] = u
+    assert batch_solve(lib, batch, [vp(mem, o) for o in ob], [vp(mem, o) for o in ou]) == 0
+    assert np.array_equal(mem.a, want)
+    lib.amg_batch_destroy(batch)
+    for h in handles:
+        lib.amg_destroy(h)
