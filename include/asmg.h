@@ -223,7 +223,12 @@ int amg_set_log_coefficients(asmg_handle h, const double* g, void* stream);
  * Replace the element coefficients (float64 [ne], > 0) and rebuild every
  * operator that depends on them (fine A, auxiliary operators, coarse
  * inverse).  The tree, the auxiliary grids, the transfer and the colourings
- * depend on geometry only and are kept.
+ * depend on geometry only and are kept.  A coefficient that is not positive
+ * and finite is refused before anything changes.  When the rebuild itself
+ * fails (device memory, a coarsest matrix that is not positive definite in
+ * FP64), the old operators are gone: every call that takes the handle returns
+ * ASMG_ERR_INVALID_ARG until an update succeeds.  Batches made before an
+ * update are refused after it (amg_batch_solve).
  */
 int amg_update_coefficients(asmg_handle h, const double* coeff, void* stream);
 
@@ -342,7 +347,10 @@ int amg_profile_levels(asmg_handle h, const double* b, double rtol, double* out,
  *                     are staged, others used in place).  iterations, status: host int
  *                     [nprob * nrhs], the PCG steps and the per-solve status
  *                     (ASMG_OK, ASMG_NOT_CONVERGED, ASMG_ERR_BREAKDOWN).
- *                     Returns the worst status.
+ *                     Returns the worst status.  ASMG_ERR_INVALID_ARG after
+ *                     a coefficient update of one of its handles, successful
+ *                     or not (the graph holds the operators it was captured
+ *                     with): create the batch anew.
  */
 typedef struct asmg_batch_s* asmg_batch;
 int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rtol, void* stream, asmg_batch* out);

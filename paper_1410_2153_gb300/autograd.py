@@ -36,12 +36,14 @@ class CoefficientSolver:
     def set_coefficients(self, coeff: torch.Tensor):
         c = coeff.detach().to(torch.float64).contiguous()
         if self._changed("a", c):
+            self._set = None      # a failed update leaves the handle without operators
             asmg.amg_update_coefficients(self.solver.h, c)
             self._set = ("a", c.clone())
 
     def set_log_coefficients(self, g: torch.Tensor):
         c = g.detach().to(torch.float64).contiguous()
         if self._changed("g", c):
+            self._set = None
             asmg.amg_set_log_coefficients(self.solver.h, c)
             self._set = ("g", c.clone())
 

@@ -1195,6 +1195,7 @@ void build_all(asmg_s& h, cudaStream_t s) {
   ASMG_CUDA(cudaStreamSynchronize(s));
   h.stats.t_slots = now() - tg;
   h.stats.t_levels = now() - t2;
+  h.ready = true;
 }
 
 // algorithmic bytes of one PCG iteration (compulsory traffic, real non-zeros)
@@ -1469,6 +1470,7 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
   B->multi = nrhs > 1;
   for (auto h : B->H) {
     if (!h) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null handle in batch");
+    h->check_ready();
     if (!multi_supported(*h)) B->multi = false;
   }
   const int ngroups = (nrhs + KRHS - 1) / KRHS;
@@ -1639,6 +1641,7 @@ void amg_batch_destroy(asmg_batch B) { delete B; }
 int amg_residual_norm_noalloc(asmg_handle h, const double* b, const double* u, double* out, void* stream) {
   API_BEGIN
   if (!h || !b || !u || !out) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null argument");
+  h->check_ready();
   residual_norm_noalloc(*h, b, u, out, (cudaStream_t)stream);
   return ASMG_OK;
   API_END
@@ -1717,6 +1720,7 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
                     double* res_history, void* stream) {
   API_BEGIN
   if (!h || !b || !u || !iterations) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null argument");
+  h->check_ready();
   if (k < 1 || k > KRHS) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "k = %d right-hand sides (1..%d)", k, KRHS);
   if (!(rtol >= 0) || !std::isfinite(rtol)) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "rtol must be finite and >= 0");
   if (!multi_supported(*h))
@@ -1871,6 +1875,12 @@ void set_coefficients(asmg_handle h, std::vector<double> c, cudaStream_t s) {
   for (int64_t e = 0; e < h->mesh.ne; ++e)
     if (!(c[e] > 0) || !std::isfinite(c[e]))
       ASMG_FAIL(ASMG_ERR_BAD_MESH, "coefficient of element %lld is not positive and finite", (long long)e);
+  // from here on the old operators go: with them the work state and graphs that
+  // point at them, and the handle's use until the new ones are complete
+  h->ready = false;
+  ++h->generation;
+  h->slots.clear();
+  h->mslots.clear();
   h->mesh.coeff = std::move(c);
   h->dCoeff.upload(h->mesh.coeff, s);
   build_all(*h, s);
@@ -1922,6 +1932,7 @@ int amg_update_coefficients(asmg_handle h, const double* coeff, void* stream) {
 int amg_info(asmg_handle h, int what, int level, int64_t* value) {
   API_BEGIN
   if (!h || !value) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null argument");
+  h->check_ready();
   auto lev_index = [&](int l) -> int {
     int k = l - (h->aux.c + 1);
     if (k < 0 || k >= (int)h->aux.levels.size()) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "level %d has no smoothing data", l);
@@ -2017,6 +2028,7 @@ int amg_info(asmg_handle h, int what, int level, int64_t* value) {
 int amg_export(asmg_handle h, int what, int level, void* buf, int64_t* count) {
   API_BEGIN
   if (!h || !count) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "null argument");
+  h->check_ready();
   cudaStream_t s = 0;
   auto put = [&](const void* src, int64_t n, size_t elem) {
     *count = n;

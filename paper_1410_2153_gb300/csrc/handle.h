@@ -177,12 +177,19 @@ struct asmg_s {
   std::vector<std::unique_ptr<asmg::Slot>> slots;
   // multiple-right-hand-side solves (slot 0 serves amg_solve_multi)
   std::vector<std::unique_ptr<asmg::MultiSlot>> mslots;
-  int64_t generation = 0;           // counts the setups of the operators (a coefficient update is one)
+  int64_t generation = 0;           // counts the changes of the operators (a coefficient update is one, failed or not)
+  bool ready = false;               // the operators are complete: false from the start of a change to its success
   int64_t bytes_iter = 0;
   asmg::Stats stats;
   int gpu_launches_per_iter = 0;
 
-  asmg::Slot& slot0() { return *slots.at(0); }
+  void check_ready() const {
+    if (!ready) ASMG_FAIL(ASMG_ERR_INVALID_ARG, "the handle has no operators: its last coefficient update failed");
+  }
+  asmg::Slot& slot0() {
+    check_ready();
+    return *slots.at(0);
+  }
 };
 
 namespace asmg {

@@ -1580,10 +1580,6 @@ void setup_solve(asmg_s& h, cudaStream_t s) {
     setup_small(h.p64, false, s);
     drop_unused_tiles(h.p64);
   }
-  // work state and graphs of an earlier setup point at its operators
-  h.slots.clear();
-  h.mslots.clear();
-  ++h.generation;
   add_slot(h, s);
   if (h.prm.tile_rows == 0 && !h.prm.inject_timeout) {
     if (h.prm.precision == ASMG_MIXED)

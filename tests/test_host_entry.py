@@ -115,3 +115,82 @@ def test_batched_arrays_may_overlap(lib, gen, nprob, nrhs, name):
     lib.amg_batch_destroy(batch)
     for h in handles:
         lib.amg_destroy(h)
+
+
+GOOD, FAILS = 1.5, 1e200          # the stand-in's coarsest matrix is not positive definite above 1e100
+
+
+def update(lib, h, m, value, log=False):
+    a = np.full(m.ne, value)
+    return lib.amg_set_log_coefficients(h, vp(np.log(a)), None) if log else lib.amg_update_coefficients(h, vp(a), None)
+
+
+@pytest.mark.parametrize("log", [False, True])
+def test_a_failed_update_leaves_no_operators_behind(lib, gen, log):
+    m = gen.grid2d(5, 1)
+    h = setup(lib, m)
+    one, many = batch_create(lib, [h], 1), batch_create(lib, [h], 2)
+    b, u = np.ones(3 * m.nv), np.zeros(3 * m.nv)
+    g, its = np.zeros(m.ne), (ctypes.c_int * 4)()
+    prof, val, count = np.zeros(64), ctypes.c_int64(), ctypes.c_int64()
+    rtol = ctypes.c_double(1e-8)
+    calls = {
+        "solve": lambda: lib.amg_solve(h, vp(b), vp(u), rtol, its, None, None),
+        "multi": lambda: lib.amg_solve_multi(h, 2, vp(b), vp(u), rtol, its, None, None, None),
+        "precond": lambda: lib.amg_precond_apply(h, vp(b), vp(u), None),
+        "spmv": lambda: lib.amg_spmv(h, vp(b), vp(u), None),
+        "mass": lambda: lib.amg_mass_apply(h, vp(b), vp(u), None),
+        "grad": lambda: lib.amg_element_grad(h, vp(b), vp(u), vp(g), None),
+        "grad_log": lambda: lib.amg_element_grad_log(h, vp(b), vp(u), vp(g), None),
+        "residual": lambda: lib.amg_residual_norm_noalloc(h, vp(b), vp(u), vp(prof), None),
+        "profile": lambda: lib.amg_profile(h, vp(b), rtol, vp(prof), its, None),
+        "profile_levels": lambda: lib.amg_profile_levels(h, vp(b), rtol, vp(prof), vp(prof), 1, its, None),
+        "info": lambda: lib.amg_info(h, 0, 0, ctypes.byref(val)),
+        "export": lambda: lib.amg_export(h, 8, 0, None, ctypes.byref(count)),
+        "batch_create": lambda: lib.amg_batch_create(1, (ctypes.c_void_p * 1)(h.value), 1, rtol, None, ctypes.byref(ctypes.c_void_p())),
+    }
+    batches = {"batch": lambda: batch_solve(lib, one, [vp(b)], [vp(u)]),
+               "batch of two": lambda: batch_solve(lib, many, [vp(b)] * 2, [vp(u), vp(u, m.nv)])}
+    for name, f in {**calls, **batches}.items():
+        if name != "batch_create":
+            assert f() == 0, (name, lib.amg_last_error())
+    assert update(lib, h, m, -1.0) < 0 if not log else True      # refused before anything changes:
+    assert calls["solve"]() == 0                                  # the handle keeps its operators
+    assert update(lib, h, m, FAILS, log) == CUDA
+    solves = lib.shim_solves()
+    for name, f in {**calls, **batches}.items():
+        assert f() == INVALID_ARG, name
+    assert lib.shim_solves() == solves
+    assert update(lib, h, m, GOOD, log) == 0
+    for name, f in calls.items():
+        if name != "batch_create":
+            assert f() == 0, (name, lib.amg_last_error())
+    for name, f in batches.items():                               # captured before the updates
+        assert f() == INVALID_ARG, name
+    lib.amg_batch_destroy(one)
+    lib.amg_batch_destroy(many)
+    lib.amg_destroy(h)
+
+
+def test_a_failed_update_is_not_taken_for_the_coefficients_held(monkeypatch):
+    torch = pytest.importorskip("torch")
+    from paper_1410_2153_gb300 import asmg, autograd
+    cs = autograd.CoefficientSolver.__new__(autograd.CoefficientSolver)
+    cs.solver, cs._set = type("S", (), {"h": None})(), None
+    held = []
+
+    def set_(h, c):
+        held.append(None)
+        if float(c[0]) > 1e100:
+            raise asmg.AsmgError(CUDA, "update failed")
+        held[-1] = float(c[0])
+
+    monkeypatch.setattr(asmg, "amg_update_coefficients", set_)
+    monkeypatch.setattr(asmg, "amg_set_log_coefficients", set_)
+    for call in (cs.set_coefficients, cs.set_log_coefficients):
+        good = torch.ones(3, dtype=torch.float64)
+        call(good)
+        with pytest.raises(asmg.AsmgError):
+            call(good * 1e200)
+        call(good)
+        assert held[-1] == 1.0
