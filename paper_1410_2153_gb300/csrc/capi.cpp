@@ -896,6 +896,7 @@ void build_prec(asmg_s& h, Prec<T>& P, const HostCSR& Aperm, const std::vector<d
     sell_build<T>(P.Up, half(false), 0, s);
   }
   if (keep_transfer) return;
+  h.transfer_rows.clear();
   // transfer P (rows: permuted fine rows) and P^T (rows: aux nodes), built
   // by counting sort into flat CSR arrays; each row sorted by column
   const Triplets& Tp = h.aux.P;
@@ -936,6 +937,7 @@ void build_prec(asmg_s& h, Prec<T>& P, const HostCSR& Aperm, const std::vector<d
   HostCSR Pc = to_csr(h.npad, h.nJpad, false), Ptc = to_csr(h.nJpad, h.npad, true);
   sell_build<T>(P.P, Pc, 0, s);
   sell_build<T>(P.PT, Ptc, 0, s);
+  h.transfer_rows = h.row_of_free;
 }
 
 // Colouring option 2 on an auxiliary level: the lattice parity of each node
@@ -1020,7 +1022,6 @@ void build_all(asmg_s& h, cudaStream_t s) {
     }
   }
   h.npad = (int64_t)sel.size();
-  const std::vector<int32_t> old_rows = std::move(h.row_of_free);
   h.row_of_free.assign(h.n, -1);
   std::vector<int32_t> vrow(h.npad, -1), rowv(nv, -1);
   for (int64_t k = 0; k < h.npad; ++k)
@@ -1053,7 +1054,7 @@ void build_all(asmg_s& h, cudaStream_t s) {
   // the transfer depends on the geometry only: a coefficient update keeps it,
   // and its device form too while the fine rows keep their order
   Triplets kept = std::move(h.aux.P);
-  const bool same_rows = !kept.r.empty() && h.row_of_free == old_rows;
+  const bool same_rows = !kept.r.empty() && h.row_of_free == h.transfer_rows;
   h.aux = AuxHost();
   if (m.dim == 2)
     build_aux_host(m, h.tree, h.prm, h.aux);

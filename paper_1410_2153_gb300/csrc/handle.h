@@ -155,6 +155,7 @@ struct asmg_s {
   // fine grid
   int64_t n = 0, npad = 0;
   std::vector<int32_t> free_of_vertex, vertex_of_free, fine_colour, row_of_free;
+  std::vector<int32_t> transfer_rows;    // the row_of_free that the device P and P^T were built for
   std::vector<int64_t> fine_cstart;      // colour blocks in permuted rows (multiples of 32)
   std::vector<int64_t> fine_cnnz, fine_crows;  // real non-zeros / rows per colour block
   std::vector<int64_t> fine_lnnz;              // real non-zeros of Prec::Lo per colour block

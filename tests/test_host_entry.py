@@ -194,3 +194,21 @@ def test_a_failed_update_is_not_taken_for_the_coefficients_held(monkeypatch):
             call(good * 1e200)
         call(good)
         assert held[-1] == 1.0
+
+
+def test_the_transfer_follows_the_row_order_after_a_failed_update(lib, gen):
+    # two colour classes from 2 on: the failed update orders the fine rows as the next good one does
+    m = gen.grid2d(5, 1)
+    h, fresh = setup(lib, m, np.full(m.ne, GOOD)), setup(lib, m, np.full(m.ne, 3.0))
+    assert update(lib, h, m, FAILS) == CUDA
+    assert update(lib, h, m, 3.0) == 0
+    lib.shim_transfer.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    lib.shim_transfer.restype = ctypes.c_int64
+    rows = []
+    for x in (h, fresh):
+        v = np.full(lib.shim_transfer(x, None), -1.0)
+        lib.shim_transfer(x, vp(v))
+        rows.append(v)
+    assert rows[1].size == 64 and np.array_equal(*rows)
+    lib.amg_destroy(h)
+    lib.amg_destroy(fresh)
