@@ -1778,10 +1778,17 @@ int amg_mass_apply(asmg_handle h, const double* f, double* bout, void* stream) {
     std::vector<int64_t> fill(ptr.begin(), ptr.end() - 1);
     for (int64_t e = 0; e < m.ne; ++e)
       for (int k = 0; k < nvert; ++k) el[fill[m.E[e * nvert + k]]++] = (int32_t)e;
-    h->d_v2e_ptr.upload(ptr, s);
-    h->d_v2e.upload(el, s);
-    h->d_elem_mass.alloc(m.ne);
-    element_mass_gpu(m.dim, m.ne, h->dX.p, h->dE.p, h->d_elem_mass.p, s);
+    // the handle takes the three arrays together: without all of them the next call builds them
+    DBuf<int64_t> dptr;
+    DBuf<int32_t> del;
+    DBuf<double> dw;
+    dptr.upload(ptr, s);
+    del.upload(el, s);
+    dw.alloc(m.ne);
+    element_mass_gpu(m.dim, m.ne, h->dX.p, h->dE.p, dw.p, s);
+    h->d_v2e_ptr = std::move(dptr);
+    h->d_v2e = std::move(del);
+    h->d_elem_mass = std::move(dw);
   }
   // the result goes straight to the caller's array unless it overlaps the input
   const bool overlap = (uintptr_t)f < (uintptr_t)(bout + nv) && (uintptr_t)bout < (uintptr_t)(f + nv);
@@ -1853,7 +1860,6 @@ void element_grad_common(asmg_handle h, const double* u, const double* lambda, d
     } catch (const Error& e) {
       h->d_elem_stiff.release();
       if (e.code != ASMG_ERR_OOM) throw;
-      cudaGetLastError();
     }
   }
   // (u, lambda) per vertex, Dirichlet entries 0

@@ -25,9 +25,11 @@ struct Error {
 #define ASMG_CUDA(call)                                                                          \
   do {                                                                                           \
     cudaError_t e_ = (call);                                                                     \
-    if (e_ != cudaSuccess)                                                                       \
+    if (e_ != cudaSuccess) {                                                                     \
+      (void)cudaGetLastError(); /* reported here: the next launch check must not see it again */ \
       throw ::asmg::Error{e_ == cudaErrorMemoryAllocation ? ASMG_ERR_OOM : ASMG_ERR_CUDA,        \
                           std::string(#call) + ": " + cudaGetErrorString(e_)};                   \
+    }                                                                                            \
   } while (0)
 
 #define ASMG_FAIL(code, ...)                                                                     \
@@ -58,8 +60,8 @@ struct DBuf {
   }
   void alloc(int64_t count) {
     release();
-    n = count;
     if (count > 0) ASMG_CUDA(cudaMalloc((void**)&p, sizeof(T) * (size_t)count));
+    n = count;
   }
   void zero(cudaStream_t s) {
     if (n) ASMG_CUDA(cudaMemsetAsync(p, 0, sizeof(T) * (size_t)n, s));

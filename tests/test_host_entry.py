@@ -212,3 +212,19 @@ def test_the_transfer_follows_the_row_order_after_a_failed_update(lib, gen):
     assert rows[1].size == 64 and np.array_equal(*rows)
     lib.amg_destroy(h)
     lib.amg_destroy(fresh)
+
+
+def test_a_mass_product_after_one_that_ran_out_of_memory(lib, gen):
+    # the first call builds three arrays: each of their allocations fails once
+    m = gen.grid2d(6, 1)
+    f, row = np.arange(1.0, m.nv + 1), m.bflag == 0          # whole numbers: exact sums
+    want = np.where(row, f * np.bincount(m.elems.ravel(), minlength=m.nv), 0)
+    for room in (0, 8 * (m.nv + 1), 8 * (m.nv + 1) + 4 * 3 * m.ne):
+        h, b = setup(lib, m), np.zeros(m.nv)
+        faults = lib.shim_faults()
+        lib.shim_capacity(lib.shim_used() + room)
+        assert lib.amg_mass_apply(h, vp(f), vp(b), None) == OOM
+        lib.shim_capacity(-1)
+        assert lib.amg_mass_apply(h, vp(f), vp(b), None) == 0, lib.amg_last_error()
+        assert lib.shim_faults() == faults and np.array_equal(b, want)
+        lib.amg_destroy(h)
