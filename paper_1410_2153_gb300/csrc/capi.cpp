@@ -1225,6 +1225,18 @@ int64_t iteration_bytes(const asmg_s& h, const Prec<T>& P) {
   return b;
 }
 
+// Adds a work state to a handle's; one that ran out of device memory half-way goes again.
+template <class V, class F>
+void grow(V& states, F add) {
+  const size_t n = states.size();
+  try {
+    add();
+  } catch (...) {
+    states.resize(n);
+    throw;
+  }
+}
+
 int finish(int rc) { return rc; }
 
 }  // namespace
@@ -1477,10 +1489,9 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
   const int ngroups = (nrhs + KRHS - 1) / KRHS;
   for (auto h : B->H) {
     if (B->multi) {
-      if (h->mslots.empty()) add_multi_slot(*h, s);
-      while ((int)h->mslots.size() < 1 + ngroups) add_multi_slot(*h, s);
+      while ((int)h->mslots.size() < 1 + ngroups) grow(h->mslots, [&] { add_multi_slot(*h, s); });
     } else {
-      while ((int)h->slots.size() < 1 + nrhs) add_slot(*h, s);
+      while ((int)h->slots.size() < 1 + nrhs) grow(h->slots, [&] { add_slot(*h, s); });
     }
   }
   B->per = B->multi ? KRHS : 1;
@@ -1728,7 +1739,7 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
     ASMG_FAIL(ASMG_ERR_UNSUPPORTED, "multiple right-hand sides need the multiplicative Gauss-Seidel PCG without "
                                     "Neumann vertices");
   cudaStream_t s = (cudaStream_t)stream;
-  if (h->mslots.empty()) add_multi_slot(*h, s);
+  if (h->mslots.empty()) grow(h->mslots, [&] { add_multi_slot(*h, s); });
   MultiSlot& S = *h->mslots[0];
   const int64_t nv = h->mesh.nv;
   const bool direct = in_place(u);

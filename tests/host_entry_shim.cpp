@@ -22,7 +22,7 @@ using namespace asmg;
 namespace {
 std::map<char*, size_t> g_live;
 std::set<char*> g_host;  // page-locked
-size_t g_used = 0, g_capacity = SIZE_MAX;
+size_t g_used = 0, g_peak = 0, g_capacity = SIZE_MAX;
 cudaError_t g_last = cudaSuccess;
 int g_faults = 0, g_solves = 0;
 double g_coef0 = 1;  // the coefficient of element 0 at the last assembly
@@ -65,6 +65,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
   *p = std::aligned_alloc(256, (n + 255) / 256 * 256);
   g_live[(char*)*p] = n;
   g_used += n;
+  g_peak = std::max(g_peak, g_used);
   return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {
@@ -81,6 +82,7 @@ cudaError_t cudaFreeHost(void* p) {
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  if (!d || !s) return ++g_faults, cudaErrorInvalidValue;
   std::memmove(d, s, n);
   return cudaSuccess;
 }
@@ -253,11 +255,13 @@ void residual_norm_noalloc(asmg_s&, const double*, const double*, double*, cudaS
 
 // column j of k interleaved ones
 static void gather_col(asmg_s& h, const double* src, double* dst, int j, int k) {
+  if (!readable(dst)) return;
   for (int64_t i = 0; i < h.npad; ++i) dst[i * k + j] = 0;
   for (int64_t v = 0; src && v < h.mesh.nv; ++v)
     if (h.d_row_of_vertex.p[v] >= 0) dst[(int64_t)h.d_row_of_vertex.p[v] * k + j] = src[v];
 }
 static void scatter_col(asmg_s& h, const double* src, double* dst, int j, int k) {
+  if (!readable(src)) return;
   for (int64_t v = 0; dst && v < h.mesh.nv; ++v)
     dst[v] = h.d_row_of_vertex.p[v] >= 0 ? src[(int64_t)h.d_row_of_vertex.p[v] * k + j] : 0;
 }
@@ -332,6 +336,12 @@ double* shim_device(int64_t n) {
 }
 void shim_device_free(double* p) { cudaFree(p); }
 int64_t shim_used() { return (int64_t)g_used; }
+// the most bytes held since the last call; starts anew from what is held now
+int64_t shim_peak() {
+  const size_t p = g_peak;
+  g_peak = g_used;
+  return (int64_t)p;
+}
 void shim_capacity(int64_t bytes) { g_capacity = bytes < 0 ? SIZE_MAX : (size_t)bytes; }
 int shim_faults() { return g_faults; }
 int shim_solves() { return g_solves; }

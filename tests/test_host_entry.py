@@ -33,7 +33,7 @@ def lib(tmp_path_factory):
     L.shim_device.argtypes = [ctypes.c_int64]
     L.shim_device_free.argtypes = [ctypes.c_void_p]
     L.shim_capacity.argtypes = [ctypes.c_int64]
-    L.shim_used.restype = ctypes.c_int64
+    L.shim_used.restype = L.shim_peak.restype = ctypes.c_int64
     L.amg_last_error.restype = ctypes.c_char_p
     L.amg_destroy.argtypes = L.amg_batch_destroy.argtypes = [ctypes.c_void_p]
     L.amg_destroy.restype = L.amg_batch_destroy.restype = None
@@ -121,8 +121,8 @@ GOOD, FAILS = 1.5, 1e200          # the stand-in's coarsest matrix is not positi
 
 
 def update(lib, h, m, value, log=False):
-    a = np.full(m.ne, value)
-    return lib.amg_set_log_coefficients(h, vp(np.log(a)), None) if log else lib.amg_update_coefficients(h, vp(a), None)
+    a = np.log(np.full(m.ne, value)) if log else np.full(m.ne, value)
+    return (lib.amg_set_log_coefficients if log else lib.amg_update_coefficients)(h, vp(a), None)
 
 
 @pytest.mark.parametrize("log", [False, True])
@@ -228,3 +228,28 @@ def test_a_mass_product_after_one_that_ran_out_of_memory(lib, gen):
         assert lib.amg_mass_apply(h, vp(f), vp(b), None) == 0, lib.amg_last_error()
         assert lib.shim_faults() == faults and np.array_equal(b, want)
         lib.amg_destroy(h)
+
+
+@pytest.mark.parametrize("where", ["multi", "batch", "batch of two"])
+def test_work_state_that_ran_out_of_memory_is_not_used(lib, gen, where):
+    # device memory for a part of the work state only, at the first call
+    m = gen.grid2d(5, 1)
+    h, x, y, its = setup(lib, m), np.ones(2 * m.nv), np.zeros(2 * m.nv), (ctypes.c_int * 4)()
+    rtol, batch, n = ctypes.c_double(1e-8), ctypes.c_void_p(), 2 if where == "batch of two" else 1
+
+    def call():
+        if where == "multi":
+            return lib.amg_solve_multi(h, 2, vp(x), vp(y), rtol, its, None, None, None)
+        return lib.amg_batch_create(1, (ctypes.c_void_p * 1)(h.value), n, rtol, None, ctypes.byref(batch))
+
+    faults = lib.shim_faults()
+    lib.shim_capacity(lib.shim_used() + 8 * 4 * 32)
+    assert call() == OOM
+    lib.shim_capacity(-1)
+    assert call() == 0, lib.amg_last_error()
+    if where != "multi":
+        assert batch_solve(lib, batch, [vp(x, j * m.nv) for j in range(n)], [vp(y, j * m.nv) for j in range(n)]) == 0
+        lib.amg_batch_destroy(batch)
+    assert lib.shim_faults() == faults
+    assert np.array_equal(y[:m.nv], m.bflag == 0)
+    lib.amg_destroy(h)
