@@ -1225,6 +1225,19 @@ int64_t iteration_bytes(const asmg_s& h, const Prec<T>& P) {
   return b;
 }
 
+// f() with the device memory it needs: when that runs out, again without the
+// handle's element stiffness, which the gradients can do without.
+template <class F>
+void with_room(asmg_s& h, F f) {
+  try {
+    f();
+  } catch (const Error& e) {
+    if (e.code != ASMG_ERR_OOM || !h.d_elem_stiff.p) throw;
+    h.d_elem_stiff.release();
+    f();
+  }
+}
+
 // Adds a work state to a handle's; one that ran out of device memory half-way goes again.
 template <class V, class F>
 void grow(V& states, F add) {
@@ -1489,9 +1502,9 @@ int amg_batch_create(int nprob, const asmg_handle* handles, int nrhs, double rto
   const int ngroups = (nrhs + KRHS - 1) / KRHS;
   for (auto h : B->H) {
     if (B->multi) {
-      while ((int)h->mslots.size() < 1 + ngroups) grow(h->mslots, [&] { add_multi_slot(*h, s); });
+      while ((int)h->mslots.size() < 1 + ngroups) with_room(*h, [&] { grow(h->mslots, [&] { add_multi_slot(*h, s); }); });
     } else {
-      while ((int)h->slots.size() < 1 + nrhs) grow(h->slots, [&] { add_slot(*h, s); });
+      while ((int)h->slots.size() < 1 + nrhs) with_room(*h, [&] { grow(h->slots, [&] { add_slot(*h, s); }); });
     }
   }
   B->per = B->multi ? KRHS : 1;
@@ -1739,7 +1752,7 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
     ASMG_FAIL(ASMG_ERR_UNSUPPORTED, "multiple right-hand sides need the multiplicative Gauss-Seidel PCG without "
                                     "Neumann vertices");
   cudaStream_t s = (cudaStream_t)stream;
-  if (h->mslots.empty()) grow(h->mslots, [&] { add_multi_slot(*h, s); });
+  if (h->mslots.empty()) with_room(*h, [&] { grow(h->mslots, [&] { add_multi_slot(*h, s); }); });
   MultiSlot& S = *h->mslots[0];
   const int64_t nv = h->mesh.nv;
   const bool direct = in_place(u);
@@ -1793,9 +1806,11 @@ int amg_mass_apply(asmg_handle h, const double* f, double* bout, void* stream) {
     DBuf<int64_t> dptr;
     DBuf<int32_t> del;
     DBuf<double> dw;
-    dptr.upload(ptr, s);
-    del.upload(el, s);
-    dw.alloc(m.ne);
+    with_room(*h, [&] {
+      dptr.upload(ptr, s);
+      del.upload(el, s);
+      dw.alloc(m.ne);
+    });
     element_mass_gpu(m.dim, m.ne, h->dX.p, h->dE.p, dw.p, s);
     h->d_v2e_ptr = std::move(dptr);
     h->d_v2e = std::move(del);
@@ -1861,8 +1876,15 @@ void element_grad_common(asmg_handle h, const double* u, const double* lambda, d
                          cudaStream_t s) {
   Slot& S0 = h->slot0();
   const int64_t nv = h->mesh.nv, ne = h->mesh.ne;
+  DBuf<double> dg;
+  const bool dev = in_place(g);
+  with_room(*h, [&] {
+    if (!h->d_pair.p) h->d_pair.alloc(2 * nv);
+    if (!dev) dg.alloc(ne);
+  });
+  double* out = dev ? g : dg.p;
   if (!h->d_elem_stiff.p && !h->elem_stiff_tried) {
-    // element stiffness (a = 1), kept for the handle's life where memory allows:
+    // element stiffness (a = 1), kept while nothing else needs its memory:
     // recomputing it bounds the gradient by the FP64 units
     h->elem_stiff_tried = true;
     try {
@@ -1874,15 +1896,7 @@ void element_grad_common(asmg_handle h, const double* u, const double* lambda, d
     }
   }
   // (u, lambda) per vertex, Dirichlet entries 0
-  if (!h->d_pair.p) h->d_pair.alloc(2 * nv);
   mask_pair(*h, input(u, S0.vb.p, nv, s), input(lambda, S0.vu.p, nv, s), h->d_pair.p, s);
-  DBuf<double> dg;
-  const bool dev = in_place(g);
-  double* out = g;
-  if (!dev) {
-    dg.alloc(ne);
-    out = dg.p;
-  }
   element_grad_gpu(h->mesh.dim, ne, h->dX.p, h->dE.p, h->d_elem_stiff.p, h->d_pair.p,
                    log_coeff ? h->dCoeff.p : nullptr, out, s);
   if (!dev) copy_out(g, dg.p, ne, s);
@@ -1900,8 +1914,10 @@ void set_coefficients(asmg_handle h, std::vector<double> c, cudaStream_t s) {
   h->slots.clear();
   h->mslots.clear();
   h->mesh.coeff = std::move(c);
-  h->dCoeff.upload(h->mesh.coeff, s);
-  build_all(*h, s);
+  with_room(*h, [&] {
+    h->dCoeff.upload(h->mesh.coeff, s);
+    build_all(*h, s);
+  });
   h->bytes_iter = h->prm.precision == ASMG_MIXED ? iteration_bytes(*h, h->p32) : iteration_bytes(*h, h->p64);
 }
 }  // namespace

@@ -253,3 +253,41 @@ def test_work_state_that_ran_out_of_memory_is_not_used(lib, gen, where):
     assert lib.shim_faults() == faults
     assert np.array_equal(y[:m.nv], m.bflag == 0)
     lib.amg_destroy(h)
+
+
+@pytest.mark.parametrize("where", ["gradient", "mass", "multi", "batch", "update"])
+def test_the_kept_element_stiffness_gives_way(lib, gen, where):
+    # device memory for what a call cannot do without, not for the optional element stiffness beside it
+    m = gen.grid2d(9, 1)
+    x, y, g, its = np.ones(4 * m.nv), np.ones(4 * m.nv), np.zeros(m.ne), (ctypes.c_int * 4)()
+    rtol, stiffness = ctypes.c_double(1e-8), 8 * 3 * m.ne
+
+    def call(h, where):
+        if where == "gradient":
+            return lib.amg_element_grad(h, vp(x), vp(x), vp(g), None)
+        if where == "mass":
+            return lib.amg_mass_apply(h, vp(x), vp(y), None)
+        if where == "multi":
+            return lib.amg_solve_multi(h, 4, vp(x), vp(y), rtol, its, None, None, None)
+        if where == "batch":
+            return lib.amg_batch_create(1, (ctypes.c_void_p * 1)(h.value), 1, rtol, None, ctypes.byref(ctypes.c_void_p()))
+        return update(lib, h, m, 3.0)
+
+    bare, h = setup(lib, m), setup(lib, m)
+    try:
+        if where == "gradient":
+            room = max(stiffness, 8 * (2 * m.nv + m.ne))        # enough for the stiffness, were it first
+        else:
+            assert call(h, "gradient") == 0
+            lib.shim_peak()
+            before = lib.shim_used()
+            assert call(bare, where) == 0
+            room = lib.shim_peak() - before - stiffness         # what the call takes, less what h can give back
+        lib.shim_capacity(lib.shim_used() + room)
+        assert call(h, where) == 0, lib.amg_last_error()
+    finally:
+        lib.shim_capacity(-1)
+    want = g.copy()
+    assert call(h, "gradient") == 0 and (where == "gradient" or np.array_equal(g, want)) and g.any()
+    lib.amg_destroy(h)
+    lib.amg_destroy(bare)
