@@ -167,7 +167,16 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
   for (int64_t r : rsel)
     if (r >= 0 && !inset[r]) gid.push_back((int32_t)r);
   const int mE = (int)gid.size();
-  if (mE > small_lmax<T>() || D.ncolours > SMALL_MAXC) return;
+  if (mE > small_lmax_long<T>() || D.ncolours > SMALL_MAXC) return;
+  if (mE > small_lmax<T>()) {
+    int64_t longest = 0;
+    for (int k = 0; k < mS; ++k) {
+      int64_t n = 0;
+      for (int64_t p = Arows.ptr[gid[k]]; p < Arows.ptr[gid[k] + 1]; ++p) n += Arows.val[p] != 0.0;
+      longest = std::max(longest, n);
+    }
+    if (longest <= TILE_MAXW) return;
+  }
   std::unordered_map<int32_t, int32_t> loc;
   loc.reserve(mE * 2);
   for (int k = 0; k < mE; ++k) loc[gid[k]] = k;
@@ -221,12 +230,6 @@ void build_small(const AuxLevelHost& L, const HostCSR& Arows, const std::vector<
     }
     rp_ptr.push_back((int32_t)rp_child.size());
   }
-  auto longest = [](const std::vector<int32_t>& ptr) {
-    int32_t w = 0;
-    for (size_t k = 1; k < ptr.size(); ++k) w = std::max(w, ptr[k] - ptr[k - 1]);
-    return w;
-  };
-  if (longest(sm_ptr) > SMALL_MAXW || longest(rs_ptr) > SMALL_MAXW) return;
   S.mS = mS;
   S.mE = mE;
   S.ncol = D.ncolours;

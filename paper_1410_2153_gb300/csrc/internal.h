@@ -265,8 +265,15 @@ template <class T>
 constexpr int small_lmax() {
   return sizeof(T) == 8 ? 512 : 1024;
 }
+// the same for a level with a smoothing row of more than TILE_MAXW entries
+// (locally refined 3D grids), which no tile takes: the alternative is a launch
+// per colour class and sweep
+template <class T>
+constexpr int small_lmax_long() {
+  return sizeof(T) == 8 ? 512 : 2048;
+}
 constexpr int SMALL_MAXC = 24;
-constexpr int SMALL_MAXW = 16;                 // longest row
+constexpr int SMALL_MAXW = 16;                 // entries of a row in ELL form; the rest of longer rows follows in CSR
 constexpr int SMALL_NONE = 0xffff;             // no parent (Dirichlet)
 constexpr int64_t SMALL_SMEM_MAX = 200 * 1024; // shared memory of a run
 
@@ -281,13 +288,21 @@ struct SmallLevel {
   std::vector<T> sm_val, dinv, rs_val;
 };
 
+// the entries past SMALL_MAXW of a level's rows (CSR with 16-bit row starts);
+// ptr = 0: no row has any
+struct SmallRest {
+  int32_t ptr, col, val;
+};
+
 // one level of a run: sizes, and byte offsets within the run's block of its
 // union rows, diagonal inverses, ELL rows (mSp / mEp rows per column, widths
-// wsm / wrs), new nodes and restriction; sm0: its first row in the run's fs, us
+// wsm / wrs) with their rests, new nodes and restriction; sm0: its first row in
+// the run's fs, us
 struct SmallHead {
   int32_t mS, mE, ncol, nnew, npar, sm0, mSp, mEp, wsm, wrs;
   int32_t cs[SMALL_MAXC + 1];
   int32_t o_row, o_dinv, o_smc, o_smv, o_nn, o_rsc, o_rsv, o_rid, o_rptr, o_rch;
+  SmallRest sm_rest, rs_rest;
 };
 
 inline __host__ __device__ int64_t small_pad16(int64_t b) { return (b + 15) / 16 * 16; }

@@ -19,6 +19,16 @@
 // graded 513^2 FP64 38.4 ms, 331^2 mixed 2,008 us; the same with levels above
 // 1,024 rows tiled 917 us, 32.4 ms, 1,727 us; these kernels 776 us, 29.7 ms,
 // 1,626 us.
+//
+// Rows of more than SMALL_MAXW entries (locally refined 3D grids: 19 to 27 on
+// levels whose mean is 8) keep their first entries in ELL form and the rest in
+// CSR, in kernels of their own; the ELL width is the one that takes the fewest
+// entries.  Such levels, which no tile takes, join a run up to twice the rows:
+// a launch per colour class and sweep is 24 to 32 launches for 88 or 1,024 rows.
+// 25^3 vertices mapped by x -> x^3, no level fused -> the two finest: mixed
+// 27.6 -> 26.6 ms, BF16 27.5 -> 26.5 ms; 41^3 mixed 68.9 -> 66.0 ms.  With a
+// fixed ELL width of 16 the level of 1,024 rows does not fit in FP32 (27.4 ms),
+// with the limit at 1,024 rows it stays out in BF16 too (27.3 ms).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -64,6 +74,29 @@ __device__ __forceinline__ void ell_sub(VecK<T, KC>& acc, const uint16_t* col, c
     }
 }
 
+// W of the kernels for runs with rows of more than SMALL_MAXW entries
+constexpr int SMALL_LONG = SMALL_MAXW + 1;
+
+// acc less row k's product (stored order): ELL entries, and with W = SMALL_LONG
+// what follows them in CSR
+template <class T, class V, int W, int KC>
+__device__ __forceinline__ void row_sub(VecK<T, KC>& acc, const uint16_t* col, const V* val, int mp, int k, int w,
+                                        const unsigned char* B, const SmallRest& R, const VecK<T, KC>* x) {
+  ell_sub<T, V, (W < SMALL_MAXW ? W : SMALL_MAXW), KC>(acc, col, val, mp, k, w, x);
+  if constexpr (W == SMALL_LONG)
+    if (R.ptr) {
+      const uint16_t* ptr = reinterpret_cast<const uint16_t*>(B + R.ptr);
+      const uint16_t* c = reinterpret_cast<const uint16_t*>(B + R.col);
+      const V* v = reinterpret_cast<const V*>(B + R.val);
+      for (int p = ptr[k]; p < ptr[k + 1]; ++p) {
+        const VecK<T, KC> xe = x[c[p]];
+        const T a = (T)val_of(v[p]);
+#pragma unroll
+        for (int j = 0; j < KC; ++j) acc.v[j] -= a * xe.v[j];
+      }
+    }
+}
+
 __device__ __forceinline__ void stage(unsigned char* dst, const unsigned char* src, int bytes) {
   for (int o = threadIdx.x * 16; o < bytes; o += blockDim.x * 16)
     *reinterpret_cast<uint4*>(dst + o) = __ldg(reinterpret_cast<const uint4*>(src + o));
@@ -105,7 +138,7 @@ __global__ void __launch_bounds__(1024, 1)
         for (int k = L.cs[c] + tid; k < L.cs[c + 1]; k += nt) {
           const int r = row[k];
           X acc = F[r], u = U[r];
-          ell_sub<T, V, W, KC>(acc, smc, smv, L.mSp, k, L.wsm, U);
+          row_sub<T, V, W, KC>(acc, smc, smv, L.mSp, k, L.wsm, B, L.sm_rest, U);
           const T di = dinv[k];
 #pragma unroll
           for (int j = 0; j < KC; ++j) u.v[j] += acc.v[j] * di;
@@ -118,7 +151,7 @@ __global__ void __launch_bounds__(1024, 1)
     for (int k = tid; k < L.mE; k += nt) {
       const int r = row[k];
       X acc = F[r];
-      ell_sub<T, V, W, KC>(acc, rsc, rsv, L.mEp, k, L.wrs, U);
+      row_sub<T, V, W, KC>(acc, rsc, rsv, L.mEp, k, L.wrs, B, L.rs_rest, U);
       F[r] = acc;
     }
     __syncthreads();
@@ -205,7 +238,7 @@ __global__ void __launch_bounds__(1024, 1)
         for (int k = L.cs[c] + tid; k < L.cs[c + 1]; k += nt) {
           const int r = row[k];
           X acc = fs[L.sm0 + k], u = U[r];
-          ell_sub<T, V, W, KC>(acc, smc, smv, L.mSp, k, L.wsm, U);
+          row_sub<T, V, W, KC>(acc, smc, smv, L.mSp, k, L.wsm, B, L.sm_rest, U);
           const T di = dinv[k];
 #pragma unroll
           for (int j = 0; j < KC; ++j) u.v[j] += acc.v[j] * di;
@@ -262,29 +295,56 @@ bool build_run(const Prec<T>& P, const std::vector<int>& li, bool bf16, int kc, 
   if (gid.size() >= SMALL_NONE) return false;
   R.v.nunion = (int)gid.size();
   R.v.o_gid = put(gid.data(), gid.size() * sizeof(int32_t));
-  // ELL form of rows given as CSR over local columns
+  auto values = [&](const std::vector<T>& v) {
+    if (!bf16) return put(v.data(), v.size() * sizeof(T));
+    std::vector<bf16v> b(v.size());
+    for (size_t q = 0; q < v.size(); ++q) b[q].bits = bf16_bits((float)v[q]);
+    return put(b.data(), b.size() * sizeof(bf16v));
+  };
+  // ELL form of rows given as CSR over local columns, and the entries past SMALL_MAXW
+  bool fits = true;
   auto ell = [&](const std::vector<uint16_t>& row, const std::vector<int32_t>& ptr, const std::vector<uint16_t>& col,
-                 const std::vector<T>& val, int& mp, int& w, int32_t& oc, int32_t& ov) {
+                 const std::vector<T>& val, int& mp, int& w, int32_t& oc, int32_t& ov, SmallRest& rest) {
     const int m = (int)ptr.size() - 1;
     mp = (m + 31) / 32 * 32;
-    w = 0;
-    for (int k = 0; k < m; ++k) w = std::max(w, ptr[k + 1] - ptr[k]);
-    width = std::max(width, w);
-    std::vector<uint16_t> c((size_t)w * mp, 0);
-    std::vector<T> v((size_t)w * mp, (T)0);
-    for (int k = 0; k < m; ++k)
-      for (int p = ptr[k], e = 0; p < ptr[k + 1]; ++p, ++e) {
-        c[(size_t)e * mp + k] = row[col[p]];
-        v[(size_t)e * mp + k] = val[p];
+    int longest = 0;
+    for (int k = 0; k < m; ++k) longest = std::max(longest, ptr[k + 1] - ptr[k]);
+    width = std::max(width, longest);
+    w = longest;
+    if (longest > SMALL_MAXW) {
+      // the ELL width that takes the fewest entries, padding included
+      int64_t least = INT64_MAX;
+      for (int x = 1; x <= SMALL_MAXW; ++x) {
+        int64_t n = (int64_t)x * mp;
+        for (int k = 0; k < m; ++k) n += std::max(0, ptr[k + 1] - ptr[k] - x);
+        if (n <= least) {
+          least = n;
+          w = x;
+        }
       }
-    oc = put(c.data(), c.size() * sizeof(uint16_t));
-    if (bf16) {
-      std::vector<bf16v> b(v.size());
-      for (size_t q = 0; q < v.size(); ++q) b[q].bits = bf16_bits((float)v[q]);
-      ov = put(b.data(), b.size() * sizeof(bf16v));
-    } else {
-      ov = put(v.data(), v.size() * sizeof(T));
     }
+    std::vector<uint16_t> c((size_t)w * mp, 0), xp(1, 0), xc;
+    std::vector<T> v((size_t)w * mp, (T)0), xv;
+    for (int k = 0; k < m; ++k) {
+      for (int p = ptr[k], e = 0; p < ptr[k + 1]; ++p, ++e) {
+        if (e < w) {
+          c[(size_t)e * mp + k] = row[col[p]];
+          v[(size_t)e * mp + k] = val[p];
+        } else {
+          xc.push_back(row[col[p]]);
+          xv.push_back(val[p]);
+        }
+      }
+      xp.push_back((uint16_t)xc.size());
+    }
+    oc = put(c.data(), c.size() * sizeof(uint16_t));
+    ov = values(v);
+    rest = SmallRest{0, 0, 0};
+    if (xc.empty()) return;
+    if (xc.size() > UINT16_MAX) fits = false;
+    rest.ptr = put(xp.data(), xp.size() * sizeof(uint16_t));
+    rest.col = put(xc.data(), xc.size() * sizeof(uint16_t));
+    rest.val = values(xv);
   };
   for (size_t d = 0; d < li.size(); ++d) {  // what both directions read
     const SmallLevel<T>& M = P.lev[li[d]].small;
@@ -299,7 +359,7 @@ bool build_run(const Prec<T>& P, const std::vector<int>& li, bool bf16, int kc, 
     for (int c = 0; c <= SMALL_MAXC; ++c) H.cs[c] = c <= M.ncol ? M.cs[c] : M.mS;
     H.o_row = put(rows[d].data(), rows[d].size() * sizeof(uint16_t));
     H.o_dinv = put(M.dinv.data(), M.dinv.size() * sizeof(T));
-    ell(rows[d], M.sm_ptr, M.sm_col, M.sm_val, H.mSp, H.wsm, H.o_smc, H.o_smv);
+    ell(rows[d], M.sm_ptr, M.sm_col, M.sm_val, H.mSp, H.wsm, H.o_smc, H.o_smv, H.sm_rest);
     std::vector<uint16_t> nn;
     for (uint16_t k : M.nn_id) nn.push_back(rows[d][k]);
     for (const auto* p : {&M.nn_p0, &M.nn_p1})
@@ -310,7 +370,7 @@ bool build_run(const Prec<T>& P, const std::vector<int>& li, bool bf16, int kc, 
   for (size_t d = 0; d < li.size(); ++d) {
     const SmallLevel<T>& M = P.lev[li[d]].small;
     SmallHead& H = head[d];
-    ell(rows[d], M.rs_ptr, M.rs_col, M.rs_val, H.mEp, H.wrs, H.o_rsc, H.o_rsv);
+    ell(rows[d], M.rs_ptr, M.rs_col, M.rs_val, H.mEp, H.wrs, H.o_rsc, H.o_rsv, H.rs_rest);
     std::vector<uint16_t> id, ptr, ch;
     for (uint16_t k : M.rp_id) id.push_back(rows[d][k]);
     for (int32_t p : M.rp_ptr) ptr.push_back((uint16_t)p);
@@ -323,7 +383,7 @@ bool build_run(const Prec<T>& P, const std::vector<int>& li, bool bf16, int kc, 
   std::memcpy(B.data(), head.data(), head.size() * sizeof(SmallHead));
   R.width = width;
   R.threads = std::min(1024, std::max(128, (max_rows + 31) / 32 * 32));
-  if (width > SMALL_MAXW || smem_down(R, kc) > SMALL_SMEM_MAX || smem_up(R, kc) > SMALL_SMEM_MAX) return false;
+  if (!fits || smem_down(R, kc) > SMALL_SMEM_MAX || smem_up(R, kc) > SMALL_SMEM_MAX) return false;
   return true;
 }
 
@@ -363,13 +423,15 @@ template <class F>
 void run_width(int width, F f) {
   if (width <= 8)
     f(std::integral_constant<int, 8>{});
-  else
+  else if (width <= SMALL_MAXW)
     f(std::integral_constant<int, SMALL_MAXW>{});
+  else
+    f(std::integral_constant<int, SMALL_LONG>{});
 }
 
 template <class T, class V, int KC>
 void set_smem_limits() {
-  for (int w : {8, SMALL_MAXW})
+  for (int w : {8, SMALL_MAXW, SMALL_LONG})
     run_width(w, [&](auto W) {
       ASMG_CUDA(cudaFuncSetAttribute(k_small_down<T, V, decltype(W)::value, KC>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM_MAX));
