@@ -261,7 +261,9 @@ enum asmg_info_what {
   ASMG_INFO_NTILES = 14,      /* tiles of the temporally blocked pre-sweeps of level `level` (0: one
                                  launch per colour class and sweep) */
   ASMG_INFO_HALO_ROWS = 15,   /* halo rows of those tiles (pre-sweeps), summed over the tiles */
-  ASMG_INFO_NTILES_UP = 16    /* tiles of the temporally blocked post-sweeps of level `level` (0: per class) */
+  ASMG_INFO_NTILES_UP = 16,   /* tiles of the temporally blocked post-sweeps of level `level` (0: per class) */
+  ASMG_INFO_TILE_SLOTS = 17,  /* rows a thread holds in those tiles: pre-sweeps + 16 * post-sweeps (0: per class) */
+  ASMG_INFO_TILE_WIDTH = 18   /* entries of their longest row: pre-sweeps + 256 * post-sweeps (0: per class) */
 };
 int amg_info(asmg_handle h, int what, int level, int64_t* value);
 

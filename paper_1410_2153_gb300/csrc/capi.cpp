@@ -2042,6 +2042,16 @@ int amg_info(asmg_handle h, int what, int level, int64_t* value) {
       *value = h->prm.precision == ASMG_MIXED ? h->p32.lev[k].tdown.halo : h->p64.lev[k].tdown.halo;
       break;
     }
+    case ASMG_INFO_TILE_SLOTS:
+    case ASMG_INFO_TILE_WIDTH: {
+      const int k = lev_index(level);
+      auto read = [&](const auto& L) -> int64_t {
+        if (what == ASMG_INFO_TILE_SLOTS) return (L.tiled_down ? L.tdown.slots : 0) + 16 * (L.tiled_up ? L.tup.slots : 0);
+        return (L.tiled_down ? L.tdown.width : 0) + 256 * (L.tiled_up ? L.tup.width : 0);
+      };
+      *value = h->prm.precision == ASMG_MIXED ? read(h->p32.lev[k]) : read(h->p64.lev[k]);
+      break;
+    }
     case 100: *value = h->gpu_launches_per_iter; break;
     case 101: *value = (int64_t)(h->stats.t_total * 1e6); break;
     case 102: *value = (int64_t)(h->stats.t_tree * 1e6); break;
