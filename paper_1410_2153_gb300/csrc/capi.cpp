@@ -1199,33 +1199,8 @@ void build_all(asmg_s& h, cudaStream_t s) {
   ASMG_CUDA(cudaStreamSynchronize(s));
   h.stats.t_slots = now() - tg;
   h.stats.t_levels = now() - t2;
+  h.bytes_iter = iteration_bytes(h);
   h.ready = true;
-}
-
-// algorithmic bytes of one PCG iteration (compulsory traffic, real non-zeros)
-template <class T>
-int64_t iteration_bytes(const asmg_s& h, const Prec<T>& P) {
-  const int64_t s = sizeof(T), n = h.n, nJ = h.nJ;
-  const int64_t nnzA = h.A64.nnz_real;
-  int64_t b = 0;
-  b += nnzA * 12 + 16 * n;                  // q = A p, <p, q>
-  b += 48 * n;                              // x += a p, r -= a q, ||r||
-  b += (s + 16) * n;                        // <z, r>, <z, q>
-  b += (s + 16) * n;                        // p = z + beta p
-  b += 2 * (nnzA * (s + 4) + 8 * n + 2 * s * n);  // two fine sweeps
-  if (nJ > 0) {
-    b += nnzA * (s + 4) + 8 * n + 2 * s * n;  // fine residual
-    b += (P.PT.nnz_real) * (s + 4) + s * n + 2 * s * nJ;  // P^T
-    b += (P.P.nnz_real) * (s + 4) + s * nJ + 2 * s * n;   // P
-    for (auto& L : P.lev) {
-      const int64_t m = L.nsm_real;
-      b += (h.prm.nu_pre + h.prm.nu_post) * (L.SM.nnz_real * (s + 4) + m * (4 + 3 * s));
-      b += L.RS.nnz_real * (s + 4) + L.nrs * (4 + 2 * s);
-      b += 2 * m * (4 + 2 * s) + L.nnew * (12 + 3 * s);
-    }
-    b += h.nc * h.nc * 8 + h.nc * (4 + 2 * s);
-  }
-  return b;
 }
 
 // f() with the device memory it needs: when that runs out, again without the
@@ -1389,7 +1364,6 @@ int amg_setup(int dim, int64_t nv, const double* vertices, int64_t ne, const int
     m.boxdomain = std::fabs(meas - box) <= 1e-12 * box;
   }
   build_all(*h, s);
-  h->bytes_iter = prm.precision == ASMG_MIXED ? iteration_bytes(*h, h->p32) : iteration_bytes(*h, h->p64);
   // load the allocation-free entry point's module (and so its fixed scratch
   // array) on this device now, so that its calls never create memory
   noalloc_scratch_for_current_device();
@@ -1921,7 +1895,6 @@ void set_coefficients(asmg_handle h, std::vector<double> c, cudaStream_t s) {
     h->dCoeff.upload(h->mesh.coeff, s);
     build_all(*h, s);
   });
-  h->bytes_iter = h->prm.precision == ASMG_MIXED ? iteration_bytes(*h, h->p32) : iteration_bytes(*h, h->p64);
 }
 }  // namespace
 

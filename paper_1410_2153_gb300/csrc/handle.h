@@ -196,6 +196,7 @@ struct asmg_s {
 namespace asmg {
 // solve.cu
 void setup_solve(asmg_s& h, cudaStream_t s);
+int64_t iteration_bytes(asmg_s& h);  // algorithmic bytes of one step, as profile_solve counts them
 int profile_solve(asmg_s& h, double rtol, cudaStream_t s, double* out, double* out_levels = nullptr,
                   int nlev_out = 0);
 // noalloc.cu

@@ -768,9 +768,14 @@ struct Profiler {
 };
 thread_local Profiler* g_prof = nullptr;
 thread_local int g_prof_level = -1;
+thread_local int64_t* g_count_bytes = nullptr;  // set: launches only add up their bytes
 
 #define LAUNCH(cls, bytes, ...)                                                  \
   do {                                                                          \
+    if (g_count_bytes) {                                                        \
+      *g_count_bytes += (int64_t)(bytes);                                       \
+      break;                                                                    \
+    }                                                                           \
     int e0_ = g_prof ? g_prof->mark() : -1;                                     \
     __VA_ARGS__;                                                                \
     if (g_prof) {                                                               \
@@ -1031,7 +1036,7 @@ int enqueue_precond(asmg_s& h, Slot& S, const double* r, cudaStream_t s, bool fi
       ++launches;
     }
   } else {
-    ASMG_CUDA(cudaMemsetAsync(SP.uf.p, 0, sizeof(T) * h.npad, s));
+    if (!g_count_bytes) ASMG_CUDA(cudaMemsetAsync(SP.uf.p, 0, sizeof(T) * h.npad, s));
     smooth(true);
   }
   // (2) multiplicative: u2 = u1 + P Btilde P^T (r - A u1);  additive: u1 + P Btilde P^T r
@@ -1289,6 +1294,16 @@ int run_solve(asmg_s& h, Slot& S, double rtol, cudaStream_t s) {
     }
   }
   return 0;
+}
+
+int64_t iteration_bytes(asmg_s& h) {
+  int64_t bytes = 0;
+  struct Counting {
+    explicit Counting(int64_t* n) { g_count_bytes = n; }
+    ~Counting() { g_count_bytes = nullptr; }
+  } counting(&bytes);
+  enqueue_body_any(h, *h.slots[0], nullptr, 0, 0);
+  return bytes;
 }
 
 // One solve without the graph, every launch timed: per class launches,

@@ -244,6 +244,7 @@ cudaGraphNode_t capture_solve_multi(asmg_s& h, MultiSlot& S, double, cudaGraph_t
   reinterpret_cast<Calls*>(g)->push_back([&] { run_solve_multi(h, S, 0, nullptr); });
   return nullptr;
 }
+int64_t iteration_bytes(asmg_s&) { return 0; }
 int profile_solve(asmg_s&, double, cudaStream_t, double*, double*, int) {
   ++g_solves;
   return 0;
