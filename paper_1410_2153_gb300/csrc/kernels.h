@@ -19,11 +19,12 @@ constexpr int VEC_BLOCKS = 152 * 8;  // grid of the vector-only PCG kernels: 8 C
 
 inline int nblk(int64_t n, int t = TPB) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + t - 1) / t, 1 << 24)); }
 // Grid of a reduction kernel: one block per TPB rows up to the persistent grid
-// `cap`.  All blocks count on one ticket and the last one sums a partial per
-// block, so blocks without rows only lengthen that tail: at 3,969 rows k_dots
-// took 16 us on 1,216 blocks (cold), and the 65^2 FP64 solve runs 1,583 us
-// with the full grids, 1,471 us with these (12 batched grids x 4 columns:
-// 10.9 ms, 8.3 ms).
+// `cap`.  Every block leaves a partial that its last block (grid_reduce) or
+// every block of the next kernel (up to DIRECT_BLOCKS) adds up, so blocks
+// without rows only lengthen that tail: at 3,969 rows k_dots took 16 us on
+// 1,216 blocks (cold), and the 65^2 FP64 solve ran 1,583 us with the full grids
+// and a ticket, 1,471 us with these (12 batched grids x 4 columns: 10.9 ms,
+// 8.3 ms).
 inline int red_grid(int64_t rows, int cap) { return std::min(cap, nblk(rows)); }
 
 // Block size of a row-parallel launch: 256 threads when that fills every SM
